@@ -337,7 +337,7 @@ int nys_op_create(nys_ctx* ctx, const nys_op_desc* d, nys_op** out) {
 int nys_op_destroy(nys_op* op) {
     if (!op) return NYS_OK;
     if (op->ctx) cudaStreamSynchronize(op->ctx->stream);
-    void* bufs[] = {op->taps_fwd, op->taps_adj, op->taps_nrm, op->rtab, op->inter, op->lines};
+    void* bufs[] = {op->taps_fwd, op->taps_adj, op->taps_nrm, op->rtab, op->inter, op->lines, op->planes};
     for (void* b : bufs)
         if (b) cudaFree(b);
     nys_ctx* ctx = op->ctx;
@@ -398,7 +398,6 @@ int nys_op_autotune(nys_op* op, int batch, int* choice) {
     if (op->kind == NYS_OP_RADON) {
         knob = &op->radon_adj_ak;
         stages.push_back({&op->radon_adj_ak, {4, 8, 16}});
-        if (batch >= 4) stages.push_back({&op->radon_adj_ib, {4, 1}});
         which = 1;
     } else if (op->kind == NYS_OP_BLUR && op->dtype != NYS_F64) {
         knob = &op->blur_tile;

@@ -111,10 +111,11 @@ struct nys_op {
     int n_angles = 0, n_bins = 0;
     double span = 0.0;
     void* rtab = nullptr;             // per-angle tables, see radon.cu
-    void* lines = nullptr;            // radon: `chunk` images as line-major copies (row-major and transposed)
+    void* lines = nullptr;            // radon: `chunk` images as interleaved lines (along rows and along columns)
+    void* planes = nullptr;           // radon adjoint: partial images (lanes and angle ranges) of a launch
+    int radon_sets = 1;               // radon: mirror lanes the angles allow (1, 2 and 4 or'ed, see radon.cu)
     double src_dist = 0.0, det_dist = 0.0, det_spacing = 1.0;   // fan beam
     int radon_adj_ak = 16;            // radon adjoint: angles per round, 4, 8 or 16 (nys_op_autotune)
-    int radon_adj_ib = 4;             // radon adjoint: images per CTA for batches of 4 or more, 1 or 4
     int blur_tile = 64;               // blur: output tile side, 32 or 64 (float32; chosen by nys_op_autotune)
     // intermediate buffer for two-pass normals (M per image, `chunk` images)
     void* inter = nullptr;

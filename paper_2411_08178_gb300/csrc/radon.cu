@@ -4,611 +4,655 @@
 //
 // Geometry: pixel (i, j) sits at x = j - c2, y = i - c1 (c = (n-1)/2); ray
 // (theta_k, t_m) is the line x cos + y sin = t with theta_k = k span / n_angles
-// and t_m = m - (n_bins - 1)/2.  A "row-step" angle (|cos| + 1e-9 >= |sin|)
-// samples the ray once per image row i at column position
-//     u(i, m) = c2 + t_m / cos - (i - c1) tan = Q_m + R_i
+// and t_m = m - cb, cb = (n_bins - 1)/2.  A "row-step" angle (|cos| + 1e-9 >=
+// |sin|, den = cos) samples the ray once per image row i at column position
+//     u(i, m) = c2 + (t_m - (i - c1) sin) / cos
 // with linear interpolation between columns floor(u) and floor(u) + 1 and
-// weight 1/|cos|; a "column-step" angle swaps the roles of rows and columns
-// (Q_m = c1 + t_m / sin, R_j = -(j - c2) cot, weight 1/|sin|).  Samples that
-// fall outside the image contribute zero.
+// weight 1/|den|; a "column-step" angle (den = sin) swaps the roles of rows
+// and columns.  Samples that fall outside the image contribute zero.  Seen
+// from a pixel, ray m carries the weight
+//     max(0, 1/|den| - |m - m*| / den^2),  m* = cb + (j - c2) cos + (i - c1) sin
+// (u - position = (m - m*) / den): at most the two bins either side of m*,
+// since |den| <= 1.  The forward walks rays, the adjoint gathers per pixel;
+// both take their positions from float64 and step them in fixed point, so the
+// weights of the two agree to about 1e-7 (float32 operators: 32 fraction bits
+// in the forward, 26 in the adjoint, relative to a 32 x 32 tile) or to the
+// last float64 bits, and the two are transposes of each other to rounding.
 //
-// Precision: Q_m and R_l are split on the host, in float64, into an integer
-// part and a fraction in [0, 1).  The device adds the two fractions (error at
-// most one float ulp of a number below 2), so interpolation weights carry an
-// absolute error near 1e-7 instead of the ~3e-5 that a float position near 500
-// would carry.  The forward (ray-driven) and the adjoint (pixel-driven gather)
-// evaluate the SAME float expressions for every (ray, line) pair, so the
-// adjoint is the exact transpose of the forward up to summation order, with
-// no atomics.
+// Lanes.  Positions and weights cost as much as the arithmetic on the data,
+// so both kernels carry IB values per position, interleaved in memory (one
+// 16-byte load feeds four float32 lanes).  A lane is an image of a batch, or
+// one of V mirror images of the same image: over 180 degrees, angle
+// n_angles - k sees the left-right mirrored image exactly as angle k sees the
+// image, and for a square image and an even number of angles n_angles/2 -+ k
+// do the same with the transposed image and its mirror image.  Base angles
+// k = 0 .. n_base - 1 and ang[k][v], the angle of lane v (-1: none, the lane
+// is a copy of another angle's), describe the set (RSet below).
 //
-// Forward: one CTA per (angle, group of IB images), each warp 96 consecutive
-// bins (three per lane), stepping along the lines of the angle that the
-// warp's rays cross inside the image.  The image is read "line-major":
-// row-step angles read the row-major image, column-step angles a transposed
-// copy (made once per batch chunk), so consecutive bins of a warp read
-// consecutive addresses for both kinds of angle.  The per-line table entries
-// are staged in shared memory and shared by the three bins and the IB images.
-// Adjoint: one CTA per (16 x 16 pixel tile, group of IB images).  Angles are
-// taken AK at a time: for each, the window of bins that can reach the tile
-// (from the four tile corners) is staged in shared memory with its tables and
-// sinogram values, so the per-pixel candidate tests read shared memory only;
-// candidates outside the window (none for |slope| <= 1, kept for safety) fall
-// back to global loads.
+// Kernels: radon_prep (images to interleaved lines with zero margins, for
+// row-step angles along rows, for column-step ones along columns), radon_fwd
+// (rays), radon_lanes (a planar sinogram to interleaved lanes), radon_adj
+// (pixels), radon_sum (the lanes and angle ranges of one image added up).
 #include "internal.cuh"
 
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 
 namespace nys {
 namespace {
 
-template <class TC>
-struct RTab {
-    const int* qi;     // [n_angles][n_bins]
-    const TC* qf;      // [n_angles][n_bins]
-    const int* ri;     // [n_angles][nl_max]
-    const TC* rf;      // [n_angles][nl_max]
-    const TC* wt;      // [n_angles] 1/|cos| or 1/|sin|
-    const TC* slope;   // [n_angles] dm/du = cos (row-step) or sin (column-step)
-    const TC* oth;     // [n_angles] sin (row-step) or cos (column-step): dm*/dl
-    const int* rowstep;// [n_angles]
-    int nl_max;
+constexpr int PAD = 3;    // zeros of an interleaved line: one before, two after
+
+// per-angle geometry, float64; the ray positions of float32 operators also as
+// integers with 40 fraction bits (GB300 issues a float64 operation every 16
+// cycles per warp and SM: evaluated in float64, the positions of a few bins per
+// warp took as long as a quarter of a warp's lines)
+struct RGeo {
+    double u0, inv, t;    // 1 + u(m, l) = u0 + m inv - l t
+    long long u0q, invq, tq;
+    double cs, sn;
+    int rs, pad;          // row-step angle
 };
 
-template <class TC>
-__device__ __forceinline__ void sample_pos(int qi, TC qf, int ri, TC rf, int& lo, TC& w) {
-    TC f = qf + rf;
-    const int carry = f >= TC(1) ? 1 : 0;
-    f -= (TC)carry;
-    lo = qi + ri + carry;
-    w = f;
-}
+// the angles of a launch: base angle kb's geometry is geo[ang[kb V]], its lane
+// v holds angle ang[kb V + v] or, when negative, nothing
+struct RSet {
+    const RGeo* geo;
+    const int* ang;
+    int V, n_base;
+};
 
-// xr (optional) / xT: line-major copies of `batch` images in the compute type;
-// xT[b][j][i] = x[b][i][j]
-template <class TI, class TC>
-__global__ void radon_prep_kernel(const TI* __restrict__ x, TC* __restrict__ xr, TC* __restrict__ xT, int n1, int n2) {
-    pdl_enter();
-    __shared__ TC tile[32][33];
-    const int b = blockIdx.z;
-    const int i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
-    const TI* xb = x + (size_t)b * n1 * n2;
-    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-        const int i = i0 + r, j = j0 + threadIdx.x;
-        TC v = TC(0);
-        if (i < n1 && j < n2) {
-            v = (TC)ldf(xb + (size_t)i * n2 + j);
-            if (xr) xr[(size_t)b * n1 * n2 + (size_t)i * n2 + j] = v;
-        }
-        tile[r][threadIdx.x] = v;
-    }
-    __syncthreads();
-    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-        const int j = j0 + r, i = i0 + threadIdx.x;
-        if (i < n1 && j < n2) xT[(size_t)b * n1 * n2 + (size_t)j * n1 + i] = tile[threadIdx.x][r];
+template <class TC, int IB>
+struct alignas(sizeof(TC) * IB >= 16 ? 16 : sizeof(TC) * IB) Lanes {
+    TC v[IB];
+};
+
+// source pixel of lane variant v at (line, pos) of orientation o (0: lines are
+// rows, 1: columns): 0 the image, 1 mirrored in j, 2 transposed, 3 transposed
+// and mirrored (2 and 3: square images)
+__device__ __forceinline__ void variant_src(int v, int& i, int& j, int n1, int n2) {
+    if (v == 1) j = n2 - 1 - j;
+    else if (v >= 2) {
+        const int t = i;
+        i = j;
+        j = v == 2 ? t : n1 - 1 - t;
     }
 }
 
-// forward: one CTA per (angle, IB images); warps over bins, three per lane
-template <class TC, class TO, int IB>
-__global__ void __launch_bounds__(256) radon_fwd2_kernel(const TC* __restrict__ xr, const TC* __restrict__ xT,
-                                                         TO* __restrict__ y, int n1, int n2, int n_angles,
-                                                         int n_bins, int batch, RTab<TC> tab) {
+// interleaved lines: rows[g][i][1 + j] and, when the set has column-step base
+// angles (cols), cols[g][j][1 + i]; lane q of group g is variant q % V of
+// image g IB / V + q / V.  One CTA writes 32 lines x 32 positions: every lane
+// is read with its image's rows along the threads, through shared memory.
+template <class TI, class TC, int IB>
+__global__ void __launch_bounds__(256) radon_prep_kernel(const TI* __restrict__ x, Lanes<TC, IB>* __restrict__ rows,
+                                                         Lanes<TC, IB>* __restrict__ cols, int n1, int n2, int V,
+                                                         int batch) {
     pdl_enter();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int k = blockIdx.x;
-    const int b0 = blockIdx.y * IB;
-    const int rs = tab.rowstep[k];
-    const int nl = rs ? n1 : n2;       // lines (rows for row-step)
-    const int na = rs ? n2 : n1;       // positions along a line
-    int* s_ri = reinterpret_cast<int*>(smem_raw);
-    TC* s_rf = reinterpret_cast<TC*>(s_ri + ((nl + 3) & ~3));
-    for (int l = threadIdx.x; l < nl; l += blockDim.x) {
-        s_ri[l] = tab.ri[(size_t)k * tab.nl_max + l];
-        s_rf[l] = tab.rf[(size_t)k * tab.nl_max + l];
-    }
-    __syncthreads();
+    __shared__ TC tile[IB][32][33];
+    const int o = cols ? (int)(blockIdx.z & 1) : 0, g = cols ? blockIdx.z >> 1 : blockIdx.z;
+    const int nl = o ? n2 : n1, na = o ? n1 : n2;
+    const int l0 = blockIdx.y * 32, p0 = blockIdx.x * 32 - 1;
+    if (l0 >= nl || p0 >= na + PAD - 1) return;
+    const int R = IB / V;
     const size_t N = (size_t)n1 * n2;
-    const TC* src = (rs ? xr : xT) + (size_t)b0 * N;
-    const TC wt = tab.wt[k];
-    // a warp takes 96 consecutive bins (three groups of 32, one bin of each
-    // per lane: the loads of a group stay coalesced)
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    // u(m, l) = Q_m + R_l with R_l = -(l - c_line) t, t = oth / den: the
-    // lines where a sample of the warp's bins can land in [-1, na) form one
-    // interval (Q is monotone in m), taken with two lines of margin; outside
-    // it every sample is out of range and adds exactly zero
-    const TC tl = tab.oth[k] / tab.slope[k];
-    const TC c_line = TC(0.5) * (TC)((rs ? n1 : n2) - 1);
-    for (int mb = warp * 96 + lane; mb - lane < n_bins; mb += nw * 96) {
-        const int mf = mb - lane, ml = min(mf + 95, n_bins - 1);
-        const TC Qa = (TC)tab.qi[(size_t)k * n_bins + mf] + tab.qf[(size_t)k * n_bins + mf];
-        const TC Qb = (TC)tab.qi[(size_t)k * n_bins + ml] + tab.qf[(size_t)k * n_bins + ml];
-        const TC Qmin = fmin(Qa, Qb), Qmax = fmax(Qa, Qb);
-        int l_beg = 0, l_end = nl;
-        if (fabs(tl) > TC(1e-6)) {
-            // -1 <= Q - (l - c_line) t < na
-            const TC e1 = c_line + (Qmin - (TC)na) / tl, e2 = c_line + (Qmax + TC(1)) / tl;
-            l_beg = max(0, (int)floor(fmin(e1, e2)) - 2);
-            l_end = min(nl, (int)ceil(fmax(e1, e2)) + 3);
-        } else if (Qmax < TC(-3) || Qmin > (TC)(na + 2)) {
-            l_end = 0;
-        }
-        int qi[3];
-        TC qf[3];
-        bool ok[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const int m = mb + c * 32;
-            ok[c] = m < n_bins;
-            // a bin past the last one gets a position far below the line, so
-            // the range tests below reject it without a separate flag
-            qi[c] = ok[c] ? tab.qi[(size_t)k * n_bins + m] : -(1 << 28);
-            qf[c] = ok[c] ? tab.qf[(size_t)k * n_bins + m] : TC(0);
-        }
-        TC acc[3][IB];
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-#pragma unroll
-            for (int q = 0; q < IB; ++q) acc[c][q] = TC(0);
-#pragma unroll 4
-        for (int l = l_beg; l < l_end; ++l) {
-            const int ri = s_ri[l];
-            const TC rf = s_rf[l];
-            const TC* line = src + (size_t)l * na;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                int lo;
-                TC w;
-                sample_pos<TC>(qi[c], qf[c], ri, rf, lo, w);
-                const bool in0 = (unsigned)lo < (unsigned)na, in1 = (unsigned)(lo + 1) < (unsigned)na;
-#pragma unroll
-                for (int q = 0; q < IB; ++q) {
-                    const TC* lq = line + (size_t)q * N;
-                    const bool live = b0 + q < batch;
-                    const TC v0 = (in0 && live) ? lq[lo] : TC(0);
-                    const TC v1 = (in1 && live) ? lq[lo + 1] : TC(0);
-                    acc[c][q] = fma(TC(1) - w, v0, acc[c][q]);
-                    acc[c][q] = fma(w, v1, acc[c][q]);
-                }
+    for (int q = 0; q < IB; ++q) {
+        const int b = g * R + q / V, v = q % V;
+        const bool along = (o == 0) == (v < 2);      // the source's j runs along the line's positions
+        for (int r = threadIdx.y; r < 32; r += 8) {
+            const int dl = along ? r : threadIdx.x, dp = along ? threadIdx.x : r;
+            const int l = l0 + dl, p = p0 + dp;
+            TC val = TC(0);
+            if (b < batch && l < nl && p >= 0 && p < na) {
+                int i = o ? p : l, j = o ? l : p;
+                variant_src(v, i, j, n1, n2);
+                val = (TC)ldf(x + (size_t)b * N + (size_t)i * n2 + j);
             }
+            tile[q][dl][dp] = val;
         }
+    }
+    __syncthreads();
+    Lanes<TC, IB>* dst = (o ? cols : rows) + (size_t)g * nl * (na + PAD);
+    for (int r = threadIdx.y; r < 32; r += 8) {
+        const int l = l0 + r, e = p0 + 1 + threadIdx.x;
+        if (l < nl && e < na + PAD) {
+            Lanes<TC, IB> w;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const int m = mb + c * 32;
-            if (!ok[c]) continue;
-#pragma unroll
-            for (int q = 0; q < IB; ++q)
-                if (b0 + q < batch) stf(y + ((size_t)(b0 + q) * n_angles + k) * n_bins + m, wt * acc[c][q]);
+            for (int q = 0; q < IB; ++q) w.v[q] = tile[q][r][threadIdx.x];
+            dst[(size_t)l * (na + PAD) + e] = w;
         }
     }
 }
 
-// adjoint, line-scatter form: one CTA per (16 x 16 pixel tile, IB images),
-// AK angles per round.  The 256 threads are (angle a, segment g, line r) with
-// r over the tile's 16 lines (tile rows for a row-step angle, tile columns for
-// a column-step one) and AK x S = 16 (S = 16 / AK segments of the line's
-// bins).  A thread walks its bins in increasing order, evaluates the
-// forward's sample position with the same float expressions (sample_pos) and
-// adds (1 - f) s[m] at position lo and f s[m] at lo + 1 into its own row of a
-// shared buffer: no other thread writes that row, so there are no races and
-// the order of the sums is fixed.  After a barrier each pixel adds, angle by
-// angle, the S segment entries of its position and then the weighted angle
-// term -- the exact transpose of the forward, up to summation order.  The
-// global loads of the next round (staged bins, sinogram values, the line's
-// table entry) are issued into registers before the current round's scatter.
-constexpr int ATS = 16;     // tile side
-// staged bins per angle: the bins reaching a line of the tile start at most
-// 4 + 1 bins above the window start and span 17 |slope| + 15 |oth| + 2 <= 25
-// more (|slope|, |oth| <= 1 and 17^2 + 15^2 < 23^2), so 32 cover them all
-constexpr int AWIN = 32;
-constexpr int AWP = AWIN + 16;   // sinogram row pitch: the two angles of a warp 16 banks apart
-
+// position of a ray on its line, stepped line by line: an integer part and a
+// binary fraction of 32 (float) or 64 (double) bits; weight() is the fraction
+// as 1 + f in [1, 2)
 template <class TC>
-struct QS {   // one staged bin: integer and fractional part of Q_m
-    int qi;
-    TC qf;
+struct RayPos;
+template <>
+struct RayPos<float> {
+    long long p;
+    __device__ __forceinline__ void set(const RGeo& g, int m, int l) { p = (g.u0q + m * g.invq - l * g.tq + 128) >> 8; }
+    __device__ __forceinline__ void set_step(const RGeo& g) { p = (128 - g.tq) >> 8; }
+    __device__ __forceinline__ void step(const RayPos& d) { p += d.p; }
+    __device__ __forceinline__ int index() const { return (int)(p >> 32); }
+    __device__ __forceinline__ float one_plus_f() const {
+        return __uint_as_float(((unsigned)p >> 9) + 0x3f800000u);
+    }
+};
+template <>
+struct RayPos<double> {
+    int i;
+    unsigned long long f;
+    __device__ __forceinline__ void set(double u) {
+        const double fl = floor(u);
+        i = (int)fl;
+        f = (unsigned long long)((u - fl) * 18446744073709551616.0);   // 2^64; saturates below it
+    }
+    __device__ __forceinline__ void set(const RGeo& g, int m, int l) { set(fma((double)m, g.inv, fma(-(double)l, g.t, g.u0))); }
+    __device__ __forceinline__ void set_step(const RGeo& g) { set(-g.t); }
+    __device__ __forceinline__ void step(const RayPos& d) {
+        const unsigned long long s = f + d.f;
+        i += d.i + (s < f ? 1 : 0);
+        f = s;
+    }
+    __device__ __forceinline__ int index() const { return i; }
+    __device__ __forceinline__ double one_plus_f() const {
+        return __longlong_as_double((long long)((f >> 12) | 0x3ff0000000000000ull));
+    }
 };
 
-template <class TI, class TO, class TC, int IB, int AK>
-__global__ void __launch_bounds__(256, IB == 1 ? 6 : 2)
-    radon_adj3_kernel(const TI* __restrict__ s, TO* __restrict__ x, int n1, int n2, int n_angles, int n_bins,
-                      int batch, RTab<TC> tab, TC c1, TC c2, TC cb) {
+// Forward: a warp takes 32 CB consecutive bins of one base angle (CB per lane,
+// 32 apart, so that a load's addresses stay together) and steps along a SEG-th
+// of the lines its rays cross; the SEG warps of a ray add up in shared memory.
+// The 8 / SEG warp groups of a CTA take neighbouring angles and the same bins,
+// so that they read the same stripe of the image and L1 serves all but one of
+// them (87% of its sectors; one angle per CTA, reading the image from L2 for
+// every angle: 35.6 against 25.5 ms for 400 images of 512 x 512, 720 x 736).
+// y: planar sinogram of type TO, or the interleaved lanes [g][kb][m] that the
+// adjoint reads (LANES).  Bound by the L1 data pipe: 96% busy on that batch,
+// where a load's 32 positions, 1 to 1.41 pixels of 16 bytes apart, take about
+// 7 wavefronts instead of 4; before the lanes (scalar loads, four images per
+// warp) 48.4 ms, and 183 us for one image (now 94 us: 181 base angles leave
+// half of the warp slots empty).
+template <class TC, class TO, int IB, int CB, int SEG, bool LANES>
+__global__ void __launch_bounds__(256) radon_fwd_kernel(const Lanes<TC, IB>* __restrict__ rows,
+                                                        const Lanes<TC, IB>* __restrict__ cols, void* __restrict__ yv,
+                                                        int n1, int n2, int n_angles, int n_bins, int batch,
+                                                        RSet set) {
     pdl_enter();
-    constexpr int S = ATS / AK;            // segments per line
-    constexpr int BP = ATS + 1;            // buffer row pitch (odd: spreads the banks)
-    constexpr int U = (AK * AWIN + 255) / 256;   // staged entries per thread
-    static_assert(AK * S == ATS, "AK divides the tile side");
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    // [buf: AK S x IB x 16 x BP][sqs: AK x AWIN][ss: AK x IB x AWP][slope, oth, wt: n_angles]
-    // [rowstep: n_angles][mlo: AK]
-    TC* buf = reinterpret_cast<TC*>(smem_raw);
-    QS<TC>* sqs = reinterpret_cast<QS<TC>*>(buf + AK * S * IB * ATS * BP);
-    TC* ss = reinterpret_cast<TC*>(sqs + AK * AWIN);
-    TC* g_slope = ss + AK * IB * AWP;
-    TC* g_oth = g_slope + n_angles;
-    TC* g_wt = g_oth + n_angles;
-    int* g_rs = reinterpret_cast<int*>(g_wt + n_angles);
-    int* s_mlo = g_rs + n_angles;
-    const int i0 = blockIdx.y * ATS, j0 = blockIdx.x * ATS;
-    const int b0 = blockIdx.z * IB;
-    const int ti = threadIdx.x / ATS, tj = threadIdx.x % ATS;
-    const int i = i0 + ti, j = j0 + tj;
-    const bool valid = i < n1 && j < n2;
-    // scatter role: line r of angle a_me, segment g_me
-    const int r = threadIdx.x % ATS, a_me = (threadIdx.x / ATS) / S, g_me = (threadIdx.x / ATS) % S;
-    const size_t M = (size_t)n_angles * n_bins;
-    for (int k = threadIdx.x; k < n_angles; k += blockDim.x) {
-        g_rs[k] = tab.rowstep[k];
-        g_slope[k] = tab.slope[k];
-        g_oth[k] = tab.oth[k];
-        g_wt[k] = tab.wt[k];
+    constexpr int FANG = 8 / SEG;
+    __shared__ Lanes<TC, IB> part[SEG > 1 ? SEG - 1 : 1][SEG > 1 ? FANG : 1][SEG > 1 ? CB : 1][32];
+    const int nch = (n_bins + 32 * CB - 1) / (32 * CB), ch = blockIdx.x % nch, lane = threadIdx.x & 31;
+    const int wa = (threadIdx.x >> 5) % FANG, seg = (threadIdx.x >> 5) / FANG;
+    const int kb_me = blockIdx.x / nch * FANG + wa, g = blockIdx.y;
+    const int kb = min(kb_me, set.n_base - 1);      // a warp without an angle repeats the last one, unwritten
+    const int* ang = set.ang + kb * set.V;
+    const RGeo geo = set.geo[ang[0]];
+    const int nl = geo.rs ? n1 : n2, na = geo.rs ? n2 : n1;   // lines, positions along a line
+    const size_t pitch = na + PAD;
+    const Lanes<TC, IB>* src = (geo.rs ? rows : cols) + (size_t)g * nl * pitch;
+    const int m0 = ch * 32 * CB;
+    // the lines where a sample of the warp's bins can land in [-1, na) form
+    // one interval (u is monotone in m), taken with two lines of margin;
+    // outside it every sample is out of range and adds exactly zero
+    RayPos<TC> pos[CB], dt;
+    dt.set_step(geo);
+    pos[0].set(geo, m0, 0);
+    const float qa = (float)(pos[0].index() - 1);
+    pos[0].set(geo, min(m0 + 32 * CB - 1, n_bins - 1), 0);
+    const float qb = (float)(pos[0].index() - 1);
+    const float qmin = fminf(qa, qb), qmax = fmaxf(qa, qb) + 1.0f, tl = (float)geo.tq * 0x1p-40f;
+    int l_beg = 0, l_end = nl;
+    if (fabsf(tl) > 1e-6f) {
+        // -1 <= q - l t < na
+        const float e1 = (qmin - (float)na) / tl, e2 = (qmax + 1.0f) / tl;
+        l_beg = (int)fmaxf(0.0f, floorf(fminf(e1, e2)) - 2.0f);
+        l_end = (int)fminf((float)nl, ceilf(fmaxf(e1, e2)) + 3.0f);
+    } else if (qmax < -3.0f || qmin > (float)(na + 2)) {
+        l_end = 0;
     }
-    __syncthreads();
-    // first staged bin of angle k for this tile: m* = cb + slope (p - cpos) + oth (l - cline)
-    // is affine in (p, l), so its minimum over the tile (positions one beyond
-    // each side included) is at a corner; four bins of margin cover the float
-    // rounding of the split tables
-    auto window = [&](int k) -> int {
-        const int rs = g_rs[k];
-        const TC sl = g_slope[k], ot = g_oth[k];
-        const TC pa = (TC)(rs ? j0 : i0) - (rs ? c2 : c1);
-        const TC la = (TC)(rs ? i0 : j0) - (rs ? c1 : c2);
-        const TC mp = fmin(sl * (pa - TC(1)), sl * (pa + TC(ATS)));
-        const TC ml = fmin(ot * la, ot * (la + TC(ATS - 1)));
-        return (int)floor(cb + mp + ml) - 4;
-    };
-    // next round's loads, held in registers through the current round
-    int pf_qi[U];
-    TC pf_qf[U];
-    TC pf_s[U][IB];
-    int pf_ri = 0;
-    TC pf_rf = TC(0);
-    auto prefetch = [&](int k0) {
+    if (SEG > 1) {
+        const int per = (max(0, l_end - l_beg) + SEG - 1) / SEG;
+        l_beg += seg * per;
+        l_end = min(l_end, l_beg + per);
+    }
+    TC acc[CB][IB];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int e = threadIdx.x + 256 * u;
-            const int a = e / AWIN, w = e % AWIN;
-            const int k = k0 + a;
-            bool ok = e < AK * AWIN && k < n_angles;
-            const int m = ok ? window(k) + w : 0;
-            ok = ok && m >= 0 && m < n_bins;
-            pf_qi[u] = ok ? tab.qi[(size_t)k * n_bins + m] : 0;
-            pf_qf[u] = ok ? tab.qf[(size_t)k * n_bins + m] : TC(0);
+    for (int c = 0; c < CB; ++c) {
+        pos[c].set(geo, m0 + 32 * c + lane, l_beg);
 #pragma unroll
-            for (int q = 0; q < IB; ++q)
-                pf_s[u][q] = (ok && b0 + q < batch) ? (TC)ldf(s + (size_t)(b0 + q) * M + (size_t)k * n_bins + m) : TC(0);
+        for (int q = 0; q < IB; ++q) acc[c][q] = TC(0);
+    }
+    const unsigned last = na + 1;   // a position outside [-1, na) reads the two zeros after the line
+    const Lanes<TC, IB>* line = src + (size_t)l_beg * pitch;
+#pragma unroll 2
+    for (int l = l_beg; l < l_end; ++l, line += pitch) {
+#pragma unroll
+        for (int c = 0; c < CB; ++c) {
+            const unsigned e = min((unsigned)pos[c].index(), last);
+            const TC F = pos[c].one_plus_f();
+            pos[c].step(dt);
+            const Lanes<TC, IB> a = line[e], b = line[e + 1];
+            const TC w1 = F - TC(1), w0 = TC(2) - F;
+#pragma unroll
+            for (int q = 0; q < IB; ++q) acc[c][q] = fma(w1, b.v[q], fma(w0, a.v[q], acc[c][q]));
         }
-        const int k = k0 + a_me;
-        pf_ri = 0;
-        pf_rf = TC(0);
-        if (k < n_angles) {
-            const int rs = g_rs[k];
-            const int l = (rs ? i0 : j0) + r;
-            if (l < (rs ? n1 : n2)) {
-                pf_ri = tab.ri[(size_t)k * tab.nl_max + l];
-                pf_rf = tab.rf[(size_t)k * tab.nl_max + l];
+    }
+    if constexpr (SEG > 1) {
+#pragma unroll
+        for (int c = 0; c < CB; ++c)
+            if (seg) {
+                Lanes<TC, IB> w;
+#pragma unroll
+                for (int q = 0; q < IB; ++q) w.v[q] = acc[c][q];
+                part[seg - 1][wa][c][lane] = w;
             }
-        }
-    };
-    TC acc[IB];
-#pragma unroll
-    for (int q = 0; q < IB; ++q) acc[q] = TC(0);
-    prefetch(0);
-    for (int k0 = 0; k0 < n_angles; k0 += AK) {
-        __syncthreads();   // the previous round's buffers and tables are consumed
-        if (threadIdx.x < AK) s_mlo[threadIdx.x] = (k0 + threadIdx.x < n_angles) ? window(k0 + threadIdx.x) : 0;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int e = threadIdx.x + 256 * u;
-            if (e < AK * AWIN) {
-                const int a = e / AWIN, w = e % AWIN;
-                sqs[e] = QS<TC>{pf_qi[u], pf_qf[u]};
-#pragma unroll
-                for (int q = 0; q < IB; ++q) ss[(a * IB + q) * AWP + w] = pf_s[u][q];
-            }
-        }
-        const int ri = pf_ri;
-        const TC rf = pf_rf;
-        // zero this thread's buffer rows (only it writes them)
-        TC* row = buf + (size_t)((a_me * S + g_me) * IB) * ATS * BP;
-        const int k_me = k0 + a_me;
-        const int rs = k_me < n_angles ? g_rs[k_me] : 1;
-        // row-step: line r is tile row r, position c is column c -> [r][c];
-        // column-step: line r is tile column r, position c is row c -> [c][r]
-        const int ls = rs ? BP : 1, ps = rs ? 1 : BP;
-#pragma unroll
-        for (int q = 0; q < IB; ++q)
-            for (int c = 0; c < ATS; ++c) row[q * ATS * BP + r * ls + c * ps] = TC(0);
         __syncthreads();
-        if (k0 + AK < n_angles) prefetch(k0 + AK);
-        const int l = (rs ? i0 : j0) + r;              // line index in the image
-        if (k_me < n_angles && l < (rs ? n1 : n2)) {
-            const int p0 = rs ? j0 : i0;               // first position of the tile on the line
-            const TC cpos = rs ? c2 : c1;
-            const TC sl = g_slope[k_me];
-            // bins whose sample lands in positions p0 - 1 .. p0 + 15 (u in
-            // [p0 - 1, p0 + 16)), from the inverse m*(p) with one bin of
-            // margin; they lie inside the staged window (see AWIN)
-            const TC base = cb - sl * (cpos + ((TC)ri + rf));
-            const TC ma = base + sl * (TC)(p0 - 1), mb = base + sl * (TC)(p0 + ATS);
-            const int wlo = s_mlo[a_me];
-            const int mlo = max(max(0, wlo), (int)floor(fmin(ma, mb)) - 1);
-            const int mhi = min(min(n_bins, wlo + AWIN) - 1, (int)ceil(fmax(ma, mb)) + 1);
-            const int len = mhi - mlo + 1;
-            if (len > 0) {
-                const int w_beg = mlo - wlo + (g_me * len) / S, w_end = mlo - wlo + ((g_me + 1) * len) / S;
-                const QS<TC>* qa = sqs + a_me * AWIN;
-                const TC* sa = ss + a_me * IB * AWP;
-                TC* rl = row + r * ls;
-                if constexpr (IB == 1) {
-                    // one image: read-modify-write of the buffer row
-                    for (int w = w_beg; w < w_end; ++w) {
-                        const QS<TC> e = qa[w];
-                        int lo;
-                        TC f;
-                        sample_pos<TC>(e.qi, e.qf, ri, rf, lo, f);
-                        const int c = lo - p0;
-                        if (c < -1 || c >= ATS) continue;
-                        const TC sv = sa[w];
-                        if (c >= 0) rl[c * ps] = fma(TC(1) - f, sv, rl[c * ps]);
-                        if (c + 1 < ATS) rl[(c + 1) * ps] = fma(f, sv, rl[(c + 1) * ps]);
-                    }
-                } else {
-                    // Several images: two positions are summed in registers and
-                    // each is written out once (fewer shared-memory accesses per
-                    // bin; measured faster for 4 images per CTA, slower for one).
-                    // lo is monotone in m, so a position's (at most two, three on
-                    // a rounding tie) contributions come from consecutive bins,
-                    // and a slot is complete as soon as a bin no longer touches
-                    // it.  The sums run in bin order, as the read-modify-write.
-                    int cA = -1000, cB = -1000;
-                    TC vA[IB], vB[IB];
+        if (seg) return;
 #pragma unroll
-                    for (int q = 0; q < IB; ++q) vA[q] = vB[q] = TC(0);
-                    auto flush = [&](int c, const TC* v) {
-                        if (c >= 0 && c < ATS) {
+        for (int z = 0; z < SEG - 1; ++z)
 #pragma unroll
-                            for (int q = 0; q < IB; ++q) rl[q * ATS * BP + c * ps] = v[q];
-                        }
-                    };
-                    for (int w = w_beg; w < w_end; ++w) {
-                        const QS<TC> e = qa[w];
-                        int lo;
-                        TC f;
-                        sample_pos<TC>(e.qi, e.qf, ri, rf, lo, f);
-                        const int c = lo - p0;
-                        if (c < -1 || c >= ATS) continue;
-                        TC sv[IB];
+            for (int c = 0; c < CB; ++c)
 #pragma unroll
-                        for (int q = 0; q < IB; ++q) sv[q] = sa[q * AWP + w];
+                for (int q = 0; q < IB; ++q) acc[c][q] += part[z][wa][c][lane].v[q];
+    }
+    const TC wt = (TC)fabs(geo.inv);
 #pragma unroll
-                        for (int t = 0; t < 2; ++t) {          // position c (weight 1 - f), then c + 1 (f)
-                            const int ct = c + t;
-                            const TC wgt = t ? f : TC(1) - f;
-                            if (ct == cA) {
+    for (int c = 0; c < CB; ++c) {
+        const int m = m0 + 32 * c + lane;
+        if (m >= n_bins || kb_me >= set.n_base) continue;
+        if constexpr (LANES) {
+            Lanes<TC, IB> w;
 #pragma unroll
-                                for (int q = 0; q < IB; ++q) vA[q] = fma(wgt, sv[q], vA[q]);
-                            } else if (ct == cB) {
-#pragma unroll
-                                for (int q = 0; q < IB; ++q) vB[q] = fma(wgt, sv[q], vB[q]);
-                            } else if (cA != c && cA != c + 1) {   // slot A is complete
-                                flush(cA, vA);
-                                cA = ct;
-#pragma unroll
-                                for (int q = 0; q < IB; ++q) vA[q] = fma(wgt, sv[q], TC(0));
-                            } else {                               // slot B is
-                                flush(cB, vB);
-                                cB = ct;
-#pragma unroll
-                                for (int q = 0; q < IB; ++q) vB[q] = fma(wgt, sv[q], TC(0));
-                            }
-                        }
-                    }
-                    flush(cA, vA);
-                    flush(cB, vB);
-                }
-            }
-        }
-        __syncthreads();
-        if (!valid) continue;
-        const int na = min(AK, n_angles - k0);
-        for (int a = 0; a < na; ++a) {
+            for (int q = 0; q < IB; ++q) w.v[q] = ang[q % set.V] >= 0 ? wt * acc[c][q] : TC(0);
+            ((Lanes<TC, IB>*)yv)[((size_t)g * set.n_base + kb) * n_bins + m] = w;
+        } else {
+            TO* y = (TO*)yv;
 #pragma unroll
             for (int q = 0; q < IB; ++q) {
-                TC part = buf[(size_t)((a * S) * IB + q) * ATS * BP + ti * BP + tj];
-#pragma unroll
-                for (int g = 1; g < S; ++g) part += buf[(size_t)((a * S + g) * IB + q) * ATS * BP + ti * BP + tj];
-                acc[q] = fma(g_wt[k0 + a], part, acc[q]);
+                const int b = g * (IB / set.V) + q / set.V, a = ang[q % set.V];
+                if (b < batch && a >= 0) stf(y + ((size_t)b * n_angles + a) * n_bins + m, wt * acc[c][q]);
             }
         }
     }
-    if (!valid) return;
+}
+
+// planar sinogram (images x angles x bins) to the interleaved lanes [g][kb][m]
+template <class TI, class TC, int IB>
+__global__ void __launch_bounds__(256) radon_lanes_kernel(const TI* __restrict__ s, Lanes<TC, IB>* __restrict__ out,
+                                                          int n_angles, int n_bins, int batch, RSet set) {
+    pdl_enter();
+    const int kb = blockIdx.y, g = blockIdx.z;
+    const int* ang = set.ang + kb * set.V;
+    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < n_bins; m += gridDim.x * blockDim.x) {
+        Lanes<TC, IB> w;
 #pragma unroll
-    for (int q = 0; q < IB; ++q)
-        if (b0 + q < batch) stf(x + ((size_t)(b0 + q) * n1 + i) * n2 + j, acc[q]);
-}
-
-template <class TC>
-void split(double v, int& I, TC& F) {
-    double fl = std::floor(v);
-    double fr = v - fl;
-    TC f = (TC)fr;
-    if (f >= TC(1)) {
-        f = TC(0);
-        fl += 1.0;
+        for (int q = 0; q < IB; ++q) {
+            const int b = g * (IB / set.V) + q / set.V, a = ang[q % set.V];
+            w.v[q] = b < batch && a >= 0 ? (TC)ldf(s + ((size_t)b * n_angles + a) * n_bins + m) : TC(0);
+        }
+        out[((size_t)g * set.n_base + kb) * n_bins + m] = w;
     }
-    I = (int)fl;
-    F = f;
 }
 
+// Fixed-point bin position within a tile's window: 6 integer bits (a 32 x 32
+// tile spans at most 31 sqrt(2) + 2 < 46 bins)
 template <class TC>
+struct TilePos;
+template <>
+struct TilePos<float> {
+    using type = unsigned;
+    static constexpr int FRAC = 26;
+    static __device__ __forceinline__ type make(double u) { return (type)__double2ll_rn(u * 67108864.0); }
+    // the fraction is used to 23 bits: half of the last one makes that a rounding
+    static __device__ __forceinline__ type half() { return 4u; }
+    static __device__ __forceinline__ float one_plus_f(type p) {
+        return __uint_as_float(((p >> 3) & 0x7fffffu) | 0x3f800000u);
+    }
+};
+template <>
+struct TilePos<double> {
+    using type = unsigned long long;
+    static constexpr int FRAC = 57;   // below 64: within a signed 64-bit conversion
+    static __device__ __forceinline__ type make(double u) { return (type)__double2ll_rn(u * 144115188075855872.0); }
+    static __device__ __forceinline__ type half() { return 16u; }
+    static __device__ __forceinline__ double one_plus_f(type p) {
+        return __longlong_as_double((long long)(((p >> 5) & 0xfffffffffffffull) | 0x3ff0000000000000ull));
+    }
+};
+
+constexpr int ATS = 32;     // tile side; a thread holds 4 pixels, 8 rows apart
+constexpr int AWIN = 48;    // staged bins per angle: 31 sqrt(2) + 2 + the margin below, rounded up
+
+template <class TC>
+struct alignas(16) TileAng {           // one base angle as a tile sees it
+    typename TilePos<TC>::type pos0, dj, di;   // position of the tile's first pixel, steps along j and i
+    TC wb, w0, w1;                     // lower bin's weight max(0, w0 - wb F), upper's max(0, w1 + wb F), F = 1 + f
+    int mlo;                           // first staged bin
+};
+
+__device__ __forceinline__ void cp_async_zfill(void* dst, const void* src, int bytes, bool ok) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    const int n = ok ? bytes : 0;
+    if (bytes == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n));
+    else if (bytes == 8) asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(n));
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(n));
+}
+
+// Adjoint: one CTA per (32 x 32 tile, group of lanes, range of base angles).
+// AK angles per round: their windows of bins and per-tile constants are staged
+// in shared memory (copies of the next round in flight during this one, one
+// barrier per round); every pixel then takes its two bins of every angle.
+// out: images of type TO (PLANES false: one angle range, no mirror lanes), or
+// one plane per (group, angle range, lane), already mirrored back, for
+// radon_sum.  Bound by shared memory: two 16-byte loads per pixel and angle, 8
+// wavefronts per warp and four lanes, 91% of the L1 data pipe busy on a batch
+// of 400 images of 512 x 512, 720 x 736: 18.1 ms (one image: 64 us).  The
+// per-line scatter into shared memory before it, 3.7 times the instructions
+// and read-modify-writes of a private row, took 117 ms (411 us).
+template <class TC, class TO, int IB, bool PLANES>
+__global__ void __launch_bounds__(256) radon_adj_kernel(const Lanes<TC, IB>* __restrict__ s, TO* __restrict__ out,
+                                                        int n1, int n2, int n_bins, int batch, int AK, int per,
+                                                        RSet set) {
+    pdl_enter();
+    using TP = TilePos<TC>;
+    using P = typename TP::type;
+    using L = Lanes<TC, IB>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    L* win = reinterpret_cast<L*>(smem_raw);                                       // [2][AK][AWIN]
+    TileAng<TC>* tab = reinterpret_cast<TileAng<TC>*>(win + 2 * AK * AWIN);        // [3][AK]
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int i0 = blockIdx.y * ATS, j0 = blockIdx.x * ATS;
+    const int g = blockIdx.z % ((batch + IB / set.V - 1) / (IB / set.V)), z = blockIdx.z / ((batch + IB / set.V - 1) / (IB / set.V));
+    const int k_beg = z * per, k_end = min(set.n_base, k_beg + per);
+    const int rounds = (k_end - k_beg + AK - 1) / AK;
+    const L* sg = s + (size_t)g * set.n_base * n_bins;
+    auto angles_of = [&](int r) {       // the tile's constants of round r
+        const int k = k_beg + r * AK + threadIdx.x;
+        if (threadIdx.x >= AK || k >= k_end) return;
+        const RGeo geo = set.geo[set.ang[k * set.V]];
+        const double m00 = fma(geo.cs, j0 - 0.5 * (n2 - 1), fma(geo.sn, i0 - 0.5 * (n1 - 1), 0.5 * (n_bins - 1)));
+        const double lo = floor(m00 + fmin(0.0, (ATS - 1) * geo.cs) + fmin(0.0, (ATS - 1) * geo.sn) - 1e-3);
+        const double a = fabs(geo.inv), b = a * a;
+        TileAng<TC> t;
+        t.pos0 = TP::make(m00 - lo) + TP::half();
+        t.dj = TP::make(geo.cs);
+        t.di = TP::make(geo.sn);
+        t.wb = (TC)b;
+        t.w0 = (TC)(a + b);
+        t.w1 = (TC)(a - 2.0 * b);
+        t.mlo = (int)lo;
+        tab[(r % 3) * AK + threadIdx.x] = t;
+    };
+    auto stage = [&](int r) {           // the windows of round r
+        L* w = win + (r & 1) * AK * AWIN;
+        for (int e = threadIdx.x; e < AK * AWIN; e += 256) {
+            const int a = e / AWIN, k = k_beg + r * AK + a;
+            if (k < k_end) {
+                const int m = tab[(r % 3) * AK + a].mlo + (e - a * AWIN);
+                const bool ok = (unsigned)m < (unsigned)n_bins;
+                const L* src = sg + (size_t)k * n_bins + (ok ? m : 0);
+#pragma unroll
+                for (int h = 0; h < (int)(sizeof(L) + 15) / 16; ++h)
+                    cp_async_zfill((char*)(w + e) + 16 * h, (const char*)src + 16 * h,
+                                   sizeof(L) < 16 ? (int)sizeof(L) : 16, ok);
+            }
+        }
+        asm volatile("cp.async.commit_group;");
+    };
+    TC acc[4][IB];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int q = 0; q < IB; ++q) acc[u][q] = TC(0);
+    angles_of(0);
+    __syncthreads();
+    stage(0);
+    angles_of(1);
+    for (int r = 0; r < rounds; ++r) {
+        asm volatile("cp.async.wait_group 0;");
+        __syncthreads();                // round r staged, round r - 1 consumed, constants of round r + 1 there
+        if (r + 2 < rounds) angles_of(r + 2);
+        if (r + 1 < rounds) stage(r + 1);
+        const L* w = win + (r & 1) * AK * AWIN;
+        const TileAng<TC>* ta = tab + (r % 3) * AK;
+        const int na = min(AK, k_end - k_beg - r * AK);
+#pragma unroll 2
+        for (int a = 0; a < na; ++a, w += AWIN) {
+            const TileAng<TC> t = ta[a];
+            P p = t.pos0 + (P)tx * t.dj + (P)ty * t.di;
+            const P d8 = t.di * 8;
+#pragma unroll
+            for (int u = 0; u < 4; ++u, p += d8) {
+                const L* e = w + (unsigned)(p >> TP::FRAC);
+                const TC F = TP::one_plus_f(p);
+                const L s0 = e[0], s1 = e[1];
+                const TC a0 = fmax(fma(-t.wb, F, t.w0), TC(0)), a1 = fmax(fma(t.wb, F, t.w1), TC(0));
+#pragma unroll
+                for (int q = 0; q < IB; ++q) acc[u][q] = fma(a1, s1.v[q], fma(a0, s0.v[q], acc[u][q]));
+            }
+        }
+    }
+    const size_t N = (size_t)n1 * n2;
+    const int j = j0 + tx;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int i = i0 + ty + 8 * u;
+        if (i >= n1 || j >= n2) continue;
+#pragma unroll
+        for (int q = 0; q < IB; ++q) {
+            if constexpr (PLANES) {
+                int si = i, sj = j;
+                variant_src(q % set.V, si, sj, n1, n2);
+                const size_t plane = ((size_t)g * (gridDim.z / ((batch + IB / set.V - 1) / (IB / set.V))) + z) * IB + q;
+                stf(out + plane * N + (size_t)si * n2 + sj, acc[u][q]);
+            } else {
+                const int b = g * IB + q;
+                if (b < batch) stf(out + (size_t)b * N + (size_t)i * n2 + j, acc[u][q]);
+            }
+        }
+    }
+}
+
+// x[b] = the sum of image b's planes: ns angle ranges x V lanes
+template <class TC, class TO, int IB>
+__global__ void __launch_bounds__(256) radon_sum_kernel(const TC* __restrict__ planes, TO* __restrict__ x, int64_t N,
+                                                        int V, int ns) {
+    pdl_enter();
+    const int b = blockIdx.y, R = IB / V, g = b / R, q0 = (b - g * R) * V;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < N; t += (int64_t)gridDim.x * blockDim.x) {
+        TC v = TC(0);
+        for (int z = 0; z < ns; ++z)
+            for (int q = 0; q < V; ++q) v += planes[(((size_t)g * ns + z) * IB + q0 + q) * N + t];
+        stf(x + (size_t)b * N + t, v);
+    }
+}
+
+// ------------------------------------------------------------- launching --
+
 int build_tables(nys_op* op) {
     const int A = op->n_angles, B = op->n_bins, n1 = op->n1, n2 = op->n2;
-    const int nl_max = std::max(n1, n2);
     const double c1 = (n1 - 1) / 2.0, c2 = (n2 - 1) / 2.0, cb = (B - 1) / 2.0;
-    std::vector<int> qi((size_t)A * B), ri((size_t)A * nl_max, 0), rowstep(A);
-    std::vector<TC> qf((size_t)A * B), rf((size_t)A * nl_max, TC(0)), wt(A), slope(A), othv(A);
+    std::vector<RGeo> geo(A);
     for (int k = 0; k < A; ++k) {
         const double th = k * (op->span / A);
         const double cs = std::cos(th), sn = std::sin(th);
         const bool rs = std::fabs(cs) + 1e-9 >= std::fabs(sn);
-        rowstep[k] = rs;
-        const double c_line = rs ? c1 : c2;   // centre of the line index
-        const double c_pos = rs ? c2 : c1;
-        const double den = rs ? cs : sn;      // u = c_pos + t/den - (l - c_line) * other/den
-        const double oth = rs ? sn : cs;
-        wt[k] = (TC)(1.0 / std::fabs(den));
-        slope[k] = (TC)den;
-        othv[k] = (TC)oth;
-        for (int m = 0; m < B; ++m) split<TC>(c_pos + (m - cb) / den, qi[(size_t)k * B + m], qf[(size_t)k * B + m]);
-        const int nl = rs ? n1 : n2;
-        for (int l = 0; l < nl; ++l)
-            split<TC>(-(l - c_line) * oth / den, ri[(size_t)k * nl_max + l], rf[(size_t)k * nl_max + l]);
+        const double c_line = rs ? c1 : c2, c_pos = rs ? c2 : c1;
+        const double den = rs ? cs : sn, oth = rs ? sn : cs;
+        const double u0 = c_pos + 1.0 - cb / den + c_line * (oth / den), inv = 1.0 / den, t = oth / den;
+        auto fix = [](double v) { return (long long)std::llrint(std::ldexp(v, 40)); };
+        geo[k] = RGeo{u0, inv, t, fix(u0), fix(inv), fix(t), cs, sn, rs ? 1 : 0, 0};
     }
-    size_t off = 0;
-    auto al = [](size_t v) { return (v + 255) & ~size_t(255); };
-    const size_t sz_qi = al(qi.size() * 4), sz_qf = al(qf.size() * sizeof(TC)), sz_ri = al(ri.size() * 4),
-                 sz_rf = al(rf.size() * sizeof(TC)), sz_a = al(A * sizeof(TC)), sz_rs = al(A * 4);
-    const size_t total = sz_qi + sz_qf + sz_ri + sz_rf + 3 * sz_a + sz_rs;
-    NYS_CK(op->ctx, cudaMalloc(&op->rtab, total));
-    char* base = (char*)op->rtab;
-    auto put = [&](const void* src, size_t n, size_t sz) {
-        cudaError_t e = cudaMemcpy(base + off, src, n, cudaMemcpyHostToDevice);
-        off += sz;
-        return e;
-    };
-    NYS_CK(op->ctx, put(qi.data(), qi.size() * 4, sz_qi));
-    NYS_CK(op->ctx, put(qf.data(), qf.size() * sizeof(TC), sz_qf));
-    NYS_CK(op->ctx, put(ri.data(), ri.size() * 4, sz_ri));
-    NYS_CK(op->ctx, put(rf.data(), rf.size() * sizeof(TC), sz_rf));
-    NYS_CK(op->ctx, put(wt.data(), A * sizeof(TC), sz_a));
-    NYS_CK(op->ctx, put(slope.data(), A * sizeof(TC), sz_a));
-    NYS_CK(op->ctx, put(othv.data(), A * sizeof(TC), sz_a));
-    NYS_CK(op->ctx, put(rowstep.data(), A * 4, sz_rs));
-    return NYS_OK;
-}
-
-template <class TC>
-RTab<TC> tables(const nys_op* op) {
-    const int A = op->n_angles, B = op->n_bins;
-    const int nl_max = std::max(op->n1, op->n2);
-    auto al = [](size_t v) { return (v + 255) & ~size_t(255); };
-    const char* base = (const char*)op->rtab;
-    RTab<TC> t;
-    size_t off = 0;
-    t.qi = (const int*)(base + off);
-    off += al((size_t)A * B * 4);
-    t.qf = (const TC*)(base + off);
-    off += al((size_t)A * B * sizeof(TC));
-    t.ri = (const int*)(base + off);
-    off += al((size_t)A * nl_max * 4);
-    t.rf = (const TC*)(base + off);
-    off += al((size_t)A * nl_max * sizeof(TC));
-    t.wt = (const TC*)(base + off);
-    off += al(A * sizeof(TC));
-    t.slope = (const TC*)(base + off);
-    off += al(A * sizeof(TC));
-    t.oth = (const TC*)(base + off);
-    off += al(A * sizeof(TC));
-    t.rowstep = (const int*)(base + off);
-    t.nl_max = nl_max;
-    return t;
-}
-
-template <class TI, class TO, class TC>
-int radon_fwd(nys_op* op, const void* x, void* y, int batch) {
-    const int nl_max = std::max(op->n1, op->n2);
-    const size_t sm = ((nl_max + 3) & ~3) * 4 + nl_max * sizeof(TC);
-    const size_t N = (size_t)op->N;
-    cudaStream_t st = op->ctx->stream;
-    TC* xT = (TC*)op->lines;
-    TC* xr = xT + (size_t)op->chunk * N;
-    for (int b0 = 0; b0 < batch; b0 += op->chunk) {
-        const int nb = std::min(op->chunk, batch - b0);
-        const TI* xb = (const TI*)x + (size_t)b0 * N;
-        // the row-major source is x itself when it already has the compute type
-        const bool same = std::is_same<TI, TC>::value;
-        NYS_CK(op->ctx, launch_pdl(radon_prep_kernel<TI, TC>, dim3((op->n2 + 31) / 32, (op->n1 + 31) / 32, nb),
-                                   dim3(32, 8), 0, st, xb, same ? nullptr : xr, xT, op->n1, op->n2));
-        NYS_LAUNCH_CK(op->ctx);
-        const TC* src_r = same ? (const TC*)xb : xr;
-        TO* yb = (TO*)y + (size_t)b0 * op->M;
-        if (nb >= 4) {
-            const int full = nb / 4 * 4;
-            NYS_CK(op->ctx, launch_pdl(radon_fwd2_kernel<TC, TO, 4>, dim3(op->n_angles, full / 4), 256, sm, st, src_r,
-                                       (const TC*)xT, yb, op->n1, op->n2, op->n_angles, op->n_bins, full,
-                                       tables<TC>(op)));
-            NYS_LAUNCH_CK(op->ctx);
-            if (full < nb) {
-                NYS_CK(op->ctx, launch_pdl(radon_fwd2_kernel<TC, TO, 1>, dim3(op->n_angles, nb - full), 256, sm, st,
-                                           src_r + (size_t)full * N, (const TC*)(xT + (size_t)full * N),
-                                           yb + (size_t)full * op->M, op->n1, op->n2, op->n_angles, op->n_bins,
-                                           nb - full, tables<TC>(op)));
-                NYS_LAUNCH_CK(op->ctx);
+    // the angle sets: every angle by itself, and over exactly 180 degrees the
+    // mirror pairs and (square image, even number of angles) the fours
+    std::vector<int> ang;
+    op->radon_sets = 1;
+    for (int k = 0; k < A; ++k) ang.push_back(k);
+    auto add = [&](int V, int n_base, auto&& lane) {
+        op->radon_sets |= V;
+        for (int k = 0; k < n_base; ++k) {
+            const size_t first = ang.size();
+            for (int v = 0; v < V; ++v) {
+                int a = lane(k, v);
+                if (a < 0 || a >= A) a = -1;
+                for (size_t p = first; p < ang.size(); ++p)
+                    if (ang[p] == a) a = -1;
+                ang.push_back(a);
             }
-        } else {
-            NYS_CK(op->ctx, launch_pdl(radon_fwd2_kernel<TC, TO, 1>, dim3(op->n_angles, nb), 256, sm, st, src_r,
-                                       (const TC*)xT, yb, op->n1, op->n2, op->n_angles, op->n_bins, nb,
-                                       tables<TC>(op)));
-            NYS_LAUNCH_CK(op->ctx);
         }
+    };
+    if (op->span == M_PI) {
+        add(2, A / 2 + 1, [&](int k, int v) { return v ? A - k : k; });
+        if (n1 == n2 && A % 2 == 0)
+            add(4, A / 4 + 1, [&](int k, int v) { return v == 0 ? k : v == 1 ? A - k : v == 2 ? A / 2 - k : A / 2 + k; });
     }
+    NYS_CK(op->ctx, cudaMalloc(&op->rtab, geo.size() * sizeof(RGeo) + ang.size() * sizeof(int)));
+    NYS_CK(op->ctx, cudaMemcpy(op->rtab, geo.data(), geo.size() * sizeof(RGeo), cudaMemcpyHostToDevice));
+    NYS_CK(op->ctx, cudaMemcpy((char*)op->rtab + geo.size() * sizeof(RGeo), ang.data(), ang.size() * sizeof(int),
+                               cudaMemcpyHostToDevice));
     return NYS_OK;
 }
 
-template <class TC, int IB, int AK>
-size_t adj3_smem(int n_angles) {
-    constexpr int S = ATS / AK;
-    return sizeof(TC) * ((size_t)AK * S * IB * ATS * (ATS + 1) + (size_t)AK * IB * AWP + 3 * (size_t)n_angles) +
-           sizeof(QS<TC>) * (size_t)AK * AWIN + sizeof(int) * ((size_t)n_angles + AK);
+RSet angle_set(const nys_op* op, int V) {
+    const int A = op->n_angles;
+    const int* ang = (const int*)((const RGeo*)op->rtab + A);
+    RSet r;
+    r.geo = (const RGeo*)op->rtab;
+    r.V = V;
+    r.n_base = V == 1 ? A : A / V + 1;
+    r.ang = V == 1 ? ang : V == 2 ? ang + A : ang + A + 2 * (A / 2 + 1);
+    return r;
 }
 
-template <class TI, class TO, class TC, int IB, int AK>
-void radon_adj_launch(nys_op* op, const TI* s, TO* x, int nb) {
-    dim3 grid((op->n2 + ATS - 1) / ATS, (op->n1 + ATS - 1) / ATS, (nb + IB - 1) / IB);
-    const size_t sm = adj3_smem<TC, IB, AK>(op->n_angles);
-    // opt in to more than 48 KB of shared memory when the buffers need it
-    (void)smem_optin(op->ctx, (const void*)radon_adj3_kernel<TI, TO, TC, IB, AK>, sm);
-    // a launch error is left for the caller's launch check (cudaGetLastError)
-    (void)launch_pdl(radon_adj3_kernel<TI, TO, TC, IB, AK>, grid, 256, sm, op->ctx->stream, s, x, op->n1, op->n2,
-                     op->n_angles, op->n_bins, nb, tables<TC>(op), (TC)((op->n1 - 1) / 2.0), (TC)((op->n2 - 1) / 2.0),
-                     (TC)((op->n_bins - 1) / 2.0));
+// Lanes and mirror lanes for a part of a batch: fours of images while there
+// are four; a rest of one to three takes four mirror lanes an image where the
+// angles allow it (a quarter of the angles each), else two (two images to a
+// launch group), else plain lanes.
+struct Part {
+    int nb, IB, V;
+};
+Part next_part(const nys_op* op, int left) {
+    if (left >= 4) return {left / 4 * 4, 4, 1};
+    if (op->radon_sets & 4) return {left, 4, 4};
+    if (op->radon_sets & 2) return left == 1 ? Part{1, 2, 2} : Part{left, 4, 2};
+    return {left, left == 3 ? 4 : left, 1};
 }
 
-template <class TI, class TO, class TC>
-int radon_adj(nys_op* op, const void* s, void* x, int batch) {
-    // images per CTA: 4 for batches of 4 or more unless nys_op_autotune chose 1;
-    // grid.z (images / ib) stays within 65535
-    const int ib = (batch >= 4 && op->radon_adj_ib == 4) ? 4 : 1;
-    for (int b0 = 0; b0 < batch; b0 += 65535 * ib) {
-        const int nb = std::min(65535 * ib, batch - b0);
-        const TI* sb = (const TI*)s + (size_t)b0 * op->M;
-        TO* xb = (TO*)x + (size_t)b0 * op->N;
-        // 4, 8 or 16 angles per round (nys_op_autotune)
-        const int ak = op->radon_adj_ak;
-        if (ib == 4 && nb >= 4) {
-            if (ak == 4) radon_adj_launch<TI, TO, TC, 4, 4>(op, sb, xb, nb);
-            else if (ak == 16) radon_adj_launch<TI, TO, TC, 4, 16>(op, sb, xb, nb);
-            else radon_adj_launch<TI, TO, TC, 4, 8>(op, sb, xb, nb);
-        } else {
-            if (ak == 4) radon_adj_launch<TI, TO, TC, 1, 4>(op, sb, xb, nb);
-            else if (ak == 16) radon_adj_launch<TI, TO, TC, 1, 16>(op, sb, xb, nb);
-            else radon_adj_launch<TI, TO, TC, 1, 8>(op, sb, xb, nb);
-        }
+// angle ranges of the adjoint: as many as keep all CTAs resident at once (4 to
+// an SM) when the image has few tiles, at least 16 base angles each (one 512 x
+// 512 image, 256 tiles: 2 ranges 64 us, 3 ranges, a second wave of a quarter
+// of the SMs, 69 us)
+int adj_ranges(const nys_op* op, int groups, int n_base) {
+    const int64_t ctas = (int64_t)((op->n1 + ATS - 1) / ATS) * ((op->n2 + ATS - 1) / ATS) * groups;
+    const int64_t want = (int64_t)op->ctx->sm_count * 4;
+    return (int)std::max<int64_t>(1, std::min<int64_t>({want / ctas, n_base / 16, 16}));
+}
+
+template <class TC, int IB>
+size_t adj_smem(int AK) {
+    return sizeof(Lanes<TC, IB>) * 2 * AK * AWIN + sizeof(TileAng<TC>) * 3 * AK;
+}
+
+template <class TI, class TC, int IB>
+int prep(nys_op* op, const TI* x, int nb, const RSet& set) {
+    const int R = IB / set.V, groups = (nb + R - 1) / R, m = std::max(op->n1, op->n2);
+    auto* rows = (Lanes<TC, IB>*)op->lines;
+    auto* cols = set.V == 4 ? nullptr : rows + (size_t)groups * op->n1 * (op->n2 + PAD);
+    NYS_CK(op->ctx, launch_pdl(radon_prep_kernel<TI, TC, IB>, dim3((m + PAD + 31) / 32, (m + 31) / 32,
+                                                                    groups * (cols ? 2 : 1)), dim3(32, 8), 0,
+                               op->ctx->stream, x, rows, cols, op->n1, op->n2, set.V, nb));
+    NYS_LAUNCH_CK(op->ctx);
+    return NYS_OK;
+}
+
+template <class TI, class TO, class TC, int IB, bool LANES>
+int fwd_part(nys_op* op, const TI* x, void* y, int nb, int V) {
+    const RSet set = angle_set(op, V);
+    if (int st = prep<TI, TC, IB>(op, x, nb, set)) return st;
+    const int R = IB / V, groups = (nb + R - 1) / R;
+    const auto* rows = (const Lanes<TC, IB>*)op->lines;
+    const auto* cols = rows + (size_t)groups * op->n1 * (op->n2 + PAD);
+    auto go = [&](auto kern, int CB, int SEG) {
+        const int nch = (op->n_bins + 32 * CB - 1) / (32 * CB), fang = 8 / SEG;
+        return launch_pdl(kern, dim3((unsigned)((set.n_base + fang - 1) / fang * nch), groups), 256, 0,
+                          op->ctx->stream, rows, cols, y, op->n1, op->n2, op->n_angles, op->n_bins, nb, set);
+    };
+    // two bins per lane share the loop and the line when that leaves 32 warps
+    // to an SM; otherwise a warp takes one bin per lane and a quarter of the
+    // lines, four warps to a ray (one 512 x 512 image: 94 against 117 us
+    // without the quarters; two bins per lane for a batch: 25.5 against 28.4
+    // ms for three and 35 ms with one)
+    const int64_t warps = (int64_t)set.n_base * ((op->n_bins + 63) / 64) * groups;
+    if (warps >= (int64_t)op->ctx->sm_count * 32)
+        NYS_CK(op->ctx, go(radon_fwd_kernel<TC, TO, IB, 2, 1, LANES>, 2, 1));
+    else
+        NYS_CK(op->ctx, go(radon_fwd_kernel<TC, TO, IB, 1, 4, LANES>, 1, 4));
+    NYS_LAUNCH_CK(op->ctx);
+    return NYS_OK;
+}
+
+// adjoint of the interleaved lanes s
+template <class TO, class TC, int IB>
+int adj_lanes(nys_op* op, const void* s, TO* x, int nb, int V) {
+    const RSet set = angle_set(op, V);
+    const int R = IB / V, groups = (nb + R - 1) / R, AK = op->radon_adj_ak;
+    const int ns = adj_ranges(op, groups, set.n_base), per = (set.n_base + ns - 1) / ns;
+    const dim3 grid((op->n2 + ATS - 1) / ATS, (op->n1 + ATS - 1) / ATS, groups * ns);
+    const size_t sm = adj_smem<TC, IB>(AK);
+    const auto* sl = (const Lanes<TC, IB>*)s;
+    if (V == 1 && ns == 1) {
+        auto kern = radon_adj_kernel<TC, TO, IB, false>;
+        if (int st = smem_optin(op->ctx, (const void*)kern, sm)) return st;
+        NYS_CK(op->ctx, launch_pdl(kern, grid, 256, sm, op->ctx->stream, sl, x, op->n1, op->n2, op->n_bins, nb, AK, per,
+                                   set));
         NYS_LAUNCH_CK(op->ctx);
+        return NYS_OK;
     }
+    TC* planes = (TC*)op->planes;
+    auto kern = radon_adj_kernel<TC, TC, IB, true>;
+    if (int st = smem_optin(op->ctx, (const void*)kern, sm)) return st;
+    NYS_CK(op->ctx, launch_pdl(kern, grid, 256, sm, op->ctx->stream, sl, planes, op->n1, op->n2, op->n_bins, nb, AK, per,
+                               set));
+    NYS_LAUNCH_CK(op->ctx);
+    NYS_CK(op->ctx, launch_pdl(radon_sum_kernel<TC, TO, IB>, dim3((unsigned)std::min<int64_t>((op->N + 255) / 256, 1024),
+                                                                  nb), 256, 0, op->ctx->stream, (const TC*)planes, x,
+                               op->N, V, ns));
+    NYS_LAUNCH_CK(op->ctx);
     return NYS_OK;
+}
+
+template <class TI, class TO, class TC, int IB>
+int part_typed(nys_op* op, int which, const TI* x, TO* y, int nb, int V) {
+    if (which == 0) return fwd_part<TI, TO, TC, IB, false>(op, x, y, nb, V);
+    if (which == 1) {
+        const RSet set = angle_set(op, V);
+        const int R = IB / V, groups = (nb + R - 1) / R;
+        NYS_CK(op->ctx, launch_pdl(radon_lanes_kernel<TI, TC, IB>, dim3((op->n_bins + 255) / 256, set.n_base, groups),
+                                   256, 0, op->ctx->stream, x, (Lanes<TC, IB>*)op->inter, op->n_angles, op->n_bins, nb,
+                                   set));
+        NYS_LAUNCH_CK(op->ctx);
+    } else {
+        if (int st = fwd_part<TI, TO, TC, IB, true>(op, x, op->inter, nb, V)) return st;
+    }
+    return adj_lanes<TO, TC, IB>(op, op->inter, y, nb, V);
 }
 
 template <class TI, class TO, class TC>
 int radon_typed(nys_op* op, int which, const void* x, void* y, int batch) {
-    if (which == 0) return radon_fwd<TI, TO, TC>(op, x, y, batch);
-    if (which == 1) return radon_adj<TI, TO, TC>(op, x, y, batch);
-    for (int b0 = 0; b0 < batch; b0 += op->chunk) {
-        const int nb = std::min(op->chunk, batch - b0);
-        if (int st = radon_fwd<TI, TC, TC>(op, (const TI*)x + (size_t)b0 * op->N, op->inter, nb)) return st;
-        if (int st = radon_adj<TC, TO, TC>(op, op->inter, (TO*)y + (size_t)b0 * op->N, nb)) return st;
+    const int64_t in = which == 1 ? op->M : op->N, out = which == 0 ? op->M : op->N;
+    for (int b0 = 0; b0 < batch;) {
+        const Part p = next_part(op, std::min(op->chunk, batch - b0));
+        const TI* xb = (const TI*)x + (size_t)b0 * in;
+        TO* yb = (TO*)y + (size_t)b0 * out;
+        int st;
+        if (p.IB == 4) st = part_typed<TI, TO, TC, 4>(op, which, xb, yb, p.nb, p.V);
+        else if (p.IB == 2) st = part_typed<TI, TO, TC, 2>(op, which, xb, yb, p.nb, p.V);
+        else st = part_typed<TI, TO, TC, 1>(op, which, xb, yb, p.nb, p.V);
+        if (st) return st;
+        b0 += p.nb;
     }
     return NYS_OK;
 }
@@ -616,13 +660,24 @@ int radon_typed(nys_op* op, int which, const void* x, void* y, int batch) {
 }  // namespace
 
 int radon_setup(nys_op* op) {
-    const bool f64 = op->dtype == NYS_F64;
-    int st = f64 ? build_tables<double>(op) : build_tables<float>(op);
-    if (st) return st;
+    if (int st = build_tables(op)) return st;
     op->chunk = 32;
-    NYS_CK(op->ctx, cudaMalloc(&op->inter, (size_t)op->chunk * op->M * (f64 ? 8 : 4)));
-    // line-major copies for the forward: transposed + row-major, `chunk` images
-    NYS_CK(op->ctx, cudaMalloc(&op->lines, (size_t)2 * op->chunk * op->N * (f64 ? 8 : 4)));
+    const size_t es = op->dtype == NYS_F64 ? 8 : 4;
+    // interleaved sinogram lanes, image lines and the adjoint's planes, for
+    // every part that a chunk of images can be cut into
+    size_t lanes = 0, lines = 0, planes = 0;
+    for (int left = 1; left <= op->chunk; ++left) {
+        const Part p = next_part(op, left);
+        const RSet set = angle_set(op, p.V);
+        const int R = p.IB / p.V, groups = (p.nb + R - 1) / R, ns = adj_ranges(op, groups, set.n_base);
+        lanes = std::max(lanes, (size_t)groups * set.n_base * p.IB);
+        lines = std::max(lines, (size_t)groups * p.IB);
+        if (p.V > 1 || ns > 1) planes = std::max(planes, (size_t)groups * ns * p.IB);
+    }
+    NYS_CK(op->ctx, cudaMalloc(&op->inter, lanes * op->n_bins * es));
+    NYS_CK(op->ctx, cudaMalloc(&op->lines, lines * es * ((size_t)op->n1 * (op->n2 + PAD) +
+                                                         (size_t)op->n2 * (op->n1 + PAD))));
+    if (planes) NYS_CK(op->ctx, cudaMalloc(&op->planes, planes * op->N * es));
     return NYS_OK;
 }
 
