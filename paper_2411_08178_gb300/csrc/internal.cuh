@@ -91,6 +91,17 @@ struct nys_ctx {
     uint64_t scratch_gen = 0;
 };
 
+// fan beam: an angle set's lists within op->rtab, and where the tables lie
+struct nys_fan_set {
+    int n_base = 0, n_seg = 0;
+    size_t ang_off = 0, seg_off = 0;
+};
+struct nys_fan {
+    size_t ang_off = 0, rs_off = 0;
+    nys_fan_set set[3];               // one, two, four lanes
+    int frac = 0;                     // fraction bits of the adjoint's offsets
+};
+
 struct nys_op {
     nys_ctx* ctx = nullptr;
     int kind = 0, dtype = 0, n1 = 0, n2 = 0;
@@ -111,10 +122,11 @@ struct nys_op {
     int n_angles = 0, n_bins = 0;
     double span = 0.0;
     void* rtab = nullptr;             // per-angle tables, see radon.cu
-    void* lines = nullptr;            // radon: `chunk` images as interleaved lines (along rows and along columns)
-    void* planes = nullptr;           // radon adjoint: partial images (lanes and angle ranges) of a launch
-    int radon_sets = 1;               // radon: mirror lanes the angles allow (1, 2 and 4 or'ed, see radon.cu)
+    void* lines = nullptr;            // rays: `chunk` images as interleaved lines (along rows and along columns)
+    void* planes = nullptr;           // ray adjoints: partial images (lanes and angle ranges) of a launch
+    int lane_sets = 1;                // rays: mirror lanes the angles allow (1, 2 and 4 or'ed, see ray_lanes.cuh)
     double src_dist = 0.0, det_dist = 0.0, det_spacing = 1.0;   // fan beam
+    nys_fan fan;
     int radon_adj_ak = 16;            // radon adjoint: angles per round, 4, 8 or 16 (nys_op_autotune)
     int blur_tile = 64;               // blur: output tile side, 32 or 64 (float32; chosen by nys_op_autotune)
     // intermediate buffer for two-pass normals (M per image, `chunk` images)

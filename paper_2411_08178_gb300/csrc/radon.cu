@@ -19,30 +19,22 @@
 // in the forward, 26 in the adjoint, relative to a 32 x 32 tile) or to the
 // last float64 bits, and the two are transposes of each other to rounding.
 //
-// Lanes.  Positions and weights cost as much as the arithmetic on the data,
-// so both kernels carry IB values per position, interleaved in memory (one
-// 16-byte load feeds four float32 lanes).  A lane is an image of a batch, or
-// one of V mirror images of the same image: over 180 degrees, angle
-// n_angles - k sees the left-right mirrored image exactly as angle k sees the
-// image, and for a square image and an even number of angles n_angles/2 -+ k
-// do the same with the transposed image and its mirror image.  Base angles
-// k = 0 .. n_base - 1 and ang[k][v], the angle of lane v (-1: none, the lane
-// is a copy of another angle's), describe the set (RSet below).
+// Lanes (ray_lanes.cuh).  Over 180 degrees, angle n_angles - k sees the
+// left-right mirrored image exactly as angle k sees the image, and for a
+// square image and an even number of angles n_angles/2 -+ k do the same with
+// the transposed image and its mirror image: a single image has two or four
+// lanes too.
 //
-// Kernels: radon_prep (images to interleaved lines with zero margins, for
+// Kernels: lane_prep (images to interleaved lines with zero margins, for
 // row-step angles along rows, for column-step ones along columns), radon_fwd
-// (rays), radon_lanes (a planar sinogram to interleaved lanes), radon_adj
-// (pixels), radon_sum (the lanes and angle ranges of one image added up).
-#include "internal.cuh"
+// (rays), lane_bins (a planar sinogram to interleaved lanes), radon_adj
+// (pixels), lane_sum (the lanes and angle ranges of one image added up).
+#include "ray_lanes.cuh"
 
-#include <algorithm>
 #include <cmath>
-#include <type_traits>
 
 namespace nys {
 namespace {
-
-constexpr int PAD = 3;    // zeros of an interleaved line: one before, two after
 
 // per-angle geometry, float64; the ray positions of float32 operators also as
 // integers with 40 fraction bits (GB300 issues a float64 operation every 16
@@ -55,113 +47,19 @@ struct RGeo {
     int rs, pad;          // row-step angle
 };
 
-// the angles of a launch: base angle kb's geometry is geo[ang[kb V]], its lane
-// v holds angle ang[kb V + v] or, when negative, nothing
-struct RSet {
+// the angles of a launch: geo[ang[kb V]] is the geometry of base angle kb
+struct RSet : LaneSet {
     const RGeo* geo;
-    const int* ang;
-    int V, n_base;
 };
 
-template <class TC, int IB>
-struct alignas(sizeof(TC) * IB >= 16 ? 16 : sizeof(TC) * IB) Lanes {
-    TC v[IB];
-};
-
-// source pixel of lane variant v at (line, pos) of orientation o (0: lines are
-// rows, 1: columns): 0 the image, 1 mirrored in j, 2 transposed, 3 transposed
-// and mirrored (2 and 3: square images)
-__device__ __forceinline__ void variant_src(int v, int& i, int& j, int n1, int n2) {
-    if (v == 1) j = n2 - 1 - j;
-    else if (v >= 2) {
-        const int t = i;
-        i = j;
-        j = v == 2 ? t : n1 - 1 - t;
-    }
+__device__ __forceinline__ void ray_at(RayPos<float>& p, const RGeo& g, int m, int l) {
+    p.set40(g.u0q + m * g.invq - l * g.tq);
 }
-
-// interleaved lines: rows[g][i][1 + j] and, when the set has column-step base
-// angles (cols), cols[g][j][1 + i]; lane q of group g is variant q % V of
-// image g IB / V + q / V.  One CTA writes 32 lines x 32 positions: every lane
-// is read with its image's rows along the threads, through shared memory.
-template <class TI, class TC, int IB>
-__global__ void __launch_bounds__(256) radon_prep_kernel(const TI* __restrict__ x, Lanes<TC, IB>* __restrict__ rows,
-                                                         Lanes<TC, IB>* __restrict__ cols, int n1, int n2, int V,
-                                                         int batch) {
-    pdl_enter();
-    __shared__ TC tile[IB][32][33];
-    const int o = cols ? (int)(blockIdx.z & 1) : 0, g = cols ? blockIdx.z >> 1 : blockIdx.z;
-    const int nl = o ? n2 : n1, na = o ? n1 : n2;
-    const int l0 = blockIdx.y * 32, p0 = blockIdx.x * 32 - 1;
-    if (l0 >= nl || p0 >= na + PAD - 1) return;
-    const int R = IB / V;
-    const size_t N = (size_t)n1 * n2;
-#pragma unroll
-    for (int q = 0; q < IB; ++q) {
-        const int b = g * R + q / V, v = q % V;
-        const bool along = (o == 0) == (v < 2);      // the source's j runs along the line's positions
-        for (int r = threadIdx.y; r < 32; r += 8) {
-            const int dl = along ? r : threadIdx.x, dp = along ? threadIdx.x : r;
-            const int l = l0 + dl, p = p0 + dp;
-            TC val = TC(0);
-            if (b < batch && l < nl && p >= 0 && p < na) {
-                int i = o ? p : l, j = o ? l : p;
-                variant_src(v, i, j, n1, n2);
-                val = (TC)ldf(x + (size_t)b * N + (size_t)i * n2 + j);
-            }
-            tile[q][dl][dp] = val;
-        }
-    }
-    __syncthreads();
-    Lanes<TC, IB>* dst = (o ? cols : rows) + (size_t)g * nl * (na + PAD);
-    for (int r = threadIdx.y; r < 32; r += 8) {
-        const int l = l0 + r, e = p0 + 1 + threadIdx.x;
-        if (l < nl && e < na + PAD) {
-            Lanes<TC, IB> w;
-#pragma unroll
-            for (int q = 0; q < IB; ++q) w.v[q] = tile[q][r][threadIdx.x];
-            dst[(size_t)l * (na + PAD) + e] = w;
-        }
-    }
+__device__ __forceinline__ void ray_at(RayPos<double>& p, const RGeo& g, int m, int l) {
+    p.set(fma((double)m, g.inv, fma(-(double)l, g.t, g.u0)));
 }
-
-// position of a ray on its line, stepped line by line: an integer part and a
-// binary fraction of 32 (float) or 64 (double) bits; weight() is the fraction
-// as 1 + f in [1, 2)
-template <class TC>
-struct RayPos;
-template <>
-struct RayPos<float> {
-    long long p;
-    __device__ __forceinline__ void set(const RGeo& g, int m, int l) { p = (g.u0q + m * g.invq - l * g.tq + 128) >> 8; }
-    __device__ __forceinline__ void set_step(const RGeo& g) { p = (128 - g.tq) >> 8; }
-    __device__ __forceinline__ void step(const RayPos& d) { p += d.p; }
-    __device__ __forceinline__ int index() const { return (int)(p >> 32); }
-    __device__ __forceinline__ float one_plus_f() const {
-        return __uint_as_float(((unsigned)p >> 9) + 0x3f800000u);
-    }
-};
-template <>
-struct RayPos<double> {
-    int i;
-    unsigned long long f;
-    __device__ __forceinline__ void set(double u) {
-        const double fl = floor(u);
-        i = (int)fl;
-        f = (unsigned long long)((u - fl) * 18446744073709551616.0);   // 2^64; saturates below it
-    }
-    __device__ __forceinline__ void set(const RGeo& g, int m, int l) { set(fma((double)m, g.inv, fma(-(double)l, g.t, g.u0))); }
-    __device__ __forceinline__ void set_step(const RGeo& g) { set(-g.t); }
-    __device__ __forceinline__ void step(const RayPos& d) {
-        const unsigned long long s = f + d.f;
-        i += d.i + (s < f ? 1 : 0);
-        f = s;
-    }
-    __device__ __forceinline__ int index() const { return i; }
-    __device__ __forceinline__ double one_plus_f() const {
-        return __longlong_as_double((long long)((f >> 12) | 0x3ff0000000000000ull));
-    }
-};
+__device__ __forceinline__ void ray_step(RayPos<float>& p, const RGeo& g) { p.set40(-g.tq); }
+__device__ __forceinline__ void ray_step(RayPos<double>& p, const RGeo& g) { p.set(-g.t); }
 
 // Forward: a warp takes 32 CB consecutive bins of one base angle (CB per lane,
 // 32 apart, so that a load's addresses stay together) and steps along a SEG-th
@@ -198,10 +96,10 @@ __global__ void __launch_bounds__(256) radon_fwd_kernel(const Lanes<TC, IB>* __r
     // one interval (u is monotone in m), taken with two lines of margin;
     // outside it every sample is out of range and adds exactly zero
     RayPos<TC> pos[CB], dt;
-    dt.set_step(geo);
-    pos[0].set(geo, m0, 0);
+    ray_step(dt, geo);
+    ray_at(pos[0], geo, m0, 0);
     const float qa = (float)(pos[0].index() - 1);
-    pos[0].set(geo, min(m0 + 32 * CB - 1, n_bins - 1), 0);
+    ray_at(pos[0], geo, min(m0 + 32 * CB - 1, n_bins - 1), 0);
     const float qb = (float)(pos[0].index() - 1);
     const float qmin = fminf(qa, qb), qmax = fmaxf(qa, qb) + 1.0f, tl = (float)geo.tq * 0x1p-40f;
     int l_beg = 0, l_end = nl;
@@ -221,7 +119,7 @@ __global__ void __launch_bounds__(256) radon_fwd_kernel(const Lanes<TC, IB>* __r
     TC acc[CB][IB];
 #pragma unroll
     for (int c = 0; c < CB; ++c) {
-        pos[c].set(geo, m0 + 32 * c + lane, l_beg);
+        ray_at(pos[c], geo, m0 + 32 * c + lane, l_beg);
 #pragma unroll
         for (int q = 0; q < IB; ++q) acc[c][q] = TC(0);
     }
@@ -279,24 +177,6 @@ __global__ void __launch_bounds__(256) radon_fwd_kernel(const Lanes<TC, IB>* __r
     }
 }
 
-// planar sinogram (images x angles x bins) to the interleaved lanes [g][kb][m]
-template <class TI, class TC, int IB>
-__global__ void __launch_bounds__(256) radon_lanes_kernel(const TI* __restrict__ s, Lanes<TC, IB>* __restrict__ out,
-                                                          int n_angles, int n_bins, int batch, RSet set) {
-    pdl_enter();
-    const int kb = blockIdx.y, g = blockIdx.z;
-    const int* ang = set.ang + kb * set.V;
-    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < n_bins; m += gridDim.x * blockDim.x) {
-        Lanes<TC, IB> w;
-#pragma unroll
-        for (int q = 0; q < IB; ++q) {
-            const int b = g * (IB / set.V) + q / set.V, a = ang[q % set.V];
-            w.v[q] = b < batch && a >= 0 ? (TC)ldf(s + ((size_t)b * n_angles + a) * n_bins + m) : TC(0);
-        }
-        out[((size_t)g * set.n_base + kb) * n_bins + m] = w;
-    }
-}
-
 // Fixed-point bin position within a tile's window: 6 integer bits (a 32 x 32
 // tile spans at most 31 sqrt(2) + 2 < 46 bins)
 template <class TC>
@@ -332,14 +212,6 @@ struct alignas(16) TileAng {           // one base angle as a tile sees it
     TC wb, w0, w1;                     // lower bin's weight max(0, w0 - wb F), upper's max(0, w1 + wb F), F = 1 + f
     int mlo;                           // first staged bin
 };
-
-__device__ __forceinline__ void cp_async_zfill(void* dst, const void* src, int bytes, bool ok) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    const int n = ok ? bytes : 0;
-    if (bytes == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n));
-    else if (bytes == 8) asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(n));
-    else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(n));
-}
 
 // Adjoint: one CTA per (32 x 32 tile, group of lanes, range of base angles).
 // AK angles per round: their windows of bins and per-tile constants are staged
@@ -445,7 +317,7 @@ __global__ void __launch_bounds__(256) radon_adj_kernel(const Lanes<TC, IB>* __r
         for (int q = 0; q < IB; ++q) {
             if constexpr (PLANES) {
                 int si = i, sj = j;
-                variant_src(q % set.V, si, sj, n1, n2);
+                lane_src(set.sym(q % set.V), si, sj, n1, n2);
                 const size_t plane = ((size_t)g * (gridDim.z / ((batch + IB / set.V - 1) / (IB / set.V))) + z) * IB + q;
                 stf(out + plane * N + (size_t)si * n2 + sj, acc[u][q]);
             } else {
@@ -453,20 +325,6 @@ __global__ void __launch_bounds__(256) radon_adj_kernel(const Lanes<TC, IB>* __r
                 if (b < batch) stf(out + (size_t)b * N + (size_t)i * n2 + j, acc[u][q]);
             }
         }
-    }
-}
-
-// x[b] = the sum of image b's planes: ns angle ranges x V lanes
-template <class TC, class TO, int IB>
-__global__ void __launch_bounds__(256) radon_sum_kernel(const TC* __restrict__ planes, TO* __restrict__ x, int64_t N,
-                                                        int V, int ns) {
-    pdl_enter();
-    const int b = blockIdx.y, R = IB / V, g = b / R, q0 = (b - g * R) * V;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < N; t += (int64_t)gridDim.x * blockDim.x) {
-        TC v = TC(0);
-        for (int z = 0; z < ns; ++z)
-            for (int q = 0; q < V; ++q) v += planes[(((size_t)g * ns + z) * IB + q0 + q) * N + t];
-        stf(x + (size_t)b * N + t, v);
     }
 }
 
@@ -489,10 +347,10 @@ int build_tables(nys_op* op) {
     // the angle sets: every angle by itself, and over exactly 180 degrees the
     // mirror pairs and (square image, even number of angles) the fours
     std::vector<int> ang;
-    op->radon_sets = 1;
+    op->lane_sets = 1;
     for (int k = 0; k < A; ++k) ang.push_back(k);
     auto add = [&](int V, int n_base, auto&& lane) {
-        op->radon_sets |= V;
+        op->lane_sets |= V;
         for (int k = 0; k < n_base; ++k) {
             const size_t first = ang.size();
             for (int v = 0; v < V; ++v) {
@@ -523,22 +381,10 @@ RSet angle_set(const nys_op* op, int V) {
     r.geo = (const RGeo*)op->rtab;
     r.V = V;
     r.n_base = V == 1 ? A : A / V + 1;
+    // lane v > 0: mirrored in j, transposed, both
+    r.tf = V == 1 ? 0 : LANE_FJ << 4 | LANE_T << 8 | (LANE_T | LANE_FJ) << 12;
     r.ang = V == 1 ? ang : V == 2 ? ang + A : ang + A + 2 * (A / 2 + 1);
     return r;
-}
-
-// Lanes and mirror lanes for a part of a batch: fours of images while there
-// are four; a rest of one to three takes four mirror lanes an image where the
-// angles allow it (a quarter of the angles each), else two (two images to a
-// launch group), else plain lanes.
-struct Part {
-    int nb, IB, V;
-};
-Part next_part(const nys_op* op, int left) {
-    if (left >= 4) return {left / 4 * 4, 4, 1};
-    if (op->radon_sets & 4) return {left, 4, 4};
-    if (op->radon_sets & 2) return left == 1 ? Part{1, 2, 2} : Part{left, 4, 2};
-    return {left, left == 3 ? 4 : left, 1};
 }
 
 // angle ranges of the adjoint: as many as keep all CTAs resident at once (4 to
@@ -556,28 +402,16 @@ size_t adj_smem(int AK) {
     return sizeof(Lanes<TC, IB>) * 2 * AK * AWIN + sizeof(TileAng<TC>) * 3 * AK;
 }
 
-template <class TI, class TC, int IB>
-int prep(nys_op* op, const TI* x, int nb, const RSet& set) {
-    const int R = IB / set.V, groups = (nb + R - 1) / R, m = std::max(op->n1, op->n2);
-    auto* rows = (Lanes<TC, IB>*)op->lines;
-    auto* cols = set.V == 4 ? nullptr : rows + (size_t)groups * op->n1 * (op->n2 + PAD);
-    NYS_CK(op->ctx, launch_pdl(radon_prep_kernel<TI, TC, IB>, dim3((m + PAD + 31) / 32, (m + 31) / 32,
-                                                                    groups * (cols ? 2 : 1)), dim3(32, 8), 0,
-                               op->ctx->stream, x, rows, cols, op->n1, op->n2, set.V, nb));
-    NYS_LAUNCH_CK(op->ctx);
-    return NYS_OK;
-}
-
 template <class TI, class TO, class TC, int IB, bool LANES>
 int fwd_part(nys_op* op, const TI* x, void* y, int nb, int V) {
     const RSet set = angle_set(op, V);
-    if (int st = prep<TI, TC, IB>(op, x, nb, set)) return st;
+    if (int st = lane_prep<TI, TC, IB>(op, x, nb, set, V < 4)) return st;
     const int R = IB / V, groups = (nb + R - 1) / R;
     const auto* rows = (const Lanes<TC, IB>*)op->lines;
     const auto* cols = rows + (size_t)groups * op->n1 * (op->n2 + PAD);
-    auto go = [&](auto kern, int CB, int SEG) {
+    auto go = [&](auto kernel, int CB, int SEG) {
         const int nch = (op->n_bins + 32 * CB - 1) / (32 * CB), fang = 8 / SEG;
-        return launch_pdl(kern, dim3((unsigned)((set.n_base + fang - 1) / fang * nch), groups), 256, 0,
+        return launch_pdl(kernel, dim3((unsigned)((set.n_base + fang - 1) / fang * nch), groups), 256, 0,
                           op->ctx->stream, rows, cols, y, op->n1, op->n2, op->n_angles, op->n_bins, nb, set);
     };
     // two bins per lane share the loop and the line when that leaves 32 warps
@@ -617,23 +451,14 @@ int adj_lanes(nys_op* op, const void* s, TO* x, int nb, int V) {
     NYS_CK(op->ctx, launch_pdl(kern, grid, 256, sm, op->ctx->stream, sl, planes, op->n1, op->n2, op->n_bins, nb, AK, per,
                                set));
     NYS_LAUNCH_CK(op->ctx);
-    NYS_CK(op->ctx, launch_pdl(radon_sum_kernel<TC, TO, IB>, dim3((unsigned)std::min<int64_t>((op->N + 255) / 256, 1024),
-                                                                  nb), 256, 0, op->ctx->stream, (const TC*)planes, x,
-                               op->N, V, ns));
-    NYS_LAUNCH_CK(op->ctx);
-    return NYS_OK;
+    return lane_sum<TC, TO, IB>(op, x, nb, V, ns);
 }
 
 template <class TI, class TO, class TC, int IB>
 int part_typed(nys_op* op, int which, const TI* x, TO* y, int nb, int V) {
     if (which == 0) return fwd_part<TI, TO, TC, IB, false>(op, x, y, nb, V);
     if (which == 1) {
-        const RSet set = angle_set(op, V);
-        const int R = IB / V, groups = (nb + R - 1) / R;
-        NYS_CK(op->ctx, launch_pdl(radon_lanes_kernel<TI, TC, IB>, dim3((op->n_bins + 255) / 256, set.n_base, groups),
-                                   256, 0, op->ctx->stream, x, (Lanes<TC, IB>*)op->inter, op->n_angles, op->n_bins, nb,
-                                   set));
-        NYS_LAUNCH_CK(op->ctx);
+        if (int st = lane_bins<TI, TC, IB>(op, x, nb, angle_set(op, V))) return st;
     } else {
         if (int st = fwd_part<TI, TO, TC, IB, true>(op, x, op->inter, nb, V)) return st;
     }
