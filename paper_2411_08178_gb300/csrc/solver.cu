@@ -94,10 +94,17 @@ __global__ void momentum_kernel(const T* __restrict__ xn, const T* __restrict__ 
                                 double* __restrict__ t_out, int64_t n, T* __restrict__ u) {
     pdl_enter();
     using TC = typename Comp<T>::type;
-    const double t = *t_in;
-    const double tn = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
-    const TC b = (TC)((t - 1.0) / tn);
-    if (blockIdx.x == 0 && threadIdx.x == 0) *t_out = tn;
+    // one thread per block: a float64 root and quotient in every thread took
+    // most of the kernel (13.6 us at 512 x 512)
+    __shared__ TC bs;
+    if (threadIdx.x == 0) {
+        const double t = *t_in;
+        const double tn = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
+        bs = (TC)((t - 1.0) / tn);
+        if (blockIdx.x == 0) *t_out = tn;
+    }
+    __syncthreads();
+    const TC b = bs;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const TC a = (TC)xn[i];
         u[i] = (T)(a + b * (a - (TC)x[i]));
