@@ -28,7 +28,11 @@
 #include "chol.cuh"
 #include "stencil.cuh"
 
+#include <cooperative_groups.h>
+
 #include <cmath>
+
+namespace cg = cooperative_groups;
 
 namespace nys {
 
@@ -279,13 +283,12 @@ __global__ void __launch_bounds__(1024) ssn_step_kernel(int nb, int ell, double 
                                                         const double* __restrict__ Fp, const double* __restrict__ Sp,
                                                         const float* __restrict__ Jp, double* __restrict__ gamma,
                                                         double* __restrict__ gtrial, double* __restrict__ dir,
-                                                        double* __restrict__ Fcur, double* __restrict__ Jw,
-                                                        SsnState* __restrict__ st) {
+                                                        double* __restrict__ Fcur, SsnState* __restrict__ st) {
     pdl_enter();
     if (st->done) return;
-    __shared__ double F[SMAXL];
+    extern __shared__ __align__(16) double Jw[];   // (ell + 1) x (ell + 1): J and, as the last row, -F
+    __shared__ double F[SMAXL], inv[SMAXL];
     __shared__ double sh[32];
-    __shared__ int flag;
     __shared__ int accept;
     for (int j = threadIdx.x; j < ell; j += blockDim.x) {
         double f = 0.0, sv = 0.0;
@@ -321,11 +324,12 @@ __global__ void __launch_bounds__(1024) ssn_step_kernel(int nb, int ell, double 
     for (int j = threadIdx.x; j < ell; j += blockDim.x) gamma[j] = gtrial[j], Fcur[j] = F[j];
     for (int e = threadIdx.x; e < ell * ell; e += blockDim.x) {
         const int j = e / ell, k = e - j * ell;
-        const int a = min(j, k), b = max(j, k);
+        if (k < j) continue;
         double v = 0.0;
-        for (int q = 0; q < nb; ++q) v += (double)Jp[(size_t)q * ell * ell + (size_t)a * ell + b];
-        Jw[e] = v + (j == k ? 1.0 : 0.0);
+        for (int q = 0; q < nb; ++q) v += (double)Jp[(size_t)q * ell * ell + e];
+        Jw[k * (ell + 1) + j] = v + (j == k ? 1.0 : 0.0);
     }
+    for (int j = threadIdx.x; j < ell; j += blockDim.x) Jw[ell * (ell + 1) + j] = -F[j];
     __syncthreads();
     if (threadIdx.x == 0) {
         if (!st->first) st->newton += 1;
@@ -338,25 +342,11 @@ __global__ void __launch_bounds__(1024) ssn_step_kernel(int nb, int ell, double 
     }
     __syncthreads();
     if (st->done) return;
-    // Newton direction: J d = -F (Cholesky, forward and back substitution)
-    const bool ok = block_cholesky(Jw, ell, &flag);
-    if (!ok) {
+    // Newton direction: J d = -F
+    if (!block_ldl_solve(Jw, ell + 1, ell, inv, dir)) {
         if (threadIdx.x == 0) st->done = 1;
         return;
     }
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < ell; ++i) {
-            double v = -F[i];
-            for (int k = 0; k < i; ++k) v -= Jw[(size_t)i * ell + k] * dir[k];
-            dir[i] = v / Jw[(size_t)i * ell + i];
-        }
-        for (int i = ell - 1; i >= 0; --i) {
-            double v = dir[i];
-            for (int k = i + 1; k < ell; ++k) v -= Jw[(size_t)k * ell + i] * dir[k];
-            dir[i] = v / Jw[(size_t)i * ell + i];
-        }
-    }
-    __syncthreads();
     for (int j = threadIdx.x; j < ell; j += blockDim.x) gtrial[j] = gamma[j] + dir[j];
 }
 
@@ -369,6 +359,208 @@ __global__ void ssn_final_kernel(const T* __restrict__ U, const double* __restri
         for (int j = 0; j < ell; ++j) z -= sqd[j] * (double)U[(size_t)j * N + i] * gamma[j];
         out[i] = (T)soft(z, tau);
     }
+}
+
+// The whole Newton iteration in one launch, for factors that fit the shared
+// memory of a cluster of SCC CTAs (64 x 64 in float64 with 32 columns: 68 KB
+// each): CTA c holds pixels c np .. of the active columns, scaled sums are
+// exchanged through distributed shared memory, every CTA takes the accept /
+// halve decisions from the same sums, and rank 0 solves for the direction.
+// Three cluster barriers per accepted step, one per rejected one; no spin
+// waits, at most max_evals evaluations.  Ten iterations of the 64 x 64 solve:
+// 4.8 ms with an evaluation and a one-CTA step kernel per evaluation, most of
+// it in serial triangular solves on global memory (37 us per step launch).
+constexpr int SCC = 16;
+constexpr int SCT = 512;
+inline __host__ __device__ size_t ssn_cluster_smem(int r, int np, size_t es) {
+    return (size_t)(3 * np + 8 * r + (r + 1) * (r + 1)) * sizeof(double) + (size_t)r * np * es +
+           ((size_t)r * np + (size_t)r * r) * sizeof(float) + 64;
+}
+
+template <class T>
+__global__ void __launch_bounds__(SCT, 1)
+    ssn_cluster_kernel(const T* __restrict__ U, const double* __restrict__ sqd, const T* __restrict__ s, int64_t N,
+                       int np, int r, double tau, double tol, int max_newton, int max_evals,
+                       double* __restrict__ gamma_io, int ell, T* __restrict__ out, SsnState* __restrict__ info) {
+    pdl_enter();
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    extern __shared__ __align__(16) double sc_smem[];
+    double* zs = sc_smem;                 // soft(z)
+    double* rr = zs + np;                 // s - soft(z)
+    double* ss = rr + np;
+    double* sd = ss + np;                 // r each: sqrt(d), gamma, trial, direction, F, partial F (two), partial Ubar^T s
+    double* gam = sd + r;
+    double* gt = gam + r;
+    double* dir = gt + r;
+    double* F = dir + r;
+    double* Fp = F + r;
+    double* Sp = Fp + 2 * r;
+    double* M = Sp + r;                   // (r + 1) x (r + 1), rank 0
+    float* ub = reinterpret_cast<float*>(M + (r + 1) * (r + 1));   // Ubar in float32
+    float* Jp = ub + (size_t)r * np;      // this CTA's J, upper triangle
+    T* Us = reinterpret_cast<T*>(Jp + (size_t)r * r + ((r * np + r * r) & 1));
+    __shared__ double inv[SMAXL], sh[32];
+    __shared__ int fail_flag;
+    const int64_t i0 = (int64_t)rank * np;
+    const int cnt = (int)max((int64_t)0, min((int64_t)np, N - i0));
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int NW = SCT / 32;
+    for (int j = threadIdx.x; j < r; j += SCT) {
+        sd[j] = sqd[j];
+        gam[j] = gt[j] = gamma_io ? gamma_io[j] : 0.0;
+    }
+    for (int t = threadIdx.x; t < np; t += SCT) ss[t] = t < cnt ? (double)s[i0 + t] : 0.0;
+    for (int j = warp; j < r; j += NW) {
+        const double dj = sqd[j];
+        for (int t = lane; t < np; t += 32) {
+            const T u = t < cnt ? U[(size_t)j * N + i0 + t] : T(0);
+            Us[(size_t)j * np + t] = u;
+            ub[(size_t)j * np + t] = (float)(dj * (double)u);
+        }
+    }
+    if (threadIdx.x == 0) fail_flag = 0;
+    __syncthreads();
+    auto soft_z = [&](const double* g, int t) -> double {     // T_tau(s - Ubar g) at pixel t
+        double z0 = ss[t], z1 = 0.0;
+        int j = 0;
+        for (; j + 1 < r; j += 2) {
+            z0 -= sd[j] * g[j] * (double)Us[(size_t)j * np + t];
+            z1 -= sd[j + 1] * g[j + 1] * (double)Us[(size_t)(j + 1) * np + t];
+        }
+        if (j < r) z0 -= sd[j] * g[j] * (double)Us[(size_t)j * np + t];
+        return soft(z0 + z1, tau);
+    };
+    double nF = 0.0, a = 1.0, scale = 1.0;
+    int tries = 0, newton = 0;
+    bool done = false, converged = false, current = false;   // current: zs belongs to gam
+    for (int e = 0; e < max_evals && !done; ++e) {
+        double* Fe = Fp + (e & 1) * r;
+        for (int t = threadIdx.x; t < np; t += SCT) {
+            const double z = t < cnt ? soft_z(gt, t) : 0.0;
+            zs[t] = z;
+            rr[t] = ss[t] - z;
+        }
+        __syncthreads();
+        for (int j = warp; j < r; j += NW) {
+            double f = 0.0, v = 0.0;
+            for (int t = lane; t < cnt; t += 32) {
+                const double u = (double)Us[(size_t)j * np + t];
+                f += u * rr[t];
+                if (e == 0) v += u * ss[t];
+            }
+            f = warp_sum(f);
+            if (e == 0) v = warp_sum(v);
+            if (lane == 0) {
+                Fe[j] = sd[j] * f;
+                if (e == 0) Sp[j] = sd[j] * v;
+            }
+        }
+        cluster.sync();
+        // the same sums in the same order in every CTA.  Fe is written again two
+        // evaluations on, past a barrier that follows every CTA's reads here
+        double n2 = 0.0, s2 = 0.0;
+        for (int j = threadIdx.x; j < r; j += SCT) {
+            double f = 0.0, v = 0.0;
+            for (int c = 0; c < SCC; ++c) {
+                f += *cluster.map_shared_rank(Fe + j, c);
+                if (e == 0) v += *cluster.map_shared_rank(Sp + j, c);
+            }
+            f += gt[j];
+            F[j] = f;
+            n2 += f * f;
+            s2 += v * v;
+        }
+        n2 = block_sum(n2, sh);
+        if (e == 0) scale = 1.0 + sqrt(block_sum(s2, sh));
+        const double nt = sqrt(n2);
+        // accept when first, improved, or after the 11th trial of this step
+        if (!(e == 0 || nt < nF || tries >= 10)) {
+            tries += 1;
+            a *= 0.5;
+            current = false;
+            for (int j = threadIdx.x; j < r; j += SCT) gt[j] = gam[j] + a * dir[j];
+            __syncthreads();
+            continue;
+        }
+        for (int j = threadIdx.x; j < r; j += SCT) gam[j] = gt[j];
+        current = true;
+        if (e) newton += 1;
+        nF = nt;
+        tries = 0;
+        a = 1.0;
+        if (nF <= tol * scale) done = converged = true;
+        else if (newton >= max_newton) done = true;
+        if (done || e + 1 >= max_evals) break;
+        // J = I + sum over the support of ub ub^T: 4 x 4 tiles, one per warp
+        const int nt4 = (r + 3) / 4;
+        for (int q = warp; q < nt4 * nt4; q += NW) {
+            const int tj = q / nt4, tk = q - tj * nt4;
+            if (tk < tj) continue;
+            float acc[4][4] = {};
+            for (int t = lane; t < cnt; t += 32) {
+                const float m = zs[t] != 0.0 ? 1.0f : 0.0f;    // |z| > tau
+                float uj[4], uk[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    uj[c] = m * ub[(size_t)min(4 * tj + c, r - 1) * np + t];
+                    uk[c] = ub[(size_t)min(4 * tk + c, r - 1) * np + t];
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+#pragma unroll
+                    for (int d = 0; d < 4; ++d) acc[c][d] = fmaf(uj[c], uk[d], acc[c][d]);
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+#pragma unroll
+                for (int d = 0; d < 4; ++d) {
+                    const float v = warp_sum(acc[c][d]);
+                    if (lane == 0 && 4 * tj + c < r && 4 * tk + d < r) Jp[(size_t)(4 * tj + c) * r + 4 * tk + d] = v;
+                }
+        }
+        cluster.sync();
+        if (rank == 0) {
+            for (int e2 = threadIdx.x; e2 < r * r; e2 += SCT) {
+                const int j = e2 / r, k = e2 - j * r;
+                if (k < j) continue;
+                double v = 0.0;
+                for (int c = 0; c < SCC; ++c) v += (double)*cluster.map_shared_rank(Jp + e2, c);
+                M[(size_t)k * (r + 1) + j] = v + (j == k ? 1.0 : 0.0);
+            }
+            for (int j = threadIdx.x; j < r; j += SCT) M[(size_t)r * (r + 1) + j] = -F[j];
+            __syncthreads();
+            if (block_ldl_solve(M, r + 1, r, inv, dir)) {
+                for (int t = threadIdx.x; t < r * (SCC - 1); t += SCT) {
+                    const int c = t / r + 1, j = t % r;
+                    *cluster.map_shared_rank(dir + j, c) = dir[j];
+                }
+            } else if (threadIdx.x < SCC) {
+                *cluster.map_shared_rank(&fail_flag, (int)threadIdx.x) = 1;
+            }
+        }
+        cluster.sync();
+        if (fail_flag) break;
+        for (int j = threadIdx.x; j < r; j += SCT) gt[j] = gam[j] + dir[j];
+        __syncthreads();
+    }
+    if (!current) {
+        __syncthreads();
+        for (int t = threadIdx.x; t < cnt; t += SCT) zs[t] = soft_z(gam, t);
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < cnt; t += SCT) out[i0 + t] = (T)zs[t];
+    if (rank == 0) {
+        if (gamma_io)
+            for (int j = threadIdx.x; j < ell; j += SCT) gamma_io[j] = j < r ? gam[j] : 0.0;
+        if (info && threadIdx.x == 0) {
+            info->newton = newton;
+            info->converged = converged;
+            info->nF = nF;
+        }
+    }
+    // no CTA leaves while another may still read its shared memory
+    cluster.sync();
 }
 
 template <class T>
@@ -399,19 +591,34 @@ __global__ void ssn_init_kernel(SsnState* st, const double* gamma_in, double* ga
 
 }  // namespace
 
-// Semi-smooth Newton prox; `max_evals` evaluation/step pairs are launched
-// (later ones exit at once when done).  If `sync_until_done`, the host keeps
-// launching batches until the device reports completion.
+template <class T>
+int soft_run(nys_ctx* ctx, double tau, int64_t N, const T* s, T* out) {
+    const int grid = (int)std::min<int64_t>((N + 255) / 256, ctx->sm_count * 8);
+    NYS_CK(ctx, launch_pdl(soft_kernel<T>, grid, 256, 0, ctx->stream, s, N, tau, out));
+    NYS_LAUNCH_CK(ctx);
+    return NYS_OK;
+}
+// Semi-smooth Newton prox over the active columns (a column with d_j = 0 has
+// Ubar_j = 0 and gamma_j = 0).  One cluster launch where the factor fits (see
+// ssn_cluster_kernel); otherwise evaluation / step pairs are launched (later
+// ones exit at once when done).  If `sync_until_done`, the host keeps launching
+// batches until the device reports completion.
 template <class T>
 int ssn_run(nys_ctx* ctx, const nys_precond* pc, double tau, int64_t N, const T* s, T* out, double* gamma_io,
             int max_newton, int evals_per_batch, bool sync_until_done, nys_prox_info* info) {
-    const int ell = pc->ell;
-    if (ell > SMAXL) return fail(ctx, NYS_EINVAL, "prox_wavelet: sketch size above %d is not supported", SMAXL);
+    if (pc->ell > SMAXL) return fail(ctx, NYS_EINVAL, "prox_wavelet: sketch size above %d is not supported", SMAXL);
     const auto* pv = (const nys_precond_priv*)pc->priv;
-    const int nb = (int)((N + SCH - 1) / SCH);
+    const int ell = pv->ell_eff;
+    cudaStream_t sm = ctx->stream;
     int st;
-    const size_t need = sizeof(SsnState) + 64 + (size_t)(6 * ell + ell * ell) * 8 + (size_t)nb * ell * 16 +
-                        (size_t)nb * ell * ell * 4;
+    if (ell == 0) {      // P = I
+        if ((st = soft_run<T>(ctx, tau, N, s, out))) return st;
+        if (gamma_io) NYS_CK(ctx, cudaMemsetAsync(gamma_io, 0, pc->ell * sizeof(double), sm));
+        if (info) info->iterations = 0, info->converged = 1, info->residual = 0.0;
+        return NYS_OK;
+    }
+    const int nb = (int)((N + SCH - 1) / SCH);
+    const size_t need = sizeof(SsnState) + 64 + (size_t)4 * ell * 8 + (size_t)nb * ell * 16 + (size_t)nb * ell * ell * 4;
     char* w = (char*)scratch(ctx, SLOT_SSN, need, &st);
     if (st) return st;
     SsnState* state = (SsnState*)w;
@@ -419,26 +626,66 @@ int ssn_run(nys_ctx* ctx, const nys_precond* pc, double tau, int64_t N, const T*
     double* gtrial = gamma + ell;
     double* dir = gtrial + ell;
     double* Fcur = dir + ell;
-    double* Jw = Fcur + ell;
-    double* Fp = Jw + (size_t)ell * ell;
+    double* Fp = Fcur + ell;
     double* Sp = Fp + (size_t)nb * ell;
     float* Jp = (float*)(Sp + (size_t)nb * ell);
-    cudaStream_t sm = ctx->stream;
     const double tol = sizeof(T) == 8 ? 1e-12 : 1e-6;
+    const T* U = (const T*)pc->U;
+    const int max_evals = max_newton * 12 + 1;
+    auto report = [&]() -> int {
+        if (!info) return NYS_OK;
+        SsnState h;
+        NYS_CK(ctx, cudaMemcpyAsync(&h, state, sizeof(h), cudaMemcpyDeviceToHost, sm));
+        NYS_CK(ctx, cudaStreamSynchronize(sm));
+        info->iterations = h.newton;
+        info->converged = h.converged;
+        info->residual = h.nF;
+        return NYS_OK;
+    };
+    // ---- one launch: the factor in a cluster's shared memory
+    const int64_t np = (N + SCC - 1) / SCC;
+    const size_t csm = np <= 8192 ? ssn_cluster_smem(ell, (int)np, sizeof(T)) : SIZE_MAX;
+    if (csm <= 220 * 1024) {
+        auto kern = ssn_cluster_kernel<T>;
+        NYS_CK(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        if ((st = smem_optin(ctx, (const void*)kern, csm))) return st;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(SCC, 1, 1);
+        cfg.blockDim = dim3(SCT, 1, 1);
+        cfg.dynamicSmemBytes = csm;
+        cfg.stream = sm;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = SCC;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters >= 1) {
+            NYS_CK(ctx, cudaLaunchKernelEx(&cfg, kern, U, (const double*)pv->sqrtd, s, N, (int)np, ell, tau, tol,
+                                           max_newton, sync_until_done ? max_evals : evals_per_batch, gamma_io, pc->ell,
+                                           out, state));
+            ++ctx->launches;
+            return report();
+        }
+        cudaGetLastError();
+    }
+    // ---- evaluation and step launches
     NYS_CK(ctx, launch_pdl(ssn_init_kernel, 1, 256, 0, sm, state, (const double*)gamma_io, gamma, gtrial, ell));
     NYS_LAUNCH_CK(ctx);
-    const T* U = (const T*)pc->U;
     const size_t esm = (size_t)(2 * SCH + 2 * ell) * sizeof(double) + (size_t)ell * (SCH + 1) * sizeof(float);
     if (int st2 = smem_optin(ctx, (const void*)ssn_eval_kernel<T>, esm)) return st2;
+    const size_t jsm = (size_t)(ell + 1) * (ell + 1) * sizeof(double);
+    if (int st2 = smem_optin(ctx, (const void*)ssn_step_kernel, jsm)) return st2;
     int launched = 0;
-    const int max_evals = max_newton * 12 + 1;
     while (true) {
         for (int e = 0; e < evals_per_batch; ++e) {
             NYS_CK(ctx, launch_pdl(ssn_eval_kernel<T>, nb, 256, esm, sm, U, (const double*)pv->sqrtd, s, N, ell, tau,
                                    (const double*)gtrial, (const SsnState*)state, Fp, Sp, Jp));
             NYS_LAUNCH_CK(ctx);
-            NYS_CK(ctx, launch_pdl(ssn_step_kernel, 1, 1024, 0, sm, nb, ell, tol, max_newton, (const double*)Fp,
-                                   (const double*)Sp, (const float*)Jp, gamma, gtrial, dir, Fcur, Jw, state));
+            NYS_CK(ctx, launch_pdl(ssn_step_kernel, 1, 1024, jsm, sm, nb, ell, tol, max_newton, (const double*)Fp,
+                                   (const double*)Sp, (const float*)Jp, gamma, gtrial, dir, Fcur, state));
             NYS_LAUNCH_CK(ctx);
         }
         launched += evals_per_batch;
@@ -452,16 +699,11 @@ int ssn_run(nys_ctx* ctx, const nys_precond* pc, double tau, int64_t N, const T*
     NYS_CK(ctx, launch_pdl(ssn_final_kernel<T>, grid, 256, 0, sm, U, (const double*)pv->sqrtd, s, N, ell, tau,
                            (const double*)gamma, out));
     NYS_LAUNCH_CK(ctx);
-    if (gamma_io) NYS_CK(ctx, cudaMemcpyAsync(gamma_io, gamma, ell * sizeof(double), cudaMemcpyDeviceToDevice, sm));
-    if (info) {
-        SsnState h;
-        NYS_CK(ctx, cudaMemcpyAsync(&h, state, sizeof(h), cudaMemcpyDeviceToHost, sm));
-        NYS_CK(ctx, cudaStreamSynchronize(sm));
-        info->iterations = h.newton;
-        info->converged = h.converged;
-        info->residual = h.nF;
+    if (gamma_io) {
+        if (ell < pc->ell) NYS_CK(ctx, cudaMemsetAsync(gamma_io + ell, 0, (pc->ell - ell) * sizeof(double), sm));
+        NYS_CK(ctx, cudaMemcpyAsync(gamma_io, gamma, ell * sizeof(double), cudaMemcpyDeviceToDevice, sm));
     }
-    return NYS_OK;
+    return report();
 }
 
 template int ssn_run<float>(nys_ctx*, const nys_precond*, double, int64_t, const float*, float*, double*, int, int,
@@ -469,13 +711,6 @@ template int ssn_run<float>(nys_ctx*, const nys_precond*, double, int64_t, const
 template int ssn_run<double>(nys_ctx*, const nys_precond*, double, int64_t, const double*, double*, double*, int, int,
                              bool, nys_prox_info*);
 
-template <class T>
-int soft_run(nys_ctx* ctx, double tau, int64_t N, const T* s, T* out) {
-    const int grid = (int)std::min<int64_t>((N + 255) / 256, ctx->sm_count * 8);
-    NYS_CK(ctx, launch_pdl(soft_kernel<T>, grid, 256, 0, ctx->stream, s, N, tau, out));
-    NYS_LAUNCH_CK(ctx);
-    return NYS_OK;
-}
 template int soft_run<float>(nys_ctx*, double, int64_t, const float*, float*);
 template int soft_run<double>(nys_ctx*, double, int64_t, const double*, double*);
 

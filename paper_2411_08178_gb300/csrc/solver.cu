@@ -55,6 +55,7 @@ struct nys_solver {
     int64_t glaunch[2] = {0, 0};
     bool gvalid = false;
     uint64_t gen = 0;   // ctx->scratch_gen when the graphs were captured
+    int gell = -1;      // active columns of the preconditioner then
 };
 
 namespace nys {
@@ -293,6 +294,10 @@ int iterate_one(nys_solver* S, int par) {
     return NYS_OK;
 }
 
+int active_columns(const nys_solver* S) {
+    return S->pc && S->pc->priv ? ((const nys_precond_priv*)S->pc->priv)->ell_eff : 0;
+}
+
 template <class T>
 int capture(nys_solver* S) {
     nys_ctx* ctx = S->ctx;
@@ -326,6 +331,7 @@ int capture(nys_solver* S) {
     }
     S->gvalid = true;
     S->gen = ctx->scratch_gen;
+    S->gell = active_columns(S);
     return NYS_OK;
 }
 
@@ -344,6 +350,9 @@ int iterate(nys_solver* S, int n_steps) {
     // the graphs hold the addresses of the context's scratch regions: if any
     // was reallocated since (by another object on this context), capture again
     if (S->gen != ctx->scratch_gen) S->gvalid = false;
+    // and the launches that fit the active columns of the preconditioner, which
+    // the caller may have factored or set up again
+    if (S->gell != active_columns(S)) S->gvalid = false;
     if (!S->gvalid && (st = capture<T>(S))) return st;
     NYS_CK(ctx, cudaEventRecord(S->ev_in, ctx->stream));
     NYS_CK(ctx, cudaStreamWaitEvent(S->gs, S->ev_in, 0));
