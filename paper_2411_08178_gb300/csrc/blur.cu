@@ -19,6 +19,7 @@
 #include "internal.cuh"
 
 #include <cmath>
+#include <type_traits>
 
 namespace nys {
 namespace {
@@ -224,6 +225,198 @@ __global__ void __launch_bounds__(256) sepcorr_kernel(const TI* __restrict__ x, 
     }
 }
 
+// Sixteen consecutive outputs of two lines a and b (the halves of a float2)
+// from a window of 24 values held in registers, eight taps at a time: 16 loads
+// (8 of bf16 pairs) and two tap loads per 128 packed FMAs.  L taps (16-byte
+// aligned, padded to a multiple of 8, the padding not used).  Reads values up
+// to index 8 (L / 8) + 23.
+struct Window16 {
+    float2 w[24], acc[16];
+    const float *sa, *sb;          // float lines
+    const unsigned *pa, *pb;       // lines of bf16 pairs
+    const float4* g;
+    int stride;
+    template <bool PAIRS, int AT>  // eight values from index t on into registers AT ..
+    __device__ __forceinline__ void load(int t) {
+        if constexpr (PAIRS) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const unsigned a = pa[t / 2 + r], b = pb[t / 2 + r];
+                w[(AT + 2 * r) % 24] = make_float2(__uint_as_float(a << 16), __uint_as_float(b << 16));
+                w[(AT + 2 * r + 1) % 24] = make_float2(__uint_as_float(a & 0xffff0000u), __uint_as_float(b & 0xffff0000u));
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < 8; ++r) w[(AT + r) % 24] = make_float2(sa[(t + r) * stride], sb[(t + r) * stride]);
+        }
+    }
+    template <bool PAIRS, int O>   // O: register of the window's first value
+    __device__ __forceinline__ void taps(int t0, int n) {
+        load<PAIRS, O + 16>(t0 + 16);
+        const float4 ga = g[t0 / 4], gb = g[t0 / 4 + 1];
+        const float tap[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
+#pragma unroll
+        for (int dt = 0; dt < 8; ++dt) {
+            if (dt >= n) break;
+            const float2 g2 = make_float2(tap[dt], tap[dt]);
+#pragma unroll
+            for (int r = 0; r < 16; ++r) acc[r] = __ffma2_rn(g2, w[(O + r + dt) % 24], acc[r]);
+        }
+    }
+    template <bool PAIRS>
+    __device__ __forceinline__ void run(int L) {
+#pragma unroll
+        for (int r = 0; r < 16; ++r) acc[r] = make_float2(0.0f, 0.0f);
+        load<PAIRS, 0>(0);
+        load<PAIRS, 8>(8);
+        const int full = L & ~7;
+        int t0 = 0;
+        for (; t0 + 24 <= full; t0 += 24) {
+            taps<PAIRS, 0>(t0, 8);
+            taps<PAIRS, 8>(t0 + 8, 8);
+            taps<PAIRS, 16>(t0 + 16, 8);
+        }
+        if (t0 < full) {
+            taps<PAIRS, 0>(t0, 8);
+            if (t0 + 8 < full) {
+                taps<PAIRS, 8>(t0 + 8, 8);
+                if (L & 7) taps<PAIRS, 16>(full, L & 7);
+            } else if (L & 7) {
+                taps<PAIRS, 8>(full, L & 7);
+            }
+        } else if (L & 7) {
+            taps<PAIRS, 0>(full, L & 7);
+        }
+    }
+};
+
+// y = H_col(gc) H_row(gr) x on many bf16 images (the sketch): a CTA walks down
+// a strip of TX columns, 64 rows at a time, keeping the row pass of the last
+// Lc - 1 rows, so that the row pass is done once per image row (and Lc - 1
+// times more at the top of a strip) instead of 1 + Lc / 64 times; the next 64 input rows arrive by cp.async (pairs of columns: n2, cr
+// and the start of the strip are even) while these are computed.  The same
+// sums in the same order as sepcorr_kernel.  Bound by FP32 FMA issue: 200
+// images of 512 x 512 with 49 taps a side (10.3 GFLOP): 241 us, 43 TFLOP/s (tiles with a 56-row halo: 572 us).
+constexpr int SY = 64;
+template <int TX>
+__host__ __device__ inline int stream_pin(int Lr) { return odd_pitch((TX + 8 * (Lr / 8) + 8) / 2); }   // words
+__host__ __device__ inline int stream_rows(int Lc) { return SY + 8 * (Lc / 8) + 8; }
+template <int TX>
+size_t stream_smem(int Lc, int Lr) {
+    return 4 * ((size_t)round8(Lc) + round8(Lr) + (size_t)2 * SY * stream_pin<TX>(Lr) + (size_t)stream_rows(Lc) * (TX | 1));
+}
+
+template <class TO, int TX>
+__global__ void __launch_bounds__(2 * TX, TX == 128 ? 2 : 3)
+    sepstream_kernel(const __nv_bfloat16* __restrict__ x, TO* __restrict__ y, int n1, int n2, int batch,
+                     const float* __restrict__ taps, int Lc, int Lr, int cc, int cr) {
+    pdl_enter();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* s_tap = reinterpret_cast<float*>(smem_raw);
+    const int Lcp = round8(Lc), Lrp = round8(Lr), pin = stream_pin<TX>(Lr), H = Lc - 1;
+    constexpr int pmid = TX | 1, NT = 2 * TX, NW = NT / 32;
+    constexpr int MQ = (TX / 2 + 32 + 31) / 32;     // staged pairs per lane and row: (TX + Lr) / 2 <= 32 MQ
+    unsigned* s_in = reinterpret_cast<unsigned*>(s_tap + Lcp + Lrp);     // [2][SY][pin] pairs
+    float* s_mid = reinterpret_cast<float*>(s_in + 2 * SY * pin);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int wq = (TX + Lr) / 2, hn = n2 / 2;      // pairs staged per row, pairs of an image row
+    for (int t = threadIdx.x; t < Lcp + Lrp; t += NT) s_tap[t] = taps[t];
+    // this CTA's share of the 64-row chunks of all strips, in order: a part of a
+    // strip at either end, whole strips between
+    const int chunks = (n1 + SY - 1) / SY, strips = (n2 + TX - 1) / TX;
+    const int64_t total = (int64_t)batch * strips * chunks;
+    const int64_t t_beg = total * blockIdx.x / gridDim.x, t_end = total * (blockIdx.x + 1) / gridDim.x;
+    const int above = (H + SY - 1) / SY;            // blocks of input rows above a part
+    for (int64_t t = t_beg; t < t_end;) {
+        const int64_t strip = t / chunks;
+        const int c0 = (int)(t - strip * chunks), nc = (int)min((int64_t)(chunks - c0), t_end - t);
+        t += nc;
+        const int b_img = (int)(strip / strips), j0 = (int)(strip - (int64_t)b_img * strips) * TX;
+        const int ib = c0 * SY, ie = min(n1, (c0 + nc) * SY);
+        const unsigned* xb = reinterpret_cast<const unsigned*>(x + (size_t)b_img * n1 * n2);
+        TO* yb = y + (size_t)b_img * n1 * n2;
+        int gj[MQ];
+#pragma unroll
+        for (int q = 0; q < MQ; ++q) gj[q] = pmod((j0 - cr) / 2 + lane + 32 * q, hn);
+        auto stage = [&](int r0, int buf, int rows) {
+            const unsigned d0 = (unsigned)__cvta_generic_to_shared(s_in + buf * SY * pin + lane);
+            for (int r = warp; r < rows; r += NW) {
+                int gi = r0 + r;
+                gi = gi < 0 ? gi + n1 : (gi >= n1 ? gi - n1 : gi);
+                if (gi < 0 || gi >= n1) gi = pmod(gi, n1);
+                const unsigned* xr = xb + (size_t)gi * hn;
+                const unsigned d = d0 + 4 * r * pin;
+#pragma unroll
+                for (int q = 0; q < MQ; ++q)
+                    if (lane + 32 * q < wq)
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + 128 * q), "l"(xr + gj[q]));
+            }
+            asm volatile("cp.async.commit_group;");
+        };
+        // blocks of input rows in order: those above (H rows), then 64 for every
+        // 64 output rows
+        const int blocks = above + nc;
+        auto first_row = [&](int b) { return ib - cc + (b < above ? b * SY : H + (b - above) * SY); };
+        __syncthreads();                            // the previous part is done with the buffers
+        stage(first_row(0), 0, above ? min(SY, H) : SY);
+        for (int b = 0; b < blocks; ++b) {
+            asm volatile("cp.async.wait_group 0;");
+            __syncthreads();
+            if (b + 1 < blocks) stage(first_row(b + 1), (b + 1) & 1, b + 1 < above ? min(SY, H - (b + 1) * SY) : SY);
+            {
+                // row pass of rows r and r + 32 of the block
+                const int rows = b < above ? min(SY, H - b * SY) : SY, at = b < above ? b * SY : H;
+                Window16 w;
+                w.pa = s_in + (b & 1) * SY * pin + lane * pin + 8 * warp;
+                w.pb = w.pa + 32 * pin;
+                w.g = reinterpret_cast<const float4*>(s_tap + Lcp);
+                w.run<true>(Lr);
+                float* m = s_mid + (at + lane) * pmid + 16 * warp;
+                if (lane < rows)
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) m[k] = w.acc[k].x;
+                if (lane + 32 < rows)
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) m[32 * pmid + k] = w.acc[k].y;
+            }
+            __syncthreads();
+            if (b < above) continue;
+            const int i0 = ib + (b - above) * SY;
+            // column pass: columns c and c + TX / 2 together
+            const int c = threadIdx.x % (TX / 2), sy = threadIdx.x / (TX / 2);
+            Window16 w;
+            w.sa = s_mid + 16 * sy * pmid + c;
+            w.sb = w.sa + TX / 2;
+            w.stride = pmid;
+            w.g = reinterpret_cast<const float4*>(s_tap);
+            w.run<false>(Lc);
+            const int left = ie - (i0 + 16 * sy);   // output rows of this thread
+            TO* yo = yb + (size_t)(i0 + 16 * sy) * n2 + j0 + c;
+            const bool ca = j0 + c < n2, cb = j0 + c + TX / 2 < n2;
+            if (left >= 16 && cb) {
+#pragma unroll
+                for (int k = 0; k < 16; ++k, yo += n2) {
+                    stf(yo, w.acc[k].x);
+                    stf(yo + TX / 2, w.acc[k].y);
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 16; ++k, yo += n2) {
+                    if (k < left && ca) stf(yo, w.acc[k].x);
+                    if (k < left && cb) stf(yo + TX / 2, w.acc[k].y);
+                }
+            }
+            // the last H rows move to the top, 64 rows at a time
+            if (b + 1 < blocks)
+                for (int d = 0; d < H; d += SY) {
+                    __syncthreads();
+                    float* m = s_mid + (d + threadIdx.x / TX) * pmid + threadIdx.x % TX;
+                    for (int r = threadIdx.x / TX; r < min(SY, H - d); r += 2, m += 2 * pmid) *m = m[SY * pmid];
+                }
+        }
+    }
+}
+
 // General (non-separable) periodic correlation with a kh x kw kernel.
 // taps: kh rows of kwp entries (zero padded).
 template <class TI, class TO, class TC, int TY, int TX>
@@ -244,6 +437,27 @@ __global__ void __launch_bounds__(256) corr2d_kernel(const TI* __restrict__ x, T
     stage_tile<TI, TC>(xb, n1, n2, i0 - ch, j0 - cw, rows, wcols, s_in, pin);
     __syncthreads();
     TO* yb = y + img;
+    if constexpr (PairWindow<TC>::on) {
+        // float32: rows r and r + TY / 2 together
+        constexpr int HY = TY / 2;
+        for (int idx = threadIdx.x; idx < HY * (TX / RB); idx += blockDim.x) {
+            const int r = idx % HY, sx = idx / HY;
+            float2 acc[RB];
+#pragma unroll
+            for (int k = 0; k < RB; ++k) acc[k] = make_float2(0.0f, 0.0f);
+            for (int a = 0; a < kh; ++a)
+                window8x2(s_in + (r + a) * pin + sx * RB, s_in + (r + HY + a) * pin + sx * RB, 1, s_tap + a * kwp, kwp,
+                          acc);
+#pragma unroll
+            for (int k = 0; k < RB; ++k) {
+                const int gj = j0 + sx * RB + k;
+                if (gj >= n2) continue;
+                if (i0 + r < n1) stf(yb + (size_t)(i0 + r) * n2 + gj, acc[k].x);
+                if (i0 + r + HY < n1) stf(yb + (size_t)(i0 + r + HY) * n2 + gj, acc[k].y);
+            }
+        }
+        return;
+    }
     for (int idx = threadIdx.x; idx < TY * (TX / RB); idx += blockDim.x) {
         const int r = idx % TY, sx = idx / TY;
         TC acc[RB];
@@ -331,7 +545,6 @@ int launch_sep(nys_op* op, const void* x, void* y, int batch, const void* taps, 
                int cr) {
     const size_t sm = sep_smem<TC>(T, T, Lcp, Lrp);
     auto k = sepcorr_kernel<TI, TO, TC, T, T>;
-    if (sm > 227 * 1024) return fail(op->ctx, NYS_EINVAL, "blur kernel too wide for the shared-memory tile");
     if (int st = smem_optin(op->ctx, (const void*)k, sm)) return st;
     for (int b0 = 0; b0 < batch; b0 += 65535) {     // images in grid.z
         dim3 grid((op->n2 + T - 1) / T, (op->n1 + T - 1) / T, std::min(65535, batch - b0));
@@ -342,12 +555,26 @@ int launch_sep(nys_op* op, const void* x, void* y, int batch, const void* taps, 
     return NYS_OK;
 }
 
+template <class TO, int TX>
+int launch_stream(nys_op* op, const __nv_bfloat16* x, TO* y, int batch, const void* taps, int Lc, int Lr, int cc,
+                  int cr) {
+    auto k = sepstream_kernel<TO, TX>;
+    const size_t sm = stream_smem<TX>(Lc, Lr);
+    if (int st = smem_optin(op->ctx, (const void*)k, sm)) return st;
+    // persistent: the CTAs that stay resident share the chunks evenly
+    const int64_t chunks = (int64_t)((op->n1 + SY - 1) / SY) * ((op->n2 + TX - 1) / TX) * batch;
+    const int grid = (int)std::min<int64_t>(chunks, (int64_t)op->ctx->sm_count * (TX == 128 ? 2 : 3));
+    NYS_CK(op->ctx, launch_pdl(k, grid, 2 * TX, sm, op->ctx->stream, x, y, op->n1, op->n2, batch, (const float*)taps, Lc,
+                               Lr, cc, cr));
+    NYS_LAUNCH_CK(op->ctx);
+    return NYS_OK;
+}
+
 template <class TI, class TO, class TC, int T>
 int launch_c2d(nys_op* op, const void* x, void* y, int batch, const void* taps) {
     const int kwp = round8(op->kw);
     const size_t sm = c2d_smem<TC>(T, T, op->kh, kwp);
     auto k = corr2d_kernel<TI, TO, TC, T, T>;
-    if (sm > 227 * 1024) return fail(op->ctx, NYS_EINVAL, "blur kernel too large for the shared-memory tile");
     if (int st = smem_optin(op->ctx, (const void*)k, sm)) return st;
     for (int b0 = 0; b0 < batch; b0 += 65535) {     // images in grid.z
         dim3 grid((op->n2 + T - 1) / T, (op->n1 + T - 1) / T, std::min(65535, batch - b0));
@@ -359,30 +586,97 @@ int launch_c2d(nys_op* op, const void* x, void* y, int batch, const void* taps) 
     return NYS_OK;
 }
 
-template <class TI, class TO, class TC, int T>
-int blur_typed_t(nys_op* op, int which, const void* x, void* y, int batch) {
+template <class TC>
+constexpr int largest_tile() { return sizeof(TC) == 8 ? 32 : 64; }
+
+// Tile side (largest, a half or a quarter of it), the one whose slowest SM has
+// the least work: whole tiles to an SM times the FMAs of a tile with its halo
+// (work(T)) and 66 thousand more for staging it and its barriers (float32
+// normal operators of 13 to 49 taps on 1 to 400 images of 64 to 512 pixels a
+// side: 0.6 us a tile and 9 us per million FMAs fit tiles of 16, 32 and 64
+// within 15%).  One 512 x 512 image in float32 takes 32 (64 leaves more than half
+// of the SMs idle), a 64 x 64 one in float64 takes 8 (64 CTAs instead of 4:
+// 21 to 16 us per normal).
+template <class Work>
+int pick_tile(const nys_op* op, int batch, int largest, Work&& work) {
+    int best = largest;
+    double best_cost = 1e300;
+    for (int T = largest; T >= largest / 4; T /= 2) {
+        const int64_t tiles = (int64_t)((op->n1 + T - 1) / T) * ((op->n2 + T - 1) / T) * batch;
+        const double cost = (double)((tiles + op->ctx->sm_count - 1) / op->ctx->sm_count) * (work(T) + 66e3);
+        if (cost < best_cost) best = T, best_cost = cost;
+    }
+    return best;
+}
+
+template <class TI, class TO, class TC>
+int sep_typed(nys_op* op, const void* x, void* y, int batch, const void* taps, int Lc, int Lr, int cc, int cr) {
+    const int Lcp = round8(Lc), Lrp = round8(Lr), SM = op->ctx->sm_count;
+    int T = sizeof(TC) == 8 ? 0 : op->blur_tile;      // 0: by size
+    // the largest kernel taken: the one that fits the largest tile (or the tuned one)
+    if (sep_smem<TC>(T ? T : largest_tile<TC>(), T ? T : largest_tile<TC>(), Lcp, Lrp) > 227 * 1024)
+        return fail(op->ctx, NYS_EINVAL, "blur kernel too wide for the shared-memory tile");
+    if constexpr (std::is_same<TI, __nv_bfloat16>::value) {
+        // Strips with the row pass carried down, TX columns wide with the least
+        // padding, when there is a chunk for every other SM; few taps on small
+        // images stay with the tiles (13 taps a side at 128 x 128: 45 against
+        // 43 us for 400 images; 49 taps at 64 x 64: 22.6 against 26.6 us)
+        const int chunks = (op->n1 + SY - 1) / SY;
+        const int TX = op->n2 > 64 && (op->n2 + 127) / 128 * 128 - op->n2 < 64 ? 128 : 64;
+        const size_t sm = TX == 128 ? stream_smem<128>(Lc, Lr) : stream_smem<64>(Lc, Lr);
+        const int64_t strips = (int64_t)((op->n2 + TX - 1) / TX) * batch;
+        if (sm <= (TX == 128 ? 113 : 75) * 1024 && Lr <= 64 && op->n2 % 2 == 0 && cr % 2 == 0 &&
+            ((uintptr_t)x & 3) == 0 && 2 * strips * chunks >= SM && (Lc + Lr >= 40 || op->n1 >= 190)) {
+            const auto* xb = (const __nv_bfloat16*)x;
+            return TX == 128 ? launch_stream<TO, 128>(op, xb, (TO*)y, batch, taps, Lc, Lr, cc, cr)
+                             : launch_stream<TO, 64>(op, xb, (TO*)y, batch, taps, Lc, Lr, cc, cr);
+        }
+    }
+    auto work = [&](int t) { return (double)(t + Lcp) * t * Lrp + (double)t * t * Lcp; };
+    if (!T) T = pick_tile(op, batch, largest_tile<TC>(), work);
+    if constexpr (sizeof(TC) == 8) {
+        if (T == 8) return launch_sep<TI, TO, TC, 8>(op, x, y, batch, taps, Lcp, Lrp, cc, cr);
+    } else {
+        if (T == 64) return launch_sep<TI, TO, TC, 64>(op, x, y, batch, taps, Lcp, Lrp, cc, cr);
+    }
+    if (T == 16) return launch_sep<TI, TO, TC, 16>(op, x, y, batch, taps, Lcp, Lrp, cc, cr);
+    return launch_sep<TI, TO, TC, 32>(op, x, y, batch, taps, Lcp, Lrp, cc, cr);
+}
+
+template <class TI, class TO, class TC>
+int c2d_typed(nys_op* op, const void* x, void* y, int batch, const void* taps) {
+    int T = sizeof(TC) == 8 ? 0 : op->blur_tile;      // 0: by size
+    const int kwp = round8(op->kw);
+    auto work = [&](int t) { return (double)t * t * op->kh * kwp + 4.0 * (t + op->kh) * (t + kwp); };
+    if (c2d_smem<TC>(T ? T : largest_tile<TC>(), T ? T : largest_tile<TC>(), op->kh, kwp) > 227 * 1024)
+        return fail(op->ctx, NYS_EINVAL, "blur kernel too large for the shared-memory tile");
+    if (!T) T = pick_tile(op, batch, largest_tile<TC>(), work);
+    if constexpr (sizeof(TC) == 8) {
+        if (T == 8) return launch_c2d<TI, TO, TC, 8>(op, x, y, batch, taps);
+    } else {
+        if (T == 64) return launch_c2d<TI, TO, TC, 64>(op, x, y, batch, taps);
+    }
+    if (T == 16) return launch_c2d<TI, TO, TC, 16>(op, x, y, batch, taps);
+    return launch_c2d<TI, TO, TC, 32>(op, x, y, batch, taps);
+}
+
+template <class TI, class TO, class TC>
+int blur_typed(nys_op* op, int which, const void* x, void* y, int batch) {
     if (op->separable) {
         if (which == 2)
-            return launch_sep<TI, TO, TC, T>(op, x, y, batch, op->taps_nrm, op->Lc_n, op->Lr_n, op->cc_n, op->cr_n);
-        return launch_sep<TI, TO, TC, T>(op, x, y, batch, which == 0 ? op->taps_fwd : op->taps_adj, op->Lc_f,
-                                         op->Lr_f, op->cc_f, op->cr_f);
+            return sep_typed<TI, TO, TC>(op, x, y, batch, op->taps_nrm, op->Lc_n, op->Lr_n, op->cc_n, op->cr_n);
+        return sep_typed<TI, TO, TC>(op, x, y, batch, which == 0 ? op->taps_fwd : op->taps_adj, op->Lc_f, op->Lr_f,
+                                     op->cc_f, op->cr_f);
     }
-    if (which != 2) return launch_c2d<TI, TO, TC, T>(op, x, y, batch, which == 0 ? op->taps_fwd : op->taps_adj);
+    if (which != 2) return c2d_typed<TI, TO, TC>(op, x, y, batch, which == 0 ? op->taps_fwd : op->taps_adj);
     // non-separable normal: H^T (H x) through the intermediate buffer, in chunks
     for (int b0 = 0; b0 < batch; b0 += op->chunk) {
         const int nb = std::min(op->chunk, batch - b0);
         const size_t in_off = (size_t)b0 * op->N * sizeof(TI), out_off = (size_t)b0 * op->N * sizeof(TO);
-        if (int st = launch_c2d<TI, TC, TC, T>(op, (const char*)x + in_off, op->inter, nb, op->taps_fwd)) return st;
-        if (int st = launch_c2d<TC, TO, TC, T>(op, op->inter, (char*)y + out_off, nb, op->taps_adj)) return st;
+        if (int st = c2d_typed<TI, TC, TC>(op, (const char*)x + in_off, op->inter, nb, op->taps_fwd)) return st;
+        if (int st = c2d_typed<TC, TO, TC>(op, op->inter, (char*)y + out_off, nb, op->taps_adj)) return st;
     }
     return NYS_OK;
-}
-
-// output tile: 32 x 32 in float64; 32 or 64 in float32 (nys_op_autotune picks)
-template <class TI, class TO, class TC>
-int blur_typed(nys_op* op, int which, const void* x, void* y, int batch) {
-    if (sizeof(TC) == 8 || op->blur_tile == 32) return blur_typed_t<TI, TO, TC, 32>(op, which, x, y, batch);
-    return blur_typed_t<TI, TO, TC, 64>(op, which, x, y, batch);
 }
 
 template <class TI, class TO, class TC>
@@ -476,23 +770,25 @@ int blur_setup(nys_op* op) {
         if ((st = up(h, &op->taps_fwd))) return st;
     } else if (op->separable) {
         // forward: [u | v], adjoint: [flip u | flip v]; each padded to a multiple of 8
-        op->Lc_f = round8(kh);
-        op->Lr_f = round8(kw);
+        op->Lc_f = kh;
+        op->Lr_f = kw;
+        const int Lcf = round8(kh), Lrf = round8(kw);
         op->cc_f = (kh - 1) / 2;
         op->cr_f = (kw - 1) / 2;
-        std::vector<double> f(op->Lc_f + op->Lr_f, 0.0), g(op->Lc_f + op->Lr_f, 0.0);
+        std::vector<double> f(Lcf + Lrf, 0.0), g(Lcf + Lrf, 0.0);
         for (int a = 0; a < kh; ++a) f[a] = u[a], g[a] = u[kh - 1 - a];
-        for (int b = 0; b < kw; ++b) f[op->Lc_f + b] = v[b], g[op->Lc_f + b] = v[kw - 1 - b];
+        for (int b = 0; b < kw; ++b) f[Lcf + b] = v[b], g[Lcf + b] = v[kw - 1 - b];
         if ((st = up(f, &op->taps_fwd))) return st;
         if ((st = up(g, &op->taps_adj))) return st;
         std::vector<double> gu = autocorr(u), gv = autocorr(v);
-        op->Lc_n = round8((int)gu.size());
-        op->Lr_n = round8((int)gv.size());
+        op->Lc_n = (int)gu.size();
+        op->Lr_n = (int)gv.size();
+        const int Lcn = round8(op->Lc_n), Lrn = round8(op->Lr_n);
         op->cc_n = kh - 1;
         op->cr_n = kw - 1;
-        std::vector<double> n(op->Lc_n + op->Lr_n, 0.0);
+        std::vector<double> n(Lcn + Lrn, 0.0);
         for (size_t a = 0; a < gu.size(); ++a) n[a] = gu[a];
-        for (size_t b = 0; b < gv.size(); ++b) n[op->Lc_n + b] = gv[b];
+        for (size_t b = 0; b < gv.size(); ++b) n[Lcn + b] = gv[b];
         if ((st = up(n, &op->taps_nrm))) return st;
     } else {
         const int kwp = round8(kw);

@@ -128,7 +128,7 @@ struct nys_op {
     double src_dist = 0.0, det_dist = 0.0, det_spacing = 1.0;   // fan beam
     nys_fan fan;
     int radon_adj_ak = 16;            // radon adjoint: angles per round, 4, 8 or 16 (nys_op_autotune)
-    int blur_tile = 64;               // blur: output tile side, 32 or 64 (float32; chosen by nys_op_autotune)
+    int blur_tile = 0;                // blur, float32: output tile side, 32 or 64 (nys_op_autotune), 0: by size
     // intermediate buffer for two-pass normals (M per image, `chunk` images)
     void* inter = nullptr;
     int chunk = 0;
