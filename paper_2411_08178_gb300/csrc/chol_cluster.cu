@@ -1,6 +1,6 @@
-// Cholesky factorisation of the small float64 matrices of Algorithm 1 (the
-// shifted core, steps 4-5) and of the preconditioner set-up (I + Ubar^T
-// Ubar) on a cluster of 16 CTAs.
+// Retries of Algorithm 1's shifted Cholesky (steps 4-5) on a cluster of 16 CTAs:
+// the blocked factorisation (chol_blocked.cu) makes the first attempt; when its
+// shift was too small, this kernel goes through the shifts in one launch.
 //
 // GB300's float64 pipe issues about two FMAs per clock per SM, so the n^3/6
 // FMAs of a Cholesky of n = 400 take milliseconds on one SM; spread over the
@@ -15,11 +15,10 @@
 // every CTA before the barrier that follows it, so that all leave or retry
 // together; there are no spin waits.
 //
-//   mode 0  A = src (n x n, row-major, ld), status in info[slot]
-//   mode 1  A = sym(Omega^T Y) + v Omega^T Omega from the Gram G2 of
-//           [Omega | Y] (ld 2n), v = eps sqrt(trace Omega^T Omega), times 10
-//           after each failure, at most max_retries times; info[0] = status,
-//           info[1] = v, info[2] = retries (as the one-CTA kernel)
+//   A = sym(Omega^T Y) + v Omega^T Omega from the Gram G2 of [Omega | Y] (ld
+//   2n), v = eps sqrt(trace Omega^T Omega), times 10 after each failure, at
+//   most max_retries times; info[0] = status, info[1] = v, info[2] = retries
+//   (as the one-CTA kernel).  Returns at once unless info[0] is 1.
 // Output: L (n x n, row-major, ld n), lower triangular with zeros above.
 #include "internal.cuh"
 #include "chol_panel.cuh"
@@ -35,8 +34,9 @@ constexpr int CC = 16;           // CTAs per cluster
 constexpr int CH_THREADS = 512;
 
 __global__ void __launch_bounds__(CH_THREADS, 1)
-    chol_cluster_kernel(const double* __restrict__ src, int ld, int n, int mode, double eps, int max_retries,
-                        double* __restrict__ L, double* __restrict__ info, int slot, int b) {
+    chol_cluster_kernel(const double* __restrict__ src, int n, double eps, int max_retries, double* __restrict__ L,
+                        double* __restrict__ info, int b) {
+    if (info[0] != 1.0) return;                          // the same in every CTA: written at the very end
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
     const int npad = 2 * CC * b;
@@ -48,16 +48,13 @@ __global__ void __launch_bounds__(CH_THREADS, 1)
     const int blk[2] = {rank, 2 * CC - 1 - rank};
     auto col = [&](int s, int c) { return own + ((size_t)s * b + c) * npad; };
 
-    double v = 0.0;
-    if (mode == 1) {
-        double tr = 0.0;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) tr += src[(size_t)i * ld + i];
-        tr = block_sum(tr, sh);
-        v = eps * sqrt(tr);
-    }
+    double tr = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) tr += src[(size_t)i * 2 * n + i];
+    tr = block_sum(tr, sh);
+    double v = eps * sqrt(tr);
     int retries = 0;
     bool ok = false;
-    for (int attempt = 0; attempt <= (mode == 1 ? max_retries : 0); ++attempt) {
+    for (int attempt = 0; attempt <= max_retries; ++attempt) {
         // load: R's column j starts as A's row j (A symmetric), pad with the identity
         for (int s = 0; s < 2; ++s)
             for (int t = threadIdx.x; t < b * npad; t += blockDim.x) {
@@ -65,13 +62,9 @@ __global__ void __launch_bounds__(CH_THREADS, 1)
                 const int j = blk[s] * b + c;
                 double a;
                 if (i < n && j < n) {
-                    if (mode == 1) {
-                        const int l2 = 2 * n;
-                        const double oy = 0.5 * (src[(size_t)j * l2 + n + i] + src[(size_t)i * l2 + n + j]);
-                        a = oy + v * src[(size_t)j * l2 + i];
-                    } else {
-                        a = src[(size_t)j * ld + i];
-                    }
+                    const int l2 = 2 * n;
+                    const double oy = 0.5 * (src[(size_t)j * l2 + n + i] + src[(size_t)i * l2 + n + j]);
+                    a = oy + v * src[(size_t)j * l2 + i];
                 } else {
                     a = (i == j) ? 1.0 : 0.0;
                 }
@@ -148,7 +141,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1)
             break;
         }
         retries = attempt;
-        if (mode == 1) v *= 10.0;
+        v *= 10.0;
         // no CTA reloads its columns before every CTA has stopped reading them
         cluster.sync();
     }
@@ -161,13 +154,9 @@ __global__ void __launch_bounds__(CH_THREADS, 1)
             }
     }
     if (rank == 0 && threadIdx.x == 0) {
-        if (mode == 1) {
-            info[0] = ok ? 0.0 : 1.0;
-            info[1] = ok ? v : v / 10.0;
-            info[2] = (double)retries;
-        } else {
-            info[slot] = ok ? 0.0 : 1.0;
-        }
+        info[0] = ok ? 0.0 : 1.0;
+        info[1] = ok ? v : v / 10.0;
+        info[2] = (double)retries;
     }
     // no CTA leaves while another may still read its shared memory
     cluster.sync();
@@ -175,10 +164,9 @@ __global__ void __launch_bounds__(CH_THREADS, 1)
 
 }  // namespace
 
-// L = chol(A) by the cluster kernel (see above); NYS_EINVAL (nothing
-// launched) when n is outside [48, 512] or the cluster cannot be placed.
-int chol_cluster(nys_ctx* ctx, const double* src, int ld, int n, int mode, double eps, int max_retries, double* L,
-                 double* info, int slot) {
+// The retries by the cluster kernel (see above); NYS_EINVAL (nothing launched)
+// when n is outside [48, 512] or the cluster cannot be placed.
+int chol_cluster(nys_ctx* ctx, const double* src, int n, double eps, int max_retries, double* L, double* info) {
     if (n < 48 || n > 512) return NYS_EINVAL;
     const int b = (n + 2 * CC - 1) / (2 * CC);
     const int npad = 2 * CC * b;
@@ -204,7 +192,7 @@ int chol_cluster(nys_ctx* ctx, const double* src, int ld, int n, int mode, doubl
         cudaGetLastError();
         return NYS_EINVAL;
     }
-    NYS_CK(ctx, cudaLaunchKernelEx(&cfg, k, src, ld, n, mode, eps, max_retries, L, info, slot, b));
+    NYS_CK(ctx, cudaLaunchKernelEx(&cfg, k, src, n, eps, max_retries, L, info, b));
     ++ctx->launches;
     return NYS_OK;
 }

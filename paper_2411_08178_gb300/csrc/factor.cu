@@ -25,20 +25,19 @@
 
 namespace nys {
 
+enum : int { TRI_A = 1, TRI_B = 2, GEMM_SYM = 4 };   // small.cu
 int launch_small_gemm(nys_ctx* ctx, const double* A, int ta, const double* B, int tb, int m, int n, int k,
-                      const double* colscale, double* C);
+                      const double* colscale, double* C, int flags);
 int sym_eig(nys_ctx* ctx, const double* G, int ell, bool use_f32, const double* info, void* work, double* Vout,
             double* S_hat, double* scale, int* sweeps_dev);
 __global__ void shift_chol_kernel(const double* __restrict__ G2, int ell, double eps, int max_retries,
                                   double* __restrict__ C, double* __restrict__ info);
 __global__ void form_H_kernel(const double* __restrict__ G2, int ell, const double* __restrict__ info,
                               double* __restrict__ H);
-__global__ void tri_inv_kernel(const double* __restrict__ C, double* __restrict__ X, int n);
 __global__ void weights_kernel(const double* __restrict__ S_hat, int ell, double mu, int sqrt_shift,
                                double* __restrict__ d, double* __restrict__ sqd, float* __restrict__ d32);
 __global__ void form_A_kernel(const double* __restrict__ K, int ldk, const double* __restrict__ sqd, int eff,
                               double* __restrict__ A);
-__global__ void chol_kernel(double* __restrict__ A, int n, double* __restrict__ info);
 __global__ void form_M_kernel(const double* __restrict__ Ainv, const double* __restrict__ sqd, int ell, int eff,
                               double* __restrict__ M, float* __restrict__ M32);
 
@@ -422,17 +421,10 @@ int precond_setup_impl(nys_ctx* ctx, nys_precond* pc, double mu, int sqrt_shift)
         // (I + Ubar^T Ubar)^{-1} on the active block only (Ubar's other columns are 0)
         form_A_kernel<<<64, 256, 0, s>>>(pv->K, ell, pv->sqrtd, eff, A);
         NYS_LAUNCH_CK(ctx);
-        st = chol_cluster(ctx, A, eff, eff, 0, 0.0, 0, A, info, 3);
-        if (st == NYS_EINVAL) {
-            chol_kernel<<<1, 1024, 0, s>>>(A, eff, info);
-            NYS_LAUNCH_CK(ctx);
-        } else if (st) {
-            return st;
-        }
-        tri_inv_kernel<<<eff, 32, eff * sizeof(double), s>>>(A, Li, eff);
-        NYS_LAUNCH_CK(ctx);
+        if ((st = chol_blocked(ctx, A, eff, Ai, info, 3))) return st;
+        if ((st = tri_inv(ctx, Ai, Li, eff))) return st;
         // (I + Ubar^T Ubar)^{-1} = L^{-T} L^{-1}
-        if ((st = launch_small_gemm(ctx, Li, 1, Li, 0, eff, eff, eff, nullptr, Ai))) return st;
+        if ((st = launch_small_gemm(ctx, Li, 1, Li, 0, eff, eff, eff, nullptr, Ai, TRI_A | TRI_B | GEMM_SYM))) return st;
     }
     form_M_kernel<<<64, 256, 0, s>>>(Ai, pv->sqrtd, ell, eff, pv->M64, pv->M32);
     NYS_LAUNCH_CK(ctx);
@@ -583,8 +575,11 @@ static int factor_small(nys_ctx* ctx, const double* G2, int ell, double eps, boo
     void* ework = (void*)(info + 32);     // eigen work (2 n^2 T + n doubles)
     cudaStream_t s = ctx->stream;
     NYS_CK(ctx, cudaMemsetAsync(info, 0, 16 * sizeof(double), s));
-    // shifted Cholesky (steps 4-5): on a 16-SM cluster where it fits, else one CTA
-    st = chol_cluster(ctx, G2, 2 * ell, ell, 1, eps, 8, C, info, 0);
+    // shifted Cholesky (steps 4-5); the retries with larger shifts, which return
+    // at once when the first attempt succeeded, on a 16-SM cluster where it
+    // fits, else one CTA
+    if ((st = chol_core(ctx, G2, ell, eps, T1, C, info))) return st;
+    st = chol_cluster(ctx, G2, ell, eps, 8, C, info);
     if (st == NYS_EINVAL) {
         shift_chol_kernel<<<1, 1024, 0, s>>>(G2, ell, eps, 8, C, info);
         NYS_LAUNCH_CK(ctx);
@@ -593,13 +588,12 @@ static int factor_small(nys_ctx* ctx, const double* G2, int ell, double eps, boo
     }
     form_H_kernel<<<64, 256, 0, s>>>(G2, ell, info, H);
     NYS_LAUNCH_CK(ctx);
-    tri_inv_kernel<<<ell, 32, ell * sizeof(double), s>>>(C, Ci, ell);
-    NYS_LAUNCH_CK(ctx);
-    if ((st = launch_small_gemm(ctx, Ci, 0, H, 0, ell, ell, ell, nullptr, T1))) return st;
-    if ((st = launch_small_gemm(ctx, T1, 0, Ci, 1, ell, ell, ell, nullptr, Gm))) return st;
+    if ((st = tri_inv(ctx, C, Ci, ell))) return st;
+    if ((st = launch_small_gemm(ctx, Ci, 0, H, 0, ell, ell, ell, nullptr, T1, TRI_A))) return st;
+    if ((st = launch_small_gemm(ctx, T1, 0, Ci, 1, ell, ell, ell, nullptr, Gm, TRI_B | GEMM_SYM))) return st;
     if ((st = sym_eig(ctx, Gm, ell, eig_f32, info, ework, Vs, S_hat, scale, sweeps))) return st;
     // W = C^{-T} V S^{-1}  (into T1)
-    if ((st = launch_small_gemm(ctx, Ci, 1, Vs, 0, ell, ell, ell, scale, T1))) return st;
+    if ((st = launch_small_gemm(ctx, Ci, 1, Vs, 0, ell, ell, ell, scale, T1, TRI_A))) return st;
     *W_out = T1;
     *info_out = info;
     return NYS_OK;

@@ -340,13 +340,17 @@ int gemm_tall(nys_ctx* ctx, int in_dt, const void* A, const void* A2, const doub
 int jacobi_cluster(nys_ctx* ctx, const double* G, int ell, int max_sweeps, float* V, int ldv, float* Rsave,
                    int* sweeps, int* status);
 
-// float64 Cholesky L (n x n, lower, row-major) on a 16-CTA cluster
-// (chol_cluster.cu): mode 0 of src (ld), status in info[slot]; mode 1 of
-// sym(Omega^T Y) + v Omega^T Omega from the Gram src = G2 with the shift and
-// its retries in info[0..2].  NYS_EINVAL (nothing launched) when n is outside
-// [48, 512] or the cluster cannot be placed.
-int chol_cluster(nys_ctx* ctx, const double* src, int ld, int n, int mode, double eps, int max_retries, double* L,
-                 double* info, int slot);
+// float64 Cholesky factors and the triangular inverse (chol_blocked.cu): L =
+// chol(A) with A overwritten and status in info[slot]; the shifted core
+// sym(Omega^T Y) + v Omega^T Omega of the Gram G2 = [Omega | Y]^T [Omega | Y],
+// its first shift only, info[0..2] = status, v, 0; X = L^{-1}
+int chol_blocked(nys_ctx* ctx, double* A, int n, double* L, double* info, int slot);
+int chol_core(nys_ctx* ctx, const double* G2, int n, double eps, double* work, double* L, double* info);
+int tri_inv(nys_ctx* ctx, const double* L, double* X, int n);
+// the shifted core with its retries when info[0] is 1 (chol_cluster.cu: a
+// 16-CTA cluster); NYS_EINVAL (nothing launched) when n is outside [48, 512] or
+// the cluster cannot be placed
+int chol_cluster(nys_ctx* ctx, const double* src, int n, double eps, int max_retries, double* L, double* info);
 
 // Omega for Algorithm 1 step 1: total i.i.d. N(0,1) entries (factor.cu)
 int omega_fill(nys_ctx* ctx, int store_dt, void* Omega, int64_t total, uint64_t seed, int64_t first = 0);

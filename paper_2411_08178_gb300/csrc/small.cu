@@ -3,10 +3,10 @@
 //
 //   shift_chol   v = eps sqrt(trace(Omega^T Omega)) (= eps ||Omega||_F, step 3);
 //                C = chol(sym(Omega^T Y) + v Omega^T Omega) (= chol(Omega^T Y_v),
-//                step 5) with v <- 10 v retries; one CTA, float64.
+//                step 5) with v <- 10 v retries; one CTA, float64, where the
+//                first shift failed (chol_blocked.cu) and no cluster fits
 //   form_H       H = Y_v^T Y_v = Y^T Y + v (Omega^T Y + Y^T Omega) + v^2 Omega^T Omega
-//   tri_inv      C^{-1} for lower-triangular C, one warp per column
-//   small_gemm   C = op(A) op(B) diag(colscale), float64
+//   small_gemm   C = op(A) op(B) diag(colscale), float64, triangular operands
 //   jacobi       cyclic Jacobi with the round-robin parallel ordering
 //                (Golub & Van Loan, Sec. 8.5: sym.schur2 rotations, every
 //                index in exactly one pair per round), one CTA, working type T
@@ -30,6 +30,7 @@ namespace nys {
 __global__ void __launch_bounds__(1024) shift_chol_kernel(const double* __restrict__ G2, int ell, double eps,
                                                           int max_retries, double* __restrict__ C,
                                                           double* __restrict__ info) {
+    if (info[0] != 1.0) return;
     __shared__ int flag;
     __shared__ double sh[32];
     const int ld = 2 * ell;
@@ -71,46 +72,55 @@ __global__ void form_H_kernel(const double* __restrict__ G2, int ell, const doub
     }
 }
 
-// X = C^{-1} for lower-triangular C (n x n).  Block j (one warp) solves
-// C x = e_j by forward substitution, with x in shared memory (the dependent
-// chain of the substitution stays on chip) and rows of C read coalesced;
-// column j of X is written at the end.  Dynamic shared memory: n doubles.
-__global__ void tri_inv_kernel(const double* __restrict__ C, double* __restrict__ X, int n) {
-    extern __shared__ __align__(16) double tx[];
-    const int j = blockIdx.x;
-    const int lane = threadIdx.x;
-    if (lane == 0) tx[j] = 1.0 / C[(size_t)j * n + j];
-    __syncwarp();
-    for (int i = j + 1; i < n; ++i) {
-        double s = 0.0;
-        for (int k = j + lane; k < i; k += 32) s += C[(size_t)i * n + k] * tx[k];
-        s = warp_sum(s);
-        if (lane == 0) tx[i] = -s / C[(size_t)i * n + i];
-        __syncwarp();
-    }
-    for (int i = lane; i < n; i += 32) X[(size_t)i * n + j] = i < j ? 0.0 : tx[i];
-}
-
-// C (m x n) = op(A) op(B) * colscale[j]  (row-major; op = transpose if flag)
+// C (m x n) = op(A) op(B) * colscale[j]  (row-major; op = transpose if flag).
+// The products of Algorithm 1 have triangular operands and symmetric results,
+// and float64 is what bounds them (two FMAs per clock and SM), so a CTA's sum
+// runs over [k_lo, k_hi) of its tile only: TRI_A / TRI_B say that op(A) / op(B)
+// is lower-triangular C^{-1} (k <= i / k <= j) or, transposed, upper (k >= i);
+// GEMM_SYM computes the tiles on and below the diagonal and mirrors them.  The
+// four products at ell = 400: 534 us in full, 275 us so.
+enum : int { TRI_A = 1, TRI_B = 2, GEMM_SYM = 4 };
 __global__ void small_gemm_kernel(const double* __restrict__ A, int ta, const double* __restrict__ B, int tb, int m,
-                                  int n, int k, const double* __restrict__ colscale, double* __restrict__ C) {
+                                  int n, int k, const double* __restrict__ colscale, double* __restrict__ C,
+                                  int flags) {
+    pdl_enter();
+    // tiles with the longest sums first
+    const int bi = flags && !ta ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
+    const int bj = flags & GEMM_SYM && tb ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    if ((flags & GEMM_SYM) && bj > bi) return;
     __shared__ double As[16][17];
     __shared__ double Bs[16][17];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int i = blockIdx.y * 16 + ty, j = blockIdx.x * 16 + tx;
+    const int i = bi * 16 + ty, j = bj * 16 + tx;
+    int k_lo = 0, k_hi = k;
+    if (flags & TRI_A) {
+        if (ta) k_lo = bi * 16;
+        else k_hi = min(k_hi, bi * 16 + 16);
+    }
+    if (flags & TRI_B) {
+        if (tb) k_hi = min(k_hi, bj * 16 + 16);
+        else k_lo = max(k_lo, bj * 16);
+    }
     double acc = 0.0;
-    for (int k0 = 0; k0 < k; k0 += 16) {
+    for (int k0 = k_lo; k0 < k_hi; k0 += 16) {
         const int ka = k0 + tx, kb = k0 + ty;
-        // A(i, ka): ta ? A[ka][i] (A is k x m) : A[i][ka] (A is m x k)
-        As[ty][tx] = (i < m && ka < k) ? (ta ? A[(size_t)ka * m + i] : A[(size_t)i * k + ka]) : 0.0;
+        // A(i, ka): ta ? A[ka][i] (A is k x m) : A[i][ka] (A is m x k), read along
+        // its rows in either case
+        if (ta) As[tx][ty] = (bi * 16 + tx < m && kb < k) ? A[(size_t)kb * m + bi * 16 + tx] : 0.0;
+        else As[ty][tx] = (i < m && ka < k) ? A[(size_t)i * k + ka] : 0.0;
         // B(kb, j): tb ? B[j][kb] (B is n x k) : B[kb][j] (B is k x n)
-        Bs[ty][tx] = (kb < k && j < n) ? (tb ? B[(size_t)j * k + kb] : B[(size_t)kb * n + j]) : 0.0;
+        if (tb) Bs[tx][ty] = (ka < k && bj * 16 + ty < n) ? B[(size_t)(bj * 16 + ty) * k + ka] : 0.0;
+        else Bs[ty][tx] = (kb < k && j < n) ? B[(size_t)kb * n + j] : 0.0;
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < 16; ++kk) acc = fma(As[ty][kk], Bs[kk][tx], acc);
         __syncthreads();
     }
-    if (i < m && j < n) C[(size_t)i * n + j] = acc * (colscale ? colscale[j] : 1.0);
+    if (i < m && j < n) {
+        const double v = acc * (colscale ? colscale[j] : 1.0);
+        C[(size_t)i * n + j] = v;
+        if ((flags & GEMM_SYM) && bj < bi) C[(size_t)j * n + i] = v;
+    }
 }
 
 template <class T>
@@ -567,42 +577,77 @@ __global__ void __launch_bounds__(256) rot_apply_kernel(const int2* __restrict__
         for (int j = lane; j < n; j += 32) V[(size_t)i * n + j] = row[j];
 }
 
-// lambda_i = v_i^T G v_i / (v_i^T v_i), G float64 (ld = ell), V (ld = n) of T.
+// Rayleigh quotients lambda_i = v_i^T G v_i / (v_i^T v_i), G float64 symmetric
+// (ld = ell), V (ld = n) of T: CTA (c, r) adds, for 16 columns i of V, the terms
+// of rows r0 .. r0 + 15, sum_r v_r (G_rr v_r + 2 sum_{k < r} G_rk v_k), into
+// part[r][0 / 1][i] (numerators, denominators).  ell = 400: 92 us (one CTA per
+// column over all of G: 337 us).
 template <class T>
-__global__ void rayleigh_kernel(const double* __restrict__ G, const T* __restrict__ V, int ell, int n,
-                                double* __restrict__ lam) {
-    __shared__ double sh[32];
-    const int i = blockIdx.x;
-    double num = 0.0, den = 0.0;
-    for (int r = threadIdx.x; r < ell; r += blockDim.x) {
-        const double vr = (double)V[(size_t)r * n + i];
-        double gv = 0.0;
-        for (int c = 0; c < ell; ++c) gv += G[(size_t)r * ell + c] * (double)V[(size_t)c * n + i];
-        num += vr * gv;
-        den += vr * vr;
+__global__ void __launch_bounds__(256) rayleigh_kernel(const double* __restrict__ G, const T* __restrict__ V, int ell,
+                                                       int n, double* __restrict__ part) {
+    pdl_enter();
+    __shared__ double Gs[16][17], Vs[16][17];
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int br = gridDim.y - 1 - blockIdx.y, r = br * 16 + ty, i = blockIdx.x * 16 + tx;   // longest sums first
+    double acc = 0.0;
+    for (int k0 = 0; k0 <= br * 16; k0 += 16) {
+        const int kg = k0 + tx, kv = k0 + ty;
+        Gs[ty][tx] = r < ell && kg <= r ? G[(size_t)r * ell + kg] * (kg < r ? 2.0 : 1.0) : 0.0;
+        Vs[ty][tx] = kv < ell && i < ell ? (double)V[(size_t)kv * n + i] : 0.0;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 16; ++k) acc = fma(Gs[ty][k], Vs[k][tx], acc);
+        __syncthreads();
     }
-    num = block_sum(num, sh);
-    den = block_sum(den, sh);
-    if (threadIdx.x == 0) lam[i] = num / den;
+    const double v = r < ell && i < ell ? (double)V[(size_t)r * n + i] : 0.0;
+    Gs[ty][tx] = v * acc;
+    Vs[ty][tx] = v * v;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const double(*src)[17] = threadIdx.x < 16 ? Gs : Vs;
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) s += src[k][tx];
+        if (i < ell) part[((size_t)br * 2 + (threadIdx.x >> 4)) * ell + i] = s;
+    }
 }
 
-// sort eigenpairs descending; Vout (ell x ell float64, column k = k-th
-// eigenvector), S2 = sorted eigenvalues, S_hat = max(0, S2 - v), scale = 1/sqrt(S2)
+// descending order of the eigenpairs: every CTA sums the quotients (nr partial
+// sums) and ranks them, then writes row blockIdx.x of Vout (ell x ell float64,
+// column k = k-th eigenvector); block 0 writes S_hat = max(0, lambda - v) and
+// scale = 1/sqrt(lambda).  Dynamic shared memory: ell doubles.
 template <class T>
-__global__ void sort_eig_kernel(const double* __restrict__ lam, const T* __restrict__ V, int ell, int n,
-                                const double* __restrict__ info, double* __restrict__ Vout,
-                                double* __restrict__ S_hat, double* __restrict__ scale) {
-    const double v = info[1];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ell; i += gridDim.x * blockDim.x) {
-        const double li = lam[i];
+__global__ void __launch_bounds__(256) sort_eig_kernel(const double* __restrict__ part, int nr,
+                                                       const T* __restrict__ V, int ell, int n,
+                                                       const double* __restrict__ info, double* __restrict__ Vout,
+                                                       double* __restrict__ S_hat, double* __restrict__ scale) {
+    pdl_enter();
+    extern __shared__ __align__(16) long long lam[];
+    for (int i = threadIdx.x; i < ell; i += blockDim.x) {
+        double num = 0.0, den = 0.0;
+        for (int r = 0; r < nr; ++r) {
+            num += part[(size_t)(2 * r) * ell + i];
+            den += part[(size_t)(2 * r + 1) * ell + i];
+        }
+        // as an integer of the same order: a float64 comparison occupies the
+        // float64 pipe (ell = 400: 115 us a CTA for the ranks, 25 us with integers)
+        const long long b = __double_as_longlong(num / den + 0.0);      // -0 becomes 0
+        lam[i] = b ^ ((b >> 63) & 0x7fffffffffffffffll);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < ell; i += blockDim.x) {
+        const long long ki = lam[i];
         int rank = 0;
         for (int j = 0; j < ell; ++j) {
-            const double lj = lam[j];
-            rank += (lj > li) || (lj == li && j < i);
+            const long long kj = lam[j];
+            rank += (kj > ki) || (kj == ki && j < i);
         }
-        S_hat[rank] = fmax(0.0, li - v);
-        scale[rank] = li > 0.0 ? 1.0 / sqrt(li) : 0.0;
-        for (int r = 0; r < ell; ++r) Vout[(size_t)r * ell + rank] = (double)V[(size_t)r * n + i];
+        const double li = __longlong_as_double(ki ^ ((ki >> 63) & 0x7fffffffffffffffll));
+        if (blockIdx.x == 0) {
+            S_hat[rank] = fmax(0.0, li - info[1]);
+            scale[rank] = li > 0.0 ? 1.0 / sqrt(li) : 0.0;
+        }
+        for (int r = blockIdx.x; r < ell; r += gridDim.x) Vout[(size_t)r * ell + rank] = (double)V[(size_t)r * n + i];
     }
 }
 
@@ -628,12 +673,6 @@ __global__ void form_A_kernel(const double* __restrict__ K, int ldk, const doubl
     }
 }
 
-__global__ void chol_kernel(double* __restrict__ A, int n, double* __restrict__ info) {
-    __shared__ int flag;
-    const bool ok = block_cholesky(A, n, &flag);
-    if (threadIdx.x == 0) info[3] = ok ? 0.0 : 1.0;
-}
-
 // M (ell x ell) = diag(sqd) Ainv diag(sqd) on the leading eff x eff block
 // (Ainv has ld = eff), zero elsewhere; also a float copy
 __global__ void form_M_kernel(const double* __restrict__ Ainv, const double* __restrict__ sqd, int ell, int eff,
@@ -648,17 +687,17 @@ __global__ void form_M_kernel(const double* __restrict__ Ainv, const double* __r
 
 // ---------------------------------------------------------------- host ---
 int launch_small_gemm(nys_ctx* ctx, const double* A, int ta, const double* B, int tb, int m, int n, int k,
-                      const double* colscale, double* C) {
+                      const double* colscale, double* C, int flags) {
     dim3 grid((n + 15) / 16, (m + 15) / 16);
-    small_gemm_kernel<<<grid, 256, 0, ctx->stream>>>(A, ta, B, tb, m, n, k, colscale, C);
+    NYS_CK(ctx, launch_pdl(small_gemm_kernel, grid, 256, 0, ctx->stream, A, ta, B, tb, m, n, k, colscale, C, flags));
     NYS_LAUNCH_CK(ctx);
     return NYS_OK;
 }
 
 // Eigen-decomposition of the symmetric ell x ell float64 matrix G:
 // Vout (ell x ell, columns sorted by descending eigenvalue), S_hat, scale.
-// `work` provides 2 n^2 + n doubles (the float path: n^2 floats each for the
-// padded copy, V and the cluster kernel's R, and n doubles).  `use_f32` picks
+// `work` provides 2 n^2 doubles (the float path: n^2 floats each for the padded
+// copy, V and the cluster kernel's R).  `use_f32` picks
 // the Jacobi type.
 int sym_eig(nys_ctx* ctx, const double* G, int ell, bool use_f32, const double* info, void* work, double* Vout,
             double* S_hat, double* scale, int* sweeps_dev) {
@@ -669,7 +708,6 @@ int sym_eig(nys_ctx* ctx, const double* G, int ell, bool use_f32, const double* 
         using T = std::remove_pointer_t<decltype(tag)>;
         T* Gw = (T*)work;
         T* V = Gw + (size_t)n * n;
-        double* lam = (double*)(V + (size_t)n * n);
         // padded copy in the working type
         NYS_CK(ctx, cudaMemsetAsync(Gw, 0, sizeof(T) * n * n, s));
         copy_pad<T><<<64, 256, 0, s>>>(G, ell, Gw, n);
@@ -684,22 +722,30 @@ int sym_eig(nys_ctx* ctx, const double* G, int ell, bool use_f32, const double* 
         const double tol = sizeof(T) == 8 ? 1e-14 : 2e-7;
         const int h = n / 2;
         int* status_dev = sweeps_dev + 2;
+        const int nt = (ell + 15) / 16;
+        auto quotients = [&]() -> int {
+            int st = NYS_OK;
+            double* part = (double*)scratch(ctx, SLOT_MISC, (size_t)2 * nt * ell * sizeof(double), &st);
+            if (st) return st;
+            NYS_CK(ctx, launch_pdl(rayleigh_kernel<T>, dim3(nt, nt), 256, 0, s, G, (const T*)V, ell, n, part));
+            NYS_LAUNCH_CK(ctx);
+            NYS_CK(ctx, launch_pdl(sort_eig_kernel<T>, std::min(ell, ctx->sm_count), 256, ell * sizeof(double), s,
+                                   (const double*)part, nt, (const T*)V, ell, n, info, Vout, S_hat, scale));
+            NYS_LAUNCH_CK(ctx);
+            return NYS_OK;
+        };
         if (sizeof(T) == 4) {
             // float32 sketches of 64..448 columns: the cluster kernel (Cholesky
             // and one-sided Jacobi spread over 8 or 16 SMs, V formed in place);
             // the two-sided kernel runs instead if its Cholesky fails
-            // R's copy for the back substitution after lam: the work area holds
-            // 2 n^2 doubles + n, the float path uses n^2 + n^2 floats + n doubles
-            float* Rsave = (float*)(lam + n);
+            // R's copy for the back substitution: the work area holds 2 n^2
+            // doubles, the float path uses three times n^2 floats
+            float* Rsave = (float*)(V + (size_t)n * n);
             const int stc = jacobi_cluster(ctx, G, ell, max_sweeps, (float*)V, n, Rsave, sweeps_dev, status_dev);
             if (stc == NYS_OK) {
                 jacobi_kernel<T><<<1, 1024, 0, s>>>(Gw, V, n, ell, max_sweeps, tol, sweeps_dev, status_dev);
                 NYS_LAUNCH_CK(ctx);
-                rayleigh_kernel<T><<<ell, 128, 0, s>>>(G, V, ell, n, lam);
-                NYS_LAUNCH_CK(ctx);
-                sort_eig_kernel<T><<<(ell + 127) / 128, 128, 0, s>>>(lam, V, ell, n, info, Vout, S_hat, scale);
-                NYS_LAUNCH_CK(ctx);
-                return NYS_OK;
+                return quotients();
             }
             if (stc != NYS_EINVAL) return stc;
         }
@@ -755,11 +801,7 @@ int sym_eig(nys_ctx* ctx, const double* G, int ell, bool use_f32, const double* 
             jacobi_kernel<T><<<1, 1024, 0, s>>>(Gw, V, n, ell, max_sweeps, tol, sweeps_dev, status_dev);
             NYS_LAUNCH_CK(ctx);
         }
-        rayleigh_kernel<T><<<ell, 128, 0, s>>>(G, V, ell, n, lam);
-        NYS_LAUNCH_CK(ctx);
-        sort_eig_kernel<T><<<(ell + 127) / 128, 128, 0, s>>>(lam, V, ell, n, info, Vout, S_hat, scale);
-        NYS_LAUNCH_CK(ctx);
-        return NYS_OK;
+        return quotients();
     };
     return use_f32 ? run((float*)nullptr) : run((double*)nullptr);
 }
