@@ -243,7 +243,8 @@ __global__ void __launch_bounds__(256) utz_vec_kernel(const TU* __restrict__ U, 
 }
 
 template <class TU, class TZ, class TA>
-int precond_vec(nys_ctx* ctx, const nys_precond* pc, int inverse, const void* z, void* out, int batch) {
+int precond_vec(nys_ctx* ctx, const nys_precond* pc, int inverse, const void* z, void* out, int batch,
+                const void* base = nullptr, double scale = 1.0) {
     constexpr int V = Vec16<TU>::n;
     const nys_precond_priv* pv = (const nys_precond_priv*)pc->priv;
     const int64_t N = pc->N;
@@ -272,6 +273,19 @@ int precond_vec(nys_ctx* ctx, const nys_precond* pc, int inverse, const void* z,
     using TM = typename std::conditional<sizeof(TA) == 8, double, float>::type;
     const TM* Mp = sizeof(TA) == 8 ? (const TM*)pv->M64 : (const TM*)pv->M32;
     const TM* dp = sizeof(TA) == 8 ? (const TM*)pv->d : (const TM*)pv->d32;
+    // few columns and pixels: the coefficients in the last pass itself, while its
+    // CTAs, which all form them, are at most two to an SM (bf16 U, one image of
+    // 256 x 256: 12 columns 6.7 against 8.0 us, 40 columns 10.4 against 11.1, 64
+    // columns 12.9 against 12.2; four such images, 12 columns: 13.2 against 12.6)
+    if (ell <= 48 && (N + 32 * V - 1) / (32 * V) * batch <= 2 * ctx->sm_count) {
+        const int P = 32 * V;
+        const size_t sm = 2 * (((size_t)ell + 3) & ~size_t(3)) * sizeof(TA) + (size_t)8 * P * sizeof(TA);
+        NYS_CK(ctx, launch_pdl(uc_coef_kernel<TU, TZ, TA, TM>, dim3((unsigned)((N + P - 1) / P), batch), 256, sm, s,
+                               (const TU*)pc->U, (const TZ*)z, N, ell, (const TA*)part, nchunk, pc->ell, inverse, Mp, dp,
+                               inverse ? TA(-1) : TA(1), (TZ*)out, (const TZ*)base, TA(scale), keep));
+        NYS_LAUNCH_CK(ctx);
+        return NYS_OK;
+    }
     if ((st = coef_run<TA, TM>(ctx, part, nchunk, ell, pc->ell, inverse, Mp, dp, coef, batch, wbuf))) return st;
     // large active sets: two 16-byte vectors per lane and two columns per
     // round (1 KB contiguous per column and warp, near the HBM rate)
@@ -281,11 +295,11 @@ int precond_vec(nys_ctx* ctx, const nys_precond* pc, int inverse, const void* z,
     const dim3 grid((unsigned)((N + P - 1) / P), batch);
     if (pvx == 1)
         NYS_CK(ctx, launch_pdl(uc_vec_kernel<TU, TZ, TA>, grid, 256, sm, s, (const TU*)pc->U, (const TZ*)z, N, ell,
-                               coef, inverse ? TA(-1) : TA(1), (TZ*)out, (const TZ*)nullptr, TA(1), keep,
+                               coef, inverse ? TA(-1) : TA(1), (TZ*)out, (const TZ*)base, TA(scale), keep,
                                DualStop{}));
     else
         NYS_CK(ctx, launch_pdl(uc_vec_kernel<TU, TZ, TA, 2, 2>, grid, 256, sm, s, (const TU*)pc->U, (const TZ*)z, N,
-                               ell, coef, inverse ? TA(-1) : TA(1), (TZ*)out, (const TZ*)nullptr, TA(1), keep,
+                               ell, coef, inverse ? TA(-1) : TA(1), (TZ*)out, (const TZ*)base, TA(scale), keep,
                                DualStop{}));
     NYS_LAUNCH_CK(ctx);
     return NYS_OK;
@@ -452,6 +466,21 @@ int precond_run(nys_ctx* ctx, const nys_precond* pc, int inverse, int dtype, con
     if (pc->dtype == NYS_F32) return precond_typed<float, float, float>(ctx, pc, inverse, z, out, batch);
     if (pc->dtype == NYS_BF16) return precond_typed<__nv_bfloat16, float, float>(ctx, pc, inverse, z, out, batch);
     return fail(ctx, NYS_EINVAL, "precond: f32 data needs an f32 or bf16 factor");
+}
+
+int precond_axpy_run(nys_ctx* ctx, const nys_precond* pc, int dtype, const void* z, const void* base, double scale,
+                     void* out) {
+    if (!pc || !pc->priv || !pc->U || pc->mu != pc->mu) return NYS_EINVAL;
+    if (((const nys_precond_priv*)pc->priv)->ell_eff == 0) return NYS_EINVAL;
+    const int V = pc->dtype == NYS_BF16 ? 8 : (pc->dtype == NYS_F32 ? 4 : 2);
+    if (pc->N % V || pc->N % 4 || (((uintptr_t)pc->U | (uintptr_t)z | (uintptr_t)base | (uintptr_t)out) & 15))
+        return NYS_EINVAL;
+    if (dtype == NYS_F64 && pc->dtype == NYS_F64)
+        return precond_vec<double, double, double>(ctx, pc, 1, z, out, 1, base, scale);
+    if (dtype != NYS_F32) return NYS_EINVAL;
+    if (pc->dtype == NYS_F32) return precond_vec<float, float, float>(ctx, pc, 1, z, out, 1, base, scale);
+    if (pc->dtype == NYS_BF16) return precond_vec<__nv_bfloat16, float, float>(ctx, pc, 1, z, out, 1, base, scale);
+    return NYS_EINVAL;
 }
 
 // Omega (total entries of store_dt, starting at element `first` of the

@@ -379,6 +379,11 @@ namespace nys {
 // not null the input is computed on the fly (used by the fused prox kernels).
 int precond_run(nys_ctx* ctx, const nys_precond* pc, int inverse, int dtype, const void* z,
                 void* out, int batch);
+// out = base + scale P^{-1} z in the apply's own last pass (one image, the same
+// operations as precond_run followed by base + scale (.)); NYS_EINVAL, nothing
+// launched, where the vectorised apply does not run
+int precond_axpy_run(nys_ctx* ctx, const nys_precond* pc, int dtype, const void* z, const void* base, double scale,
+                     void* out);
 // the contexts an unrolled-solve handle launches on (unroll.cu)
 void unroll_contexts(const nys_unroll* U, nys_ctx** ctx, nys_ctx** op_ctx);
 // dual APG prox with the fused two-launch (TV) or three-launch (HS) step

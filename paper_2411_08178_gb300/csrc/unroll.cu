@@ -62,6 +62,7 @@ struct UB {
     T *s, *g, *xt, *xbar, *ubar, *sbar, *t1, *nb;
     T *R, *Qp, *Qbar, *Rbar, *Qbw;
     T* a1;
+    T* w;
     T* y;
     size_t rec_stride;
     T* rec;
@@ -85,7 +86,8 @@ UB<T> bufs(const nys_unroll* U) {
     b.sbar = t + 5 * N; b.t1 = t + 6 * N; b.nb = t + 7 * N;
     T* t2 = t + 8 * N;
     b.R = t2; b.Qp = t2 + 2 * N; b.Qbar = t2 + 4 * N; b.Rbar = t2 + 6 * N; b.Qbw = t2 + 8 * N;
-    b.a1 = t2 + 10 * N;
+    b.w = t2 + 10 * N;
+    b.a1 = t2 + 11 * N;
     b.y = (T*)U->y;
     b.rec_stride = (size_t)N + M + (size_t)(U->J + 1) * 2 * N;
     b.rec = (T*)U->rec;
@@ -104,12 +106,14 @@ __device__ __forceinline__ typename Comp<T>::type clip1(T v) {
 // r = r - y
 template <class T>
 __global__ void sub_kernel(T* __restrict__ r, const T* __restrict__ y, int64_t n) {
+    pdl_enter();
     GRID_LOOP(t, n) r[t] = r[t] - y[t];
 }
 
 // out = a + c * b
 template <class T>
 __global__ void axpy_kernel(const T* __restrict__ a, const T* __restrict__ b, double c, int64_t n, T* __restrict__ out) {
+    pdl_enter();
     using TC = typename Comp<T>::type;
     GRID_LOOP(t, n) out[t] = (T)((TC)a[t] + (TC)c * (TC)b[t]);
 }
@@ -118,6 +122,7 @@ __global__ void axpy_kernel(const T* __restrict__ a, const T* __restrict__ b, do
 template <class T>
 __global__ void lt_tv_kernel(const T* __restrict__ Q, int n1, int n2, T* __restrict__ out, T* __restrict__ acc_into,
                              double c) {
+    pdl_enter();
     using TC = typename Comp<T>::type;
     const int64_t N = (int64_t)n1 * n2;
     GRID_LOOP(t, N) {
@@ -128,27 +133,38 @@ __global__ void lt_tv_kernel(const T* __restrict__ Q, int n1, int n2, T* __restr
     }
 }
 
-// forward dual step: z = R + step L x; Q' = clip(z); R <- Q' + beta (Q' - Qp);
-// Qp <- Q'; z stored if zout
+// forward dual step and the L^T after it: z = Ro + step L x; Q' = clip(z);
+// R' = Q' + beta (Q' - Qo); g = L^T R' (Rn null, the last step: L^T Q'); z stored
+// if zout.  The values that L^T needs from the lower and the right neighbour are
+// recomputed with the same operations that store them, so (R, Q) live in two
+// buffers and the sums are those of a dual step and an L^T launched one after
+// the other.
 template <class T>
-__global__ void dual_step_kernel(const T* __restrict__ x, T* __restrict__ R, T* __restrict__ Qp,
-                                 T* __restrict__ zout, double step, double beta, int n1, int n2) {
+__global__ void __launch_bounds__(256) dual_lt_kernel(const T* __restrict__ x, const T* __restrict__ Ro,
+                                                      const T* __restrict__ Qo, T* __restrict__ Rn,
+                                                      T* __restrict__ Qn, T* __restrict__ zout, T* __restrict__ g,
+                                                      typename Comp<T>::type step, typename Comp<T>::type beta, int n1,
+                                                      int n2) {
+    pdl_enter();
     using TC = typename Comp<T>::type;
     const int64_t N = (int64_t)n1 * n2;
     GRID_LOOP(t, N) {
         const int i = (int)(t / n2), j = (int)(t - (int64_t)i * n2);
+        const int64_t td = (i + 1 < n1 ? t + n2 : j), tr = (j + 1 < n2 ? t + 1 : t - j);
         const TC xc = (TC)x[t];
-        const TC v[2] = {xc - (TC)at(x, i - 1, j, n1, n2), xc - (TC)at(x, i, j - 1, n1, n2)};
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const int64_t e = t + c * N;
-            const T z = (T)((TC)R[e] + (TC)step * v[c]);
-            const TC q = clip1(z);
-            const TC o = (TC)Qp[e];
-            R[e] = (T)(q + (TC)beta * (q - o));
-            Qp[e] = (T)q;
-            if (zout) zout[e] = z;
-        }
+        auto z_of = [&](int64_t e, TC lx) { return (TC)(T)fma(step, lx, (TC)Ro[e]); };
+        // R' (Q' on the last step) of component entry e
+        auto r_of = [&](int64_t e, TC z) {
+            const TC q = clip1((T)z);
+            return Rn ? (TC)(T)fma(beta, q - (TC)Qo[e], q) : q;
+        };
+        const TC z1 = z_of(t, xc - (TC)at(x, i - 1, j, n1, n2)), z2 = z_of(t + N, xc - (TC)at(x, i, j - 1, n1, n2));
+        const TC r1 = r_of(t, z1), r2 = r_of(t + N, z2);
+        const TC r1d = r_of(td, z_of(td, (TC)x[td] - xc)), r2r = r_of(tr + N, z_of(tr + N, (TC)x[tr] - xc));
+        if (zout) zout[t] = (T)z1, zout[t + N] = (T)z2;
+        if (Rn) Rn[t] = (T)r1, Rn[t + N] = (T)r2;
+        Qn[t] = (T)clip1((T)z1), Qn[t + N] = (T)clip1((T)z2);
+        g[t] = (T)(r1 - r1d + r2 - r2r);          // the order of lt_q
     }
 }
 
@@ -156,6 +172,7 @@ __global__ void dual_step_kernel(const T* __restrict__ x, T* __restrict__ R, T* 
 template <class T>
 __global__ void momentum_kernel(const T* __restrict__ xn, T* __restrict__ x, T* __restrict__ u, double gamma,
                                 int64_t N) {
+    pdl_enter();
     using TC = typename Comp<T>::type;
     GRID_LOOP(t, N) {
         const TC a = (TC)xn[t], b = (TC)x[t];
@@ -175,6 +192,7 @@ __device__ __forceinline__ void acc_add(double v, double* acc, double* sh) {
 template <class T>
 __global__ void mom_bwd_kernel(T* __restrict__ xbar, const T* __restrict__ ubar, T* __restrict__ sbar, double g,
                                int64_t N) {
+    pdl_enter();
     using TC = typename Comp<T>::type;
     GRID_LOOP(t, N) {
         const TC ub = (TC)ubar[t];
@@ -189,6 +207,7 @@ __global__ void __launch_bounds__(256) out_bwd_kernel(const T* __restrict__ w, c
                                                       const T* __restrict__ QJ, double lb, int n1, int n2,
                                                       T* __restrict__ Qbar, T* __restrict__ Rbar,
                                                       double* __restrict__ acc) {
+    pdl_enter();
     using TC = typename Comp<T>::type;
     __shared__ double sh[32];
     const int64_t N = (int64_t)n1 * n2;
@@ -212,6 +231,7 @@ __global__ void __launch_bounds__(256) out_bwd_kernel(const T* __restrict__ w, c
 template <class T>
 __global__ void zbar_kernel(T* __restrict__ Qbar, T* __restrict__ Rbar, const T* __restrict__ z, double beta,
                             int64_t n) {
+    pdl_enter();
     using TC = typename Comp<T>::type;
     GRID_LOOP(t, n) {
         const TC rb = (TC)Rbar[t];
@@ -222,33 +242,94 @@ __global__ void zbar_kernel(T* __restrict__ Qbar, T* __restrict__ Rbar, const T*
     }
 }
 
-// Rbar <- zbar - (1/8) L w (w = P^{-1} L^T zbar, before the step factor);
-// acc += -(1/lb) <zbar, z - R_j> - step <L w, R_j>, with R_j from the slots
-// (R_0 = Q_0, R_j = (1 + b) clip(slot_j) - b clip(slot_{j-1}), b = beta_{j-1})
+// The reverse of dual step j in terms of w = P^{-1} L^T zbar (before the step
+// factor): Rbar_j = zbar - (1/8) L w, and acc += -(1/lb) <zbar, z_j - R_j> -
+// step <L w, R_j>, with R_j from the recorded slots (R_0 = Q_0, R_j = (1 + b)
+// clip(slot_j) - b clip(slot_{j-1}), b = beta_{j-1}).
 template <class T>
-__global__ void __launch_bounds__(256) rbar_kernel(const T* __restrict__ w, const T* __restrict__ z,
-                                                   const T* __restrict__ Sj, const T* __restrict__ Sjm,
-                                                   double bprev, double lb, double step, int n1, int n2,
-                                                   T* __restrict__ Rbar, double* __restrict__ acc) {
+struct RevStep {
+    const T *w, *z, *Sj, *Sjm;
+    typename Comp<T>::type bprev, bprev1;      // b, 1 + b
+    double inv_lb, step;
+    // the two inner products at entry e; the factors 1/lb and step are left for
+    // the end (a float64 quotient per entry took most of the pass: 11.3 us for
+    // 256 x 256 pixels, 6.0 with zbar and L^T in it)
+    __device__ __forceinline__ void products(int64_t e, typename Comp<T>::type zb, typename Comp<T>::type Lw, double& p1,
+                                             double& p2) const {
+        using TC = typename Comp<T>::type;
+        const TC qj = clip1(Sj[e]);
+        const TC Rj = Sjm ? bprev1 * qj - bprev * clip1(Sjm[e]) : qj;
+        p1 += (double)zb * ((double)z[e] - (double)Rj);
+        p2 += (double)Lw * (double)Rj;
+    }
+    __device__ __forceinline__ double total(double p1, double p2) const { return -(p1 * inv_lb + step * p2); }
+};
+
+template <class T>
+__global__ void __launch_bounds__(256) rbar_kernel(RevStep<T> r, int n1, int n2, T* __restrict__ Rbar,
+                                                   double* __restrict__ acc) {
+    pdl_enter();
     using TC = typename Comp<T>::type;
     __shared__ double sh[32];
     const int64_t N = (int64_t)n1 * n2;
-    double part = 0.0;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < N; t += (int64_t)gridDim.x * blockDim.x) {
+    double p1 = 0.0, p2 = 0.0;
+    GRID_LOOP(t, N) {
         const int i = (int)(t / n2), j = (int)(t - (int64_t)i * n2);
-        const TC wc = (TC)w[t];
-        const TC Lw[2] = {wc - (TC)at(w, i - 1, j, n1, n2), wc - (TC)at(w, i, j - 1, n1, n2)};
+        const TC wc = (TC)r.w[t];
+        const TC Lw[2] = {wc - (TC)at(r.w, i - 1, j, n1, n2), wc - (TC)at(r.w, i, j - 1, n1, n2)};
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
             const int64_t e = t + c * N;
-            const TC qj = clip1(Sj[e]);
-            const TC Rj = Sjm ? (TC)(1.0 + bprev) * qj - (TC)bprev * clip1(Sjm[e]) : qj;
             const TC zb = (TC)Rbar[e];
-            part -= (double)zb * ((double)z[e] - (double)Rj) / lb + step * (double)Lw[c] * (double)Rj;
-            Rbar[e] = (T)(zb - TC(0.125) * Lw[c]);
+            r.products(e, zb, Lw[c], p1, p2);
+            Rbar[e] = (T)fma(TC(-0.125), Lw[c], zb);
         }
     }
-    acc_add<T>(part, acc, sh);
+    acc_add<T>(r.total(p1, p2), acc, sh);
+}
+
+// rbar of step j + 1, zbar of step j and L^T of it in one pass: from (zbar,
+// Qbar) of step j + 1 in Zo / Qo and its w, to those of step j in Zn / Qn (other
+// buffers: neighbours are recomputed, as in dual_lt_kernel), g = L^T zbar_j and
+// sbar += step g.
+template <class T>
+__global__ void __launch_bounds__(256) rev_step_kernel(RevStep<T> r, const T* __restrict__ Zo,
+                                                       const T* __restrict__ Qo, T* __restrict__ Zn,
+                                                       T* __restrict__ Qn, const T* __restrict__ z,
+                                                       typename Comp<T>::type beta, typename Comp<T>::type beta1,
+                                                       int n1, int n2, T* __restrict__ g, T* __restrict__ sbar,
+                                                       typename Comp<T>::type step, double* __restrict__ acc) {
+    pdl_enter();
+    using TC = typename Comp<T>::type;
+    __shared__ double sh[32];
+    const int64_t N = (int64_t)n1 * n2;
+    double p1 = 0.0, p2 = 0.0;
+    GRID_LOOP(t, N) {
+        const int i = (int)(t / n2), j = (int)(t - (int64_t)i * n2);
+        const int64_t td = (i + 1 < n1 ? t + n2 : j), tr = (j + 1 < n2 ? t + 1 : t - j);
+        const TC wc = (TC)r.w[t];
+        auto rbar = [&](int64_t e, TC lw) { return (TC)(T)fma(TC(-0.125), lw, (TC)Zo[e]); };
+        auto zbar = [&](int64_t e, TC rb) {
+            const TC qb = fma(beta1, rb, (TC)Qo[e]), zz = (TC)z[e];
+            return (zz < TC(1) && zz > TC(-1)) ? (TC)(T)qb : TC(0);
+        };
+        const TC Lw[2] = {wc - (TC)at(r.w, i - 1, j, n1, n2), wc - (TC)at(r.w, i, j - 1, n1, n2)};
+        TC zb[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int64_t e = t + c * N;
+            r.products(e, (TC)Zo[e], Lw[c], p1, p2);
+            const TC rb = rbar(e, Lw[c]);
+            zb[c] = zbar(e, rb);
+            Zn[e] = (T)zb[c];
+            Qn[e] = (T)(-beta * rb);
+        }
+        const TC zd = zbar(td, rbar(td, (TC)r.w[td] - wc)), zr = zbar(tr + N, rbar(tr + N, (TC)r.w[tr] - wc));
+        const TC gv = zb[0] - zd + zb[1] - zr;     // the order of lt_q
+        g[t] = (T)gv;
+        sbar[t] = (T)fma(step, gv, (TC)sbar[t]);
+    }
+    acc_add<T>(r.total(p1, p2), acc, sh);
 }
 
 // out += scale * dK(w, x): the derivative of <w, h (*) x> with respect to each
@@ -258,6 +339,7 @@ constexpr int KT = 32;
 template <class T>
 __global__ void __launch_bounds__(256) kgrad_kernel(const T* __restrict__ w, const T* __restrict__ x, int n1, int n2,
                                                     int kh, int kw, double scale, double* __restrict__ part) {
+    pdl_enter();
     using TC = typename Comp<T>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int ch = (kh - 1) / 2, cw = (kw - 1) / 2;
@@ -292,6 +374,7 @@ __global__ void __launch_bounds__(256) kgrad_kernel(const T* __restrict__ w, con
 // dlam = alpha * sum(acc);  dh[tap] = sum over CTAs of the tap partials
 __global__ void final_kernel(const double* __restrict__ acc, int grid, const double* __restrict__ kpart, int kgrid,
                              int ntaps, double alpha, double* __restrict__ out) {
+    pdl_enter();
     __shared__ double sh[32];
     double v = 0.0;
     for (int t = threadIdx.x; t < grid; t += blockDim.x) v += acc[t];
@@ -305,6 +388,25 @@ __global__ void final_kernel(const double* __restrict__ acc, int grid, const dou
 }
 
 // ---------------------------------------------------------------- host ---
+#define UNROLL_GO(kernel, grid, smem, ...)                                                    \
+    do {                                                                                     \
+        NYS_CK(ctx, launch_pdl(kernel, grid, 256, smem, ctx->stream, __VA_ARGS__));          \
+        NYS_LAUNCH_CK(ctx);                                                                  \
+    } while (0)
+
+// out = base + scale P^{-1} z (z overwritten or kept)
+template <class T>
+int pinv_axpy(nys_unroll* U, T* z, const T* base, double scale, T* out) {
+    nys_ctx* ctx = U->ctx;
+    if (U->pc) {
+        const int st = precond_axpy_run(ctx, U->pc, U->dtype, z, base, scale, out);
+        if (st != NYS_EINVAL) return st;
+        if (int st2 = precond_run(ctx, U->pc, 1, U->dtype, z, z, 1)) return st2;
+    }
+    UNROLL_GO(axpy_kernel<T>, U->grid, 0, base, (const T*)z, scale, U->N, out);
+    return NYS_OK;
+}
+
 template <class T>
 int pinv(nys_unroll* U, const T* z, T* out) {
     if (!U->pc) {
@@ -317,6 +419,7 @@ int pinv(nys_unroll* U, const T* z, T* out) {
 // one forward outer iteration k; rec_i >= 0 records into record slot rec_i
 template <class T>
 int fwd_iter(nys_unroll* U, const UB<T>& b, int k, int rec_i) {
+    using TC = typename Comp<T>::type;
     nys_ctx* ctx = U->ctx;
     cudaStream_t s = ctx->stream;
     const int64_t N = U->N, M = U->M;
@@ -327,34 +430,28 @@ int fwd_iter(nys_unroll* U, const UB<T>& b, int k, int rec_i) {
     T* r = rec_i >= 0 ? b.rec_r(rec_i, N) : b.a1;
     if (rec_i >= 0) NYS_CK(ctx, cudaMemcpyAsync(b.rec_u(rec_i), b.u, sizeof(T) * N, cudaMemcpyDeviceToDevice, s));
     if ((st = op_run(U->op, 0, b.u, r, 1, U->dtype, U->dtype))) return st;
-    sub_kernel<T><<<g, 256, 0, s>>>(r, b.y, M);
-    NYS_LAUNCH_CK(ctx);
+    UNROLL_GO(sub_kernel<T>, g, 0, r, (const T*)b.y, M);
     if ((st = op_run(U->op, 1, r, b.g, 1, U->dtype, U->dtype))) return st;
-    if ((st = pinv<T>(U, b.g, b.g))) return st;
-    axpy_kernel<T><<<g, 256, 0, s>>>(b.u, b.g, -U->alpha, N, b.s);
-    NYS_LAUNCH_CK(ctx);
+    if ((st = pinv_axpy<T>(U, b.g, b.u, -U->alpha, b.s))) return st;
     if (rec_i >= 0)
         NYS_CK(ctx, cudaMemcpyAsync(b.rec_slot(rec_i, 0, N, M), b.Q, sizeof(T) * 2 * N, cudaMemcpyDeviceToDevice, s));
-    NYS_CK(ctx, cudaMemcpyAsync(b.R, b.Q, sizeof(T) * 2 * N, cudaMemcpyDeviceToDevice, s));
-    NYS_CK(ctx, cudaMemcpyAsync(b.Qp, b.Q, sizeof(T) * 2 * N, cudaMemcpyDeviceToDevice, s));
+    UNROLL_GO(lt_tv_kernel<T>, g, 0, (const T*)b.Q, n1, n2, b.g, (T*)nullptr, 0.0);
+    // (R, Q) ping-pong between two pairs (Qbar and Rbar are free here); step 0
+    // starts from Q itself, the last step writes it (through a copy if it is
+    // the first one too)
+    T* RQ[2][2] = {{b.R, b.Qp}, {b.Qbar, b.Rbar}};
     for (int j = 0; j < U->J; ++j) {
-        lt_tv_kernel<T><<<g, 256, 0, s>>>(b.R, n1, n2, b.g, nullptr, 0.0);
-        NYS_LAUNCH_CK(ctx);
-        if ((st = pinv<T>(U, b.g, b.g))) return st;
-        axpy_kernel<T><<<g, 256, 0, s>>>(b.s, b.g, -lb, N, b.xt);
-        NYS_LAUNCH_CK(ctx);
+        if ((st = pinv_axpy<T>(U, b.g, b.s, -lb, b.xt))) return st;
+        const bool last = j + 1 == U->J;
         T* z = rec_i >= 0 ? b.rec_slot(rec_i, j + 1, N, M) : nullptr;
-        dual_step_kernel<T><<<g, 256, 0, s>>>(b.xt, b.R, b.Qp, z, step, U->bet[j], n1, n2);
-        NYS_LAUNCH_CK(ctx);
+        UNROLL_GO(dual_lt_kernel<T>, g, 0, (const T*)b.xt, (const T*)(j ? RQ[j & 1][0] : b.Q),
+                  (const T*)(j ? RQ[j & 1][1] : b.Q), last ? (T*)nullptr : RQ[(j + 1) & 1][0],
+                  last && j ? b.Q : RQ[(j + 1) & 1][1], z, b.g, (TC)step, (TC)U->bet[j], n1, n2);
     }
-    NYS_CK(ctx, cudaMemcpyAsync(b.Q, b.Qp, sizeof(T) * 2 * N, cudaMemcpyDeviceToDevice, s));
-    lt_tv_kernel<T><<<g, 256, 0, s>>>(b.Q, n1, n2, b.g, nullptr, 0.0);
-    NYS_LAUNCH_CK(ctx);
-    if ((st = pinv<T>(U, b.g, b.g))) return st;
-    axpy_kernel<T><<<g, 256, 0, s>>>(b.s, b.g, -lb, N, b.xn);
-    NYS_LAUNCH_CK(ctx);
-    momentum_kernel<T><<<g, 256, 0, s>>>(b.xn, b.x, b.u, U->gam[k], N);
-    NYS_LAUNCH_CK(ctx);
+    if (U->J == 1)
+        NYS_CK(ctx, cudaMemcpyAsync(b.Q, RQ[1][1], sizeof(T) * 2 * N, cudaMemcpyDeviceToDevice, s));
+    if ((st = pinv_axpy<T>(U, b.g, b.s, -lb, b.xn))) return st;
+    UNROLL_GO(momentum_kernel<T>, g, 0, (const T*)b.xn, b.x, b.u, U->gam[k], N);
     return NYS_OK;
 }
 
@@ -384,6 +481,7 @@ int forward_typed(nys_unroll* U, const void* y, void* x_out) {
 
 template <class T>
 int backward_typed(nys_unroll* U, const void* xbar_in, double* grads) {
+    using TC = typename Comp<T>::type;
     nys_ctx* ctx = U->ctx;
     cudaStream_t s = ctx->stream;
     UB<T> b = bufs<T>(U);
@@ -408,44 +506,58 @@ int backward_typed(nys_unroll* U, const void* xbar_in, double* grads) {
             if ((st = fwd_iter<T>(U, b, k, k - k0))) return st;
         for (int k = k1 - 1; k >= k0; --k) {
             const int ri = k - k0;
-            mom_bwd_kernel<T><<<g, 256, 0, s>>>(b.xbar, b.ubar, b.sbar, U->gam[k], N);
-            NYS_LAUNCH_CK(ctx);
+            UNROLL_GO(mom_bwd_kernel<T>, g, 0, b.xbar, (const T*)b.ubar, b.sbar, U->gam[k], N);
             if ((st = pinv<T>(U, b.sbar, b.g))) return st;
-            out_bwd_kernel<T><<<g, 256, 0, s>>>(b.g, b.Qbw, b.rec_slot(ri, J, N, M), lb, n1, n2, b.Qbar, b.Rbar, acc);
-            NYS_LAUNCH_CK(ctx);
+            UNROLL_GO(out_bwd_kernel<T>, g, 0, (const T*)b.g, (const T*)b.Qbw, (const T*)b.rec_slot(ri, J, N, M), lb, n1,
+                      n2, b.Qbar, b.Rbar, acc);
+            // (zbar, Qbar) of the steps ping-pong (R and Qp are free here)
+            T* ZQ[2][2] = {{b.Rbar, b.Qbar}, {b.R, b.Qp}};
+            int p = 0;
+            T* gt = b.g;          // where the next L^T zbar goes; without P it is w itself
+            RevStep<T> rs{};
+            rs.inv_lb = 1.0 / lb;
+            rs.step = step;
             for (int j = J - 1; j >= 0; --j) {
-                zbar_kernel<T><<<g, 256, 0, s>>>(b.Qbar, b.Rbar, b.rec_slot(ri, j + 1, N, M), U->bet[j], 2 * N);
-                NYS_LAUNCH_CK(ctx);
-                lt_tv_kernel<T><<<g, 256, 0, s>>>(b.Rbar, n1, n2, b.g, b.sbar, step);
-                NYS_LAUNCH_CK(ctx);
-                if ((st = pinv<T>(U, b.g, b.g))) return st;
-                const T* Sjm = j >= 1 ? b.rec_slot(ri, j - 1, N, M) : nullptr;
-                const double bprev = j >= 1 ? U->bet[j - 1] : 0.0;
-                rbar_kernel<T><<<g, 256, 0, s>>>(b.g, b.rec_slot(ri, j + 1, N, M), b.rec_slot(ri, j, N, M), Sjm,
-                                                 bprev, lb, step, n1, n2, b.Rbar, acc);
-                NYS_LAUNCH_CK(ctx);
+                const T* z = b.rec_slot(ri, j + 1, N, M);
+                if (j == J - 1) {
+                    UNROLL_GO(zbar_kernel<T>, g, 0, b.Qbar, b.Rbar, z, U->bet[j], 2 * N);
+                    UNROLL_GO(lt_tv_kernel<T>, g, 0, (const T*)b.Rbar, n1, n2, gt, b.sbar, step);
+                } else {
+                    UNROLL_GO(rev_step_kernel<T>, g, 0, rs, (const T*)ZQ[p][0], (const T*)ZQ[p][1], ZQ[p ^ 1][0],
+                              ZQ[p ^ 1][1], z, (TC)U->bet[j], (TC)(1.0 + U->bet[j]), n1, n2, gt, b.sbar, (TC)step, acc);
+                    p ^= 1;
+                }
+                if (U->pc) {
+                    if ((st = pinv<T>(U, gt, b.w))) return st;
+                    rs.w = b.w;
+                } else {
+                    rs.w = gt;
+                    gt = gt == b.g ? b.w : b.g;
+                }
+                rs.z = z;
+                rs.Sj = b.rec_slot(ri, j, N, M);
+                rs.Sjm = j >= 1 ? b.rec_slot(ri, j - 1, N, M) : nullptr;
+                const double bp = j >= 1 ? U->bet[j - 1] : 0.0;
+                rs.bprev = (TC)bp;
+                rs.bprev1 = (TC)(1.0 + bp);
             }
-            axpy_kernel<T><<<g, 256, 0, s>>>(b.Qbar, b.Rbar, 1.0, 2 * N, b.Qbw);
-            NYS_LAUNCH_CK(ctx);
+            if (J) UNROLL_GO(rbar_kernel<T>, g, 0, rs, n1, n2, ZQ[p][0], acc);
+            UNROLL_GO(axpy_kernel<T>, g, 0, (const T*)ZQ[p][1], (const T*)ZQ[p][0], 1.0, 2 * N, b.Qbw);
             // ubar_k = sbar - alpha A^T A P^{-1} sbar
             if ((st = pinv<T>(U, b.sbar, b.t1))) return st;
             if ((st = op_run(U->op, 0, b.t1, b.a1, 1, U->dtype, U->dtype))) return st;
             if ((st = op_run(U->op, 1, b.a1, b.nb, 1, U->dtype, U->dtype))) return st;
-            axpy_kernel<T><<<g, 256, 0, s>>>(b.sbar, b.nb, -U->alpha, N, b.ubar);
-            NYS_LAUNCH_CK(ctx);
+            UNROLL_GO(axpy_kernel<T>, g, 0, (const T*)b.sbar, (const T*)b.nb, -U->alpha, N, b.ubar);
             if (want_h) {
-                kgrad_kernel<T><<<U->kgrid, 256, ksmem, s>>>(b.rec_r(ri, N), b.t1, n1, n2, U->op->kh, U->op->kw,
-                                                             -U->alpha, kpart);
-                NYS_LAUNCH_CK(ctx);
-                kgrad_kernel<T><<<U->kgrid, 256, ksmem, s>>>(b.a1, b.rec_u(ri), n1, n2, U->op->kh, U->op->kw,
-                                                             -U->alpha, kpart);
-                NYS_LAUNCH_CK(ctx);
+                UNROLL_GO(kgrad_kernel<T>, U->kgrid, ksmem, (const T*)b.rec_r(ri, N), (const T*)b.t1, n1, n2, U->op->kh,
+                          U->op->kw, -U->alpha, kpart);
+                UNROLL_GO(kgrad_kernel<T>, U->kgrid, ksmem, (const T*)b.a1, (const T*)b.rec_u(ri), n1, n2, U->op->kh,
+                          U->op->kw, -U->alpha, kpart);
             }
         }
     }
-    final_kernel<<<1, 256, 0, s>>>(acc, g, kpart, want_h ? U->kgrid : 0, want_h ? U->ntaps : 0, U->alpha,
-                                   acc + g + (size_t)U->kgrid * U->ntaps);
-    NYS_LAUNCH_CK(ctx);
+    UNROLL_GO(final_kernel, 1, 0, (const double*)acc, g, (const double*)kpart, want_h ? U->kgrid : 0,
+              want_h ? U->ntaps : 0, U->alpha, acc + g + (size_t)U->kgrid * U->ntaps);
     NYS_CK(ctx, cudaMemcpyAsync(grads, acc + g + (size_t)U->kgrid * U->ntaps, sizeof(double) * (1 + (want_h ? U->ntaps : 0)),
                                 cudaMemcpyDeviceToDevice, s));
     return NYS_OK;
@@ -522,7 +634,7 @@ int nys_unroll_create(nys_ctx* ctx, nys_op* op, const nys_precond* pc, const nys
     if (e == cudaSuccess) e = alloc(&U->st, es * 5 * N);
     if (e == cudaSuccess) e = alloc(&U->ckpt, es * 4 * N * U->nseg);
     if (e == cudaSuccess) e = alloc(&U->rec, es * rec_stride * U->C);
-    if (e == cudaSuccess) e = alloc(&U->tmp, es * (18 * N + M));
+    if (e == cudaSuccess) e = alloc(&U->tmp, es * (19 * N + M));
     if (e == cudaSuccess)
         e = alloc((void**)&U->acc, sizeof(double) * ((size_t)U->grid + (size_t)U->kgrid * U->ntaps + 1 + U->ntaps));
     if (e == cudaSuccess && kbytes > 48 * 1024) {

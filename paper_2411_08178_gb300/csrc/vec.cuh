@@ -270,33 +270,16 @@ __device__ __forceinline__ void last_cta_coef_t(const TA* partT, int le, int ldm
 
 // out = z + sign * U c, or with base: out = base + scale (z + sign U c).  A CTA
 // owns 32 V PV pixels (PV 16-byte vectors per lane); its 8 warps split the
-// columns, NQ columns per round, and their partial sums meet in shared memory
-template <class TU, class TZ, class TA, int NQ = 4, int PV = 1>
-__global__ void __launch_bounds__(256) uc_vec_kernel(const TU* __restrict__ U, const TZ* __restrict__ z, int64_t N,
-                                                     int ell, const TA* __restrict__ coef, TA sign,
-                                                     TZ* __restrict__ out, const TZ* __restrict__ base, TA scale,
-                                                     int keep, DualStop stop) {
-    pdl_enter();
+// columns, NQ columns per round, and their partial sums meet in shared memory.
+// c (ell) is in shared memory, red has 8 x 32 V PV entries.
+template <class TU, class TZ, class TA, int NQ, int PV>
+__device__ __forceinline__ void uc_body(const TU* __restrict__ U, const TZ* __restrict__ z, int64_t N, int ell,
+                                        const TA* c, TA* red, TA sign, TZ* __restrict__ out,
+                                        const TZ* __restrict__ base, TA scale, int keep) {
     constexpr int V = Vec16<TU>::n;
     constexpr int P = 32 * V * PV;
-    if (dual_skip(stop)) {
-        if (stop.copy)
-            for (int p = threadIdx.x; p < P; p += blockDim.x) {
-                const int64_t ii = (int64_t)blockIdx.x * P + p;
-                if (ii < N) {
-                    const size_t o = (size_t)blockIdx.y * N + ii;
-                    out[o] = reinterpret_cast<const TZ*>(stop.copy)[o];
-                }
-            }
-        return;
-    }
     const L2Pol pol = make_l2_pol();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    TA* c = reinterpret_cast<TA*>(smem_raw);
-    TA* red = c + ((ell + 3) & ~3);            // [8][P]
     const int b = blockIdx.y;
-    for (int j = threadIdx.x; j < ell; j += blockDim.x) c[j] = coef[(size_t)b * ell + j];
-    __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     TA acc[PV][V];
 #pragma unroll
@@ -344,6 +327,55 @@ __global__ void __launch_bounds__(256) uc_vec_kernel(const TU* __restrict__ U, c
         const TA v = (TA)ldf(z + o) + sign * s;
         stf(out + o, base ? (TA)ldf(base + o) + scale * v : v);
     }
+}
+
+template <class TU, class TZ, class TA, int NQ = 4, int PV = 1>
+__global__ void __launch_bounds__(256) uc_vec_kernel(const TU* __restrict__ U, const TZ* __restrict__ z, int64_t N,
+                                                     int ell, const TA* __restrict__ coef, TA sign,
+                                                     TZ* __restrict__ out, const TZ* __restrict__ base, TA scale,
+                                                     int keep, DualStop stop) {
+    pdl_enter();
+    constexpr int V = Vec16<TU>::n;
+    constexpr int P = 32 * V * PV;
+    if (dual_skip(stop)) {
+        if (stop.copy)
+            for (int p = threadIdx.x; p < P; p += blockDim.x) {
+                const int64_t ii = (int64_t)blockIdx.x * P + p;
+                if (ii < N) {
+                    const size_t o = (size_t)blockIdx.y * N + ii;
+                    out[o] = reinterpret_cast<const TZ*>(stop.copy)[o];
+                }
+            }
+        return;
+    }
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    TA* c = reinterpret_cast<TA*>(smem_raw);
+    TA* red = c + ((ell + 3) & ~3);            // [8][P]
+    const int b = blockIdx.y;
+    for (int j = threadIdx.x; j < ell; j += blockDim.x) c[j] = coef[(size_t)b * ell + j];
+    __syncthreads();
+    uc_body<TU, TZ, TA, NQ, PV>(U, z, N, ell, c, red, sign, out, base, scale, keep);
+}
+
+// The same with c = M w (or d .* w) formed by every CTA from the partial sums of
+// U^T z, with the operations of coef_vec_kernel: for few columns and CTAs that
+// costs less than a launch between the two passes.
+// Dynamic shared memory: 2 ell (padded) + 8 x 32 V entries.
+template <class TU, class TZ, class TA, class TM>
+__global__ void __launch_bounds__(256) uc_coef_kernel(const TU* __restrict__ U, const TZ* __restrict__ z, int64_t N,
+                                                      int ell, const TA* __restrict__ part, int nb, int ldm,
+                                                      int inverse, const TM* __restrict__ M, const TM* __restrict__ d,
+                                                      TA sign, TZ* __restrict__ out, const TZ* __restrict__ base,
+                                                      TA scale, int keep) {
+    pdl_enter();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    TA* c = reinterpret_cast<TA*>(smem_raw);
+    TA* w = c + ((ell + 3) & ~3);
+    TA* red = w + ((ell + 3) & ~3);
+    reduce_partials_t<TA>(part + (size_t)blockIdx.y * nb * ell, nb, ell, w);
+    coef_rows<TA, TM>(w, ell, ldm, inverse, M, d, 0, ell, c);
+    __syncthreads();
+    uc_body<TU, TZ, TA, 4, 1>(U, z, N, ell, c, red, sign, out, base, scale, keep);
 }
 
 }  // namespace
