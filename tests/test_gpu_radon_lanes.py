@@ -53,3 +53,18 @@ def test_pair_and_normal(env, geom, batch, dt):
     close(api.op_apply(op, t(x)), fwd, TOL[dt])
     close(api.op_adjoint(op, t(s)), adj, TOL[dt])
     close(api.op_normal(op, t(x)), O.radon_adjoint(fwd, n1, n2, span), TOL[dt])
+
+
+@pytest.mark.parametrize("geom,ell", [((96, 96, 180, 140, math.pi), 32), ((70, 130, 200, 157, math.pi), 45),
+                                      ((65, 64, 300, 130, 2.0 * math.pi), 41)])
+def test_bf16_batch_in_eights(env, geom, ell):
+    """The sketch's bf16 images, eight to a group (the last group of a chunk
+    half full, or of fours and a rest): Y against the oracle on the stored
+    Omega, within bf16's rounding of Y and the float32 operator's 1e-5."""
+    torch, api, ctx = env
+    n1, n2, A, B, span = geom
+    op = api.Operator(ctx, "radon", n1, n2, dtype=torch.float32, n_angles=A, n_bins=B, angle_span=span)
+    Om, Y = api.nys_sketch(ctx, op, ell, 3, store_dtype=torch.bfloat16)
+    ref = O.radon_adjoint(O.radon_apply(Om.double().cpu().numpy(), A, B, span), n1, n2, span)
+    err = np.abs(Y.double().cpu().numpy() - ref)
+    assert np.all(err <= 2.0 ** -8 * np.abs(ref) + 1e-5 * np.abs(ref).max())
