@@ -11,9 +11,10 @@
 // L = first differences (anisotropic TV, ||L||^2 = 8, Proj = clip to [-1,1])
 // or second differences (Hessian Schatten-1, ||L||^2 = 32 in the inner
 // product q11 v11 + 2 q12 v12 + q22 v22, Proj = clip the eigenvalues of each
-// symmetric 2 x 2 block to [-1, 1]).  Kernels: one stencil pass for L^T R
-// (fused with x = s - lb L^T R when P = I), P^{-1} through precond_run, and
-// one pass that forms L x, projects and extrapolates.  beta_k depends only on
+// symmetric 2 x 2 block to [-1, 1]).  Kernels: with P = I one launch a step (L x,
+// the projection, the extrapolation and the next x); otherwise one stencil
+// pass for L^T R, P^{-1} through precond_run, and one pass that forms L x,
+// projects and extrapolates (or the fused steps of prox_fused.cu).  beta_k depends only on
 // k, so it is a kernel argument and no host synchronisation is needed.
 //
 // prox_wavelet: Theorem 1 with D = I, W = I + Ubar Ubar^T: out =
@@ -97,6 +98,126 @@ __global__ void tv_dual_x_kernel(TvDual<T> d, const T* __restrict__ s, typename 
     dual_stop_report(stop, chg);
 }
 
+// Plain (P = I) dual step of the other mixed norms fused with the x after it,
+// as tv_dual_x_kernel: their projections take square roots and quotients, so
+// the new R is not recomputed per neighbour but once per pixel of a 32 x 16
+// tile and the ring around it, in shared memory (x staged two pixels around).
+// (R, Q) live in two buffers; Rn null = the last step (L^T Q_new, Q alone
+// written).  Bound by latency (the iterates stay in L2): HS_1 at 512 x 512,
+// 6.8 us a step against 8.4 for an update and an L^T launch; 640 threads (one
+// ring round) 7.2, 32 x 8 tiles 7.1, 32 x 4 7.9.
+constexpr int MTX = 32, MTY = 16, MNT = 320;
+template <class T, int REG>
+__global__ void __launch_bounds__(MNT) mixed_dual_x_kernel(const T* __restrict__ x, const T* __restrict__ Ro,
+                                                           const T* __restrict__ Qo, T* __restrict__ Rn,
+                                                           T* __restrict__ Qn, const T* __restrict__ s,
+                                                           typename Comp<T>::type lb, typename Comp<T>::type step,
+                                                           typename Comp<T>::type beta, int n1, int n2,
+                                                           T* __restrict__ out, DualStop stop) {
+    pdl_enter();
+    using TC = typename Comp<T>::type;
+    constexpr int G = dual_components(REG);
+    constexpr int XW = MTX + 4, XH = MTY + 4, RW = MTX + 2, RH = MTY + 2;
+    __shared__ TC xs[XH * XW];
+    __shared__ TC rs[G][RH * RW];
+    const int64_t N = (int64_t)n1 * n2;
+    const int tiles2 = (n2 + MTX - 1) / MTX;
+    const int i0 = (int)(blockIdx.x / tiles2) * MTY, j0 = (int)(blockIdx.x % tiles2) * MTX;
+    const bool skip = dual_skip(stop);
+    dual_stop_enter(stop, skip);
+    if (skip) {
+        if (!Rn)
+            for (int e = threadIdx.x; e < MTX * MTY; e += MNT) {
+                const int i = i0 + e / MTX, j = j0 + e % MTX;
+                if (i >= n1 || j >= n2) continue;
+                const int64_t t = (int64_t)i * n2 + j;
+#pragma unroll
+                for (int c = 0; c < G; ++c) Qn[t + c * N] = Qo[t + c * N];
+                out[t] = x[t];
+            }
+        return;
+    }
+    auto wrap = [](int v, int n) {
+        v = v < 0 ? v + n : (v >= n ? v - n : v);
+        return v < 0 || v >= n ? pmod(v, n) : v;
+    };
+    // this thread's (R, Q) are in flight while x is staged
+    constexpr int NE = (RH * RW + MNT - 1) / MNT;
+    TC r[NE][G], o[NE][G];
+#pragma unroll
+    for (int u = 0; u < NE; ++u) {
+        const int e = threadIdx.x + u * MNT;
+        if (e >= RH * RW) break;
+        const int64_t t = (int64_t)wrap(i0 - 1 + e / RW, n1) * n2 + wrap(j0 - 1 + e % RW, n2);
+#pragma unroll
+        for (int c = 0; c < G; ++c) {
+            r[u][c] = (TC)Ro[t + c * N];
+            if (Rn) o[u][c] = (TC)Qo[t + c * N];
+        }
+    }
+    for (int e = threadIdx.x; e < XH * XW; e += MNT) {
+        const int i = wrap(i0 - 2 + e / XW, n1), j = wrap(j0 - 2 + e % XW, n2);
+        xs[e] = (TC)x[(int64_t)i * n2 + j];
+    }
+    __syncthreads();
+    bool chg = false;
+#pragma unroll
+    for (int u = 0; u < NE; ++u) {
+        const int e = threadIdx.x + u * MNT;
+        if (e >= RH * RW) break;
+        const int ri = e / RW, rj = e % RW;
+        const int ti = i0 - 1 + ri, tj = j0 - 1 + rj;
+        const bool mine = ri >= 1 && ri <= MTY && rj >= 1 && rj <= MTX && ti < n1 && tj < n2;
+        const int64_t t = (int64_t)ti * n2 + tj;
+        const TC* p = xs + (ri + 1) * XW + rj + 1;
+        const TC xc = p[0];
+        TC Lx[3];
+        if (first_order(REG)) {
+            Lx[0] = xc - p[-XW];
+            Lx[1] = xc - p[-1];
+            Lx[2] = TC(0);
+        } else {
+            Lx[0] = p[-XW] - TC(2) * xc + p[XW];
+            Lx[2] = p[-1] - TC(2) * xc + p[1];
+            Lx[1] = TC(0.25) * (p[XW + 1] - p[XW - 1] - p[-XW + 1] + p[-XW - 1]);
+        }
+        TC q[G];
+        dual_project<TC, REG>(Lx, r[u], step, q);
+#pragma unroll
+        for (int c = 0; c < G; ++c) {
+            TC rn = q[c];
+            if (Rn) {
+                rn = q[c] + beta * (q[c] - o[u][c]);
+                if (mine) {
+                    Rn[t + c * N] = (T)rn;
+                    if (!(q[c] == r[u][c] && q[c] == o[u][c])) chg = true;
+                }
+            }
+            rs[c][e] = rn;
+            if (mine) Qn[t + c * N] = (T)q[c];
+        }
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < MTX * MTY; e += MNT) {
+        const int ri = e / MTX, rj = e % MTX, i = i0 + ri, j = j0 + rj;
+        if (i >= n1 || j >= n2) continue;
+        const int64_t t = (int64_t)i * n2 + j;
+        const int o = (ri + 1) * RW + rj + 1;
+        TC g;
+        if (first_order(REG)) {
+            g = rs[0][o] - rs[0][o + RW] + rs[1][o] - rs[1][o + 1];
+        } else {
+            const TC *q11 = rs[0] + o, *q12 = rs[1] + o, *q22 = rs[G - 1] + o;
+            const TC a11 = q11[-RW] - TC(2) * q11[0] + q11[RW];
+            const TC a22 = q22[-1] - TC(2) * q22[0] + q22[1];
+            const TC a12 = TC(0.25) * (q12[RW + 1] - q12[RW - 1] - q12[-RW + 1] + q12[-RW - 1]);
+            g = a11 + TC(2) * a12 + a22;
+        }
+        out[t] = (T)((TC)s[t] - lb * g);
+    }
+    dual_stop_report(stop, chg);
+}
+
 template <class T, int REG>
 int prox_dual_typed(nys_ctx* ctx, const nys_precond* pc, double lb, int n_inner, int n1, int n2, const T* s, T* out,
                     T* Q) {
@@ -120,12 +241,13 @@ int prox_dual_typed(nys_ctx* ctx, const nys_precond* pc, double lb, int n_inner,
     const int dt = sizeof(T) == 8 ? NYS_F64 : NYS_F32;
     const TC step = (TC)(1.0 / (lb * normL2));
     double t = 1.0;
-    if (!pc && REG == NYS_REG_TV) {
+    if (!pc) {
         // one launch per dual step: x ping-pongs between X[0] and X[1], (R, Q)
         // as in the preconditioned fused step (warm start from Q itself, the
         // last step writes Q unless it reads it)
         T* X[2] = {work, work + N};
         T* RQ[2][2] = {{work + 2 * N, work + 2 * N + G * N}, {work + 2 * N + 2 * G * N, work + 2 * N + 3 * G * N}};
+        const int tiles = ((n1 + MTY - 1) / MTY) * ((n2 + MTX - 1) / MTX);
         NYS_CK(ctx, launch_pdl(lt_kernel<T, REG>, grid, 256, 0, sm, Q, s, (TC)lb, n1, n2, n_inner ? X[0] : out,
                                DualStop{}));
         NYS_LAUNCH_CK(ctx);
@@ -145,8 +267,12 @@ int prox_dual_typed(nys_ctx* ctx, const nys_precond* pc, double lb, int n_inner,
             DualStop ds;
             if (ctx->dual_stop) ds.flags = ctx->counters + COUNTER_DUAL_STOP;
             ds.k = k;
-            NYS_CK(ctx, launch_pdl(tv_dual_x_kernel<T>, grid, 256, 0, sm, d, s, (TC)lb, n1, n2,
-                                   fin ? out : X[(k + 1) & 1], ds));
+            T* xo = fin ? out : X[(k + 1) & 1];
+            if constexpr (REG == NYS_REG_TV)
+                NYS_CK(ctx, launch_pdl(tv_dual_x_kernel<T>, grid, 256, 0, sm, d, s, (TC)lb, n1, n2, xo, ds));
+            else
+                NYS_CK(ctx, launch_pdl(mixed_dual_x_kernel<T, REG>, tiles, MNT, 0, sm, d.x, d.Ro, d.Qo, d.Rn, d.Qn, s,
+                                       (TC)lb, d.step, d.beta, n1, n2, xo, ds));
             NYS_LAUNCH_CK(ctx);
         }
         if (n_inner == 1) NYS_CK(ctx, cudaMemcpyAsync(Q, RQ[1][1], sizeof(T) * G * N, cudaMemcpyDeviceToDevice, sm));
@@ -159,36 +285,27 @@ int prox_dual_typed(nys_ctx* ctx, const nys_precond* pc, double lb, int n_inner,
     NYS_CK(ctx, cudaMemcpyAsync(R, Q, sizeof(T) * G * N, cudaMemcpyDeviceToDevice, sm));
     NYS_CK(ctx, cudaMemcpyAsync(Qp, Q, sizeof(T) * G * N, cudaMemcpyDeviceToDevice, sm));
     for (int k = 0; k < n_inner; ++k) {
-        // the exact early stop (internal.cuh): dual_update keeps the flags;
-        // the x of a skipped step is not recomputed (P = I)
-        DualStop ds;
-        if (ctx->dual_stop) ds.flags = ctx->counters + COUNTER_DUAL_STOP;
-        ds.k = k;
-        if (pc) {
-            NYS_CK(ctx, launch_pdl(lt_kernel<T, REG>, grid, 256, 0, sm, R, nullptr, TC(0), n1, n2, g, DualStop{}));
-            NYS_LAUNCH_CK(ctx);
-            if ((st = precond_run(ctx, pc, 1, dt, g, g, 1))) return st;
-            NYS_CK(ctx, launch_pdl(axpy_kernel<T>, grid, 256, 0, sm, s, g, (TC)lb, N, x));
-        } else {
-            NYS_CK(ctx, launch_pdl(lt_kernel<T, REG>, grid, 256, 0, sm, R, s, (TC)lb, n1, n2, x, ds));
-        }
+        NYS_CK(ctx, launch_pdl(lt_kernel<T, REG>, grid, 256, 0, sm, R, nullptr, TC(0), n1, n2, g, DualStop{}));
+        NYS_LAUNCH_CK(ctx);
+        if ((st = precond_run(ctx, pc, 1, dt, g, g, 1))) return st;
+        NYS_CK(ctx, launch_pdl(axpy_kernel<T>, grid, 256, 0, sm, s, g, (TC)lb, N, x));
         NYS_LAUNCH_CK(ctx);
         const double tn = 0.5 * (1.0 + std::sqrt(1.0 + 4.0 * t * t));
         const double beta = (t - 1.0) / tn;
         t = tn;
+        // the exact early stop (internal.cuh): dual_update keeps the flags
+        DualStop ds;
+        if (ctx->dual_stop) ds.flags = ctx->counters + COUNTER_DUAL_STOP;
+        ds.k = k;
         NYS_CK(ctx, launch_pdl(dual_update_kernel<T, REG>, grid, 256, 0, sm, x, R, Qp, step, (TC)beta, n1, n2, ds));
         NYS_LAUNCH_CK(ctx);
     }
     // Q_io <- last Q; out = s - lb P^{-1} L^T Q
     NYS_CK(ctx, cudaMemcpyAsync(Q, Qp, sizeof(T) * G * N, cudaMemcpyDeviceToDevice, sm));
-    if (pc) {
-        NYS_CK(ctx, launch_pdl(lt_kernel<T, REG>, grid, 256, 0, sm, Qp, nullptr, TC(0), n1, n2, g, DualStop{}));
-        NYS_LAUNCH_CK(ctx);
-        if ((st = precond_run(ctx, pc, 1, dt, g, g, 1))) return st;
-        NYS_CK(ctx, launch_pdl(axpy_kernel<T>, grid, 256, 0, sm, s, g, (TC)lb, N, out));
-    } else {
-        NYS_CK(ctx, launch_pdl(lt_kernel<T, REG>, grid, 256, 0, sm, Qp, s, (TC)lb, n1, n2, out, DualStop{}));
-    }
+    NYS_CK(ctx, launch_pdl(lt_kernel<T, REG>, grid, 256, 0, sm, Qp, nullptr, TC(0), n1, n2, g, DualStop{}));
+    NYS_LAUNCH_CK(ctx);
+    if ((st = precond_run(ctx, pc, 1, dt, g, g, 1))) return st;
+    NYS_CK(ctx, launch_pdl(axpy_kernel<T>, grid, 256, 0, sm, s, g, (TC)lb, N, out));
     NYS_LAUNCH_CK(ctx);
     return NYS_OK;
 }

@@ -59,63 +59,37 @@ __device__ __forceinline__ typename Comp<T>::type lt_q(const T* __restrict__ Q, 
 // the eigenvalues of the symmetric 2 x 2 block (HS_1), scale it to Frobenius
 // norm <= 1 (HS_2), or move its eigenvalue pair onto the l1 unit ball
 // (HS_inf).  chg: set when the new Q at the pixel differs from the old R or
-// Q there (the test of the exact early stop, internal.cuh).
-template <class T, int REG>
-__device__ __forceinline__ void dual_pixel(const typename Comp<T>::type* Lx, T* __restrict__ R, T* __restrict__ Qp,
-                                           int64_t t, int64_t N, typename Comp<T>::type step,
-                                           typename Comp<T>::type beta, bool* chg = nullptr) {
-    using TC = typename Comp<T>::type;
-    auto note = [&](TC q, TC r, TC o) {
-        if (chg && !(q == r && q == o)) *chg = true;
-    };
+// Q there (the test of the exact early stop, internal.cuh).  dual_project is
+// the projection alone, q = Proj(r + step Lx).
+template <class TC, int REG>
+__device__ __forceinline__ void dual_project(const TC* Lx, const TC* r, TC step, TC* q) {
     if (REG == NYS_REG_TV) {
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const int64_t e = t + c * N;
-            const TC r = (TC)R[e];
-            const TC q = fmin(TC(1), fmax(TC(-1), r + step * Lx[c]));
-            const TC o = (TC)Qp[e];
-            note(q, r, o);
-            R[e] = (T)(q + beta * (q - o));
-            Qp[e] = (T)q;
-        }
+        for (int c = 0; c < 2; ++c) q[c] = fmin(TC(1), fmax(TC(-1), r[c] + step * Lx[c]));
     } else if (REG == NYS_REG_ISOTV) {
-        TC q[2], r[2];
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            r[c] = (TC)R[t + c * N];
-            q[c] = r[c] + step * Lx[c];
-        }
+        for (int c = 0; c < 2; ++c) q[c] = r[c] + step * Lx[c];
         const TC den = fmax(TC(1), sqrt(q[0] * q[0] + q[1] * q[1]));
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const int64_t e = t + c * N;
-            const TC qc = q[c] / den;
-            const TC o = (TC)Qp[e];
-            note(qc, r[c], o);
-            R[e] = (T)(qc + beta * (qc - o));
-            Qp[e] = (T)qc;
-        }
+        for (int c = 0; c < 2; ++c) q[c] = q[c] / den;
     } else {
-        const TC ra = (TC)R[t], rb = (TC)R[t + N], rc = (TC)R[t + 2 * N];
-        const TC a = ra + step * Lx[0];
-        const TC b = rb + step * Lx[1];
-        const TC c = rc + step * Lx[2];
-        TC pa, pb, pc;
+        const TC a = r[0] + step * Lx[0];
+        const TC b = r[1] + step * Lx[1];
+        const TC c = r[2] + step * Lx[2];
         if (REG == NYS_REG_HS2) {
             const TC den = fmax(TC(1), sqrt(a * a + TC(2) * b * b + c * c));
-            pa = a / den;
-            pb = b / den;
-            pc = c / den;
+            q[0] = a / den;
+            q[1] = b / den;
+            q[2] = c / den;
         } else {
-            // eigenvalues m +- r of [[a, b], [b, c]], projected, recomposed on
+            // eigenvalues m +- e of [[a, b], [b, c]], projected, recomposed on
             // the same eigenvectors
             const TC m = TC(0.5) * (a + c), h = TC(0.5) * (a - c);
-            const TC r = sqrt(h * h + b * b);
+            const TC e = sqrt(h * h + b * b);
             TC l1, l2;
             if (REG == NYS_REG_HSINF) {
                 // onto |l1| + |l2| <= 1: soft-threshold both magnitudes by theta
-                const TC e1 = m + r, e2 = m - r;
+                const TC e1 = m + e, e2 = m - e;
                 const TC a1 = fabs(e1), a2 = fabs(e2);
                 const TC big = fmax(a1, a2), small = fmin(a1, a2);
                 TC th = big - small >= TC(1) ? big - TC(1) : TC(0.5) * (big + small - TC(1));
@@ -123,30 +97,38 @@ __device__ __forceinline__ void dual_pixel(const typename Comp<T>::type* Lx, T* 
                 l1 = copysign(fmax(a1 - th, TC(0)), e1);
                 l2 = copysign(fmax(a2 - th, TC(0)), e2);
             } else {
-                l1 = fmin(TC(1), fmax(TC(-1), m + r));
-                l2 = fmin(TC(1), fmax(TC(-1), m - r));
+                l1 = fmin(TC(1), fmax(TC(-1), m + e));
+                l2 = fmin(TC(1), fmax(TC(-1), m - e));
             }
             const TC mp = TC(0.5) * (l1 + l2), dp = TC(0.5) * (l1 - l2);
-            if (r > TC(0)) {
-                pa = mp + dp * (h / r);
-                pb = dp * (b / r);
-                pc = mp - dp * (h / r);
+            if (e > TC(0)) {
+                q[0] = mp + dp * (h / e);
+                q[1] = dp * (b / e);
+                q[2] = mp - dp * (h / e);
             } else {
-                pa = mp;
-                pb = TC(0);
-                pc = mp;
+                q[0] = mp;
+                q[1] = TC(0);
+                q[2] = mp;
             }
         }
-        const TC oa = (TC)Qp[t], ob = (TC)Qp[t + N], oc = (TC)Qp[t + 2 * N];
-        note(pa, ra, oa);
-        note(pb, rb, ob);
-        note(pc, rc, oc);
-        R[t] = (T)(pa + beta * (pa - oa));
-        R[t + N] = (T)(pb + beta * (pb - ob));
-        R[t + 2 * N] = (T)(pc + beta * (pc - oc));
-        Qp[t] = (T)pa;
-        Qp[t + N] = (T)pb;
-        Qp[t + 2 * N] = (T)pc;
+    }
+}
+template <class T, int REG>
+__device__ __forceinline__ void dual_pixel(const typename Comp<T>::type* Lx, T* __restrict__ R, T* __restrict__ Qp,
+                                           int64_t t, int64_t N, typename Comp<T>::type step,
+                                           typename Comp<T>::type beta, bool* chg = nullptr) {
+    using TC = typename Comp<T>::type;
+    constexpr int G = dual_components(REG);
+    TC r[G], q[G];
+#pragma unroll
+    for (int c = 0; c < G; ++c) r[c] = (TC)R[t + c * N];
+    dual_project<TC, REG>(Lx, r, step, q);
+#pragma unroll
+    for (int c = 0; c < G; ++c) {
+        const TC o = (TC)Qp[t + c * N];
+        if (chg && !(q[c] == r[c] && q[c] == o)) *chg = true;
+        R[t + c * N] = (T)(q[c] + beta * (q[c] - o));
+        Qp[t + c * N] = (T)q[c];
     }
 }
 
