@@ -275,10 +275,9 @@ __device__ __forceinline__ void last_cta_coef_t(const TA* partT, int le, int ldm
 template <class TU, class TZ, class TA, int NQ, int PV>
 __device__ __forceinline__ void uc_body(const TU* __restrict__ U, const TZ* __restrict__ z, int64_t N, int ell,
                                         const TA* c, TA* red, TA sign, TZ* __restrict__ out,
-                                        const TZ* __restrict__ base, TA scale, int keep) {
+                                        const TZ* __restrict__ base, TA scale, int keep, const L2Pol& pol) {
     constexpr int V = Vec16<TU>::n;
     constexpr int P = 32 * V * PV;
-    const L2Pol pol = make_l2_pol();
     const int b = blockIdx.y;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     TA acc[PV][V];
@@ -348,13 +347,14 @@ __global__ void __launch_bounds__(256) uc_vec_kernel(const TU* __restrict__ U, c
             }
         return;
     }
+    const L2Pol pol = make_l2_pol();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TA* c = reinterpret_cast<TA*>(smem_raw);
     TA* red = c + ((ell + 3) & ~3);            // [8][P]
     const int b = blockIdx.y;
     for (int j = threadIdx.x; j < ell; j += blockDim.x) c[j] = coef[(size_t)b * ell + j];
     __syncthreads();
-    uc_body<TU, TZ, TA, NQ, PV>(U, z, N, ell, c, red, sign, out, base, scale, keep);
+    uc_body<TU, TZ, TA, NQ, PV>(U, z, N, ell, c, red, sign, out, base, scale, keep, pol);
 }
 
 // The same with c = M w (or d .* w) formed by every CTA from the partial sums of
@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(256) uc_coef_kernel(const TU* __restrict__ U, 
     reduce_partials_t<TA>(part + (size_t)blockIdx.y * nb * ell, nb, ell, w);
     coef_rows<TA, TM>(w, ell, ldm, inverse, M, d, 0, ell, c);
     __syncthreads();
-    uc_body<TU, TZ, TA, 4, 1>(U, z, N, ell, c, red, sign, out, base, scale, keep);
+    uc_body<TU, TZ, TA, 4, 1>(U, z, N, ell, c, red, sign, out, base, scale, keep, make_l2_pol());
 }
 
 }  // namespace
