@@ -17,7 +17,7 @@ namespace {
 
 constexpr int PB = 32;
 
-// 1 / d by two Newton steps from the hardware's approximation (20 bits): one
+// 1 / d by two Newton-Raphson steps from the hardware's approximation (20 bits): one
 // rounding off at most, a third of the latency of a correctly rounded division
 __device__ __forceinline__ double recip(double d) {
     double r;
