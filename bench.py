@@ -59,7 +59,7 @@ SECONDARY = ("deblur512_tv_f32", "superres4x_hs_huber_f32")
 # (the native arm's first-hit count on a GB300, bench.py's k_precond): the
 # reference arm, which cannot run the solve, extrapolates its sample to this
 # count so that both arms time the same work
-NATIVE_K = {"ct512_parallel_tv_f32": 1774, "deblur512_tv_f32": 192, "superres4x_hs_huber_f32": 40}
+NATIVE_K = {"ct512_parallel_tv_f32": 1775, "deblur512_tv_f32": 192, "superres4x_hs_huber_f32": 40}
 
 
 def dist_env():

@@ -11,13 +11,13 @@
 //
 // Kernel design (sm_103a): batches of bf16 images stream down strips of
 // columns in persistent CTAs (sepstream_kernel below); everything else takes
-// one CTA per output tile, its side chosen by size (pick_tile).  The input tile and
-// its periodic halo are staged once in shared memory; the row pass writes an
-// intermediate tile to shared memory; the column pass writes the output.  Each
-// thread computes 8 consecutive outputs of a row (or column) with a sliding
-// register window, so every shared-memory load feeds 8 FMAs and the tile kernel is
-// bound by the FP32 FMA pipe rather than by shared-memory bandwidth.  Row
-// pitches are odd so that lanes reading consecutive rows hit distinct banks.
+// one CTA per output tile, its side chosen by size (pick_tile).  The input
+// tile and its periodic halo are staged once in shared memory; the row pass
+// writes an intermediate tile to shared memory; the column pass writes the
+// output.  Each thread computes 8 consecutive outputs of a row (or column)
+// with a sliding register window, so every shared-memory load feeds 8 FMAs and
+// the tile kernel is bound by the FP32 FMA pipe rather than by shared-memory
+// bandwidth.  Row pitches are odd so that lanes reading consecutive rows hit distinct banks.
 #include "internal.cuh"
 
 #include <cmath>

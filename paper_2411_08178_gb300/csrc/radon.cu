@@ -249,14 +249,15 @@ struct alignas(16) TileAng {           // one base angle as a tile sees it
 // barrier per round); every pixel then takes its two bins of every angle.
 // out: images of type TO (PLANES false: one angle range, no mirror lanes), or
 // one plane per (group, angle range, lane), already mirrored back, for
-// lane_sum.  RAW: s is the sinogram itself (type TC), its lanes gathered while
-// staging, which saves adjoint calls on one to three images the pass that
-// interleaves it (257 x 301 pixels, 363 angles, forward and
-// adjoint called from Python: 4 launches for 5, 153 to 150 us, host-bound).  Bound by shared memory: two 16-byte loads per pixel and angle, 8
-// wavefronts per warp and four lanes, 91% of the L1 data pipe busy on a batch
-// of 400 images of 512 x 512, 720 x 736: 18.1 ms (one image: 64 us).  The
-// per-line scatter into shared memory before it, 3.7 times the instructions
-// and read-modify-writes of a private row, took 117 ms (411 us).
+// lane_sum.  RAW: s is the sinogram itself (type TC), its lanes gathered
+// while staging, which saves adjoint calls on one to three images the pass
+// that interleaves it (257 x 301 pixels, 363 angles, forward and adjoint
+// called from Python: 4 launches for 5, 153 to 150 us, host-bound).  Bound
+// by shared memory: two 16-byte loads per pixel and angle, 8 wavefronts per
+// warp and four lanes, 91% of the L1 data pipe busy on a batch of 400 images
+// of 512 x 512, 720 x 736: 18.1 ms (one image: 64 us).  The per-line scatter
+// into shared memory before it, 3.7 times the instructions and read-modify-
+// writes of a private row, took 117 ms (411 us).
 template <class TC, class TO, int IB, bool PLANES, bool RAW>
 __global__ void __launch_bounds__(256) radon_adj_kernel(const void* __restrict__ s, TO* __restrict__ out, int n1,
                                                         int n2, int n_angles, int n_bins, int batch, int AK, int per,

@@ -119,7 +119,9 @@ __device__ __forceinline__ void dual_pixel(const typename Comp<T>::type* Lx, T* 
                                            typename Comp<T>::type beta, bool* chg = nullptr) {
     using TC = typename Comp<T>::type;
     constexpr int G = dual_components(REG);
-    TC r[G], o[G], q[G];   // every load before any store (HS_1, 128 x 128: 2.0 us a step, 2.6 with Q loaded per component)
+    // every load before any store (HS_1, 128 x 128: 2.0 us a step, 2.6 with Q
+    // loaded per component between the stores)
+    TC r[G], o[G], q[G];
 #pragma unroll
     for (int c = 0; c < G; ++c) r[c] = (TC)R[t + c * N], o[c] = (TC)Qp[t + c * N];
     dual_project<TC, REG>(Lx, r, step, q);
