@@ -12,7 +12,7 @@
 //
 // The per-ray a, b come from a host table in float64; float32 operators keep
 // them as integers with 40 fraction bits and step positions in fixed point (32
-// fraction bits in the forward, 27 at the usual bin spacings in the adjoint),
+// fraction bits in the forward, 27 in the adjoint),
 // so that no weight carries the rounding of a float position.
 //
 // Lanes (ray_lanes.cuh).  Over a full circle, -theta sees the image turned
@@ -192,9 +192,9 @@ constexpr int AWIN = 192;     // staged bins per segment and piece
 constexpr int AJ = 4;         // segments per round
 constexpr int AKMAX = 64;     // most candidate bins per pixel of the unrolled path
 
-// Offsets of the rays from a pixel, in fixed point that wraps: only offsets
-// within a few pixels matter (the host picks the fraction bits so that every
-// candidate's fits)
+// Offsets of the rays from a pixel, in fixed point that wraps at 2^(bits -
+// frac) pixels (32 in float32, 512 in float64): an offset more than a pixel
+// below that keeps a weight of zero (the jobs below see to it)
 template <class TC> struct FanOff;
 template <> struct FanOff<float> {
     using S = int;
@@ -220,18 +220,21 @@ template <> struct FanOff<double> {
 
 // a segment as a tile sees it: bins near a point (r, p) (line, position from
 // the tile's corner) are around m = mc + g (a0 + ar r + ap p) / (d0 + dr r +
-// dp p) from the first staged bin on
+// dp p) from the first staged bin on, to within eps bins
 struct FanJob {
     int kb, lo, hi, rs, sgn;
-    int mlo, wn, K;           // first staged bin, bins staged, candidates per pixel
-    float mc, a0, ar, ap, d0, dr, dp;
+    int mlo, wn, K;           // first staged bin, bins staged, candidates per pixel (0: pixel by pixel)
+    float mc, a0, ar, ap, d0, dr, dp, eps;
 };
 
 // Adjoint: one CTA per (32 x 32 tile, group of lanes, range of segments).  The
 // segments that reach the tile are listed, then taken AJ at a time: their bins
 // near the tile are staged in shared memory (offset and slope of the ray in
 // tile coordinates, the lanes scaled by the ray's weight), and every pixel
-// walks the K bins that can pass within one pixel of it along the line.  A
+// walks the K bins that can pass within one pixel of it along the line.  K is
+// what the pixel with most of them needs; where so many bins reach past the
+// wrapping offsets from another pixel (depths several times apart within the
+// tile), every pixel finds its own first and last bin.  A
 // quarter warp holds 4 x 2 pixels, so that its bins stay close for both kinds
 // of ray.  Windows larger than AWIN bins are taken in pieces.
 // Bound by instruction issue (about 60%) and the uneven tiles: one 512 x 512
@@ -259,7 +262,8 @@ __global__ void __launch_bounds__(256) fan_adj_kernel(const Lanes<TC, IB>* __res
     const int g = blockIdx.z / ns, z = blockIdx.z - g * ns;
     const int per = (n_seg + ns - 1) / ns, q_beg = z * per, q_end = min(n_seg, q_beg + per);
     const L* sg = s + (size_t)g * set.n_base * n_bins;
-    const float eps = 0.01f;          // float rounding of m, in bins
+    // offsets below this many pixels do not wrap onto the hat function
+    const float reach = ldexpf(1.0f, 8 * (int)sizeof(typename FO::U) - frac) - 2.0f;
     TC acc[4][IB];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
@@ -283,7 +287,8 @@ __global__ void __launch_bounds__(256) fan_adj_kernel(const Lanes<TC, IB>* __res
             const float tr = sgm.rs ? ti : tj, tp = sgm.rs ? tj : ti, sf = (float)sgm.sgn;
             const float cb = 0.5f * (float)(n_bins - 1);
             // lower edge m(p - sgn) and upper edge m(p + sgn) over the tile's corners
-            float lo_min = 3e38f, lo_max = -3e38f, hi_max = -3e38f, d_min = 3e38f, num = 0.0f;
+            float lo_min = 3e38f, lo_max = -3e38f, hi_max = -3e38f;
+            float d_min = 3e38f, d_max = 0.0f, a_max = 0.0f, num = 0.0f, num_min = 3e38f;
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const float r = c & 1 ? tr : 0.0f, p = c & 2 ? tp : 0.0f;
@@ -291,17 +296,27 @@ __global__ void __launch_bounds__(256) fan_adj_kernel(const Lanes<TC, IB>* __res
                 const float ml = cb + G * (a - sf * J.ap) / (d - sf * J.dp);
                 const float mh = cb + G * (a + sf * J.ap) / (d + sf * J.dp);
                 lo_min = fminf(lo_min, ml), lo_max = fmaxf(lo_max, ml), hi_max = fmaxf(hi_max, mh);
-                d_min = fminf(d_min, d - fabsf(J.dp));
-                num = fmaxf(num, fabsf(J.ap * d - a * J.dp));
+                d_min = fminf(d_min, d - fabsf(J.dp)), d_max = fmaxf(d_max, d + fabsf(J.dp));
+                a_max = fmaxf(a_max, fabsf(a));
+                const float nm = fabsf(J.ap * d - a * J.dp);
+                num = fmaxf(num, nm), num_min = fminf(num_min, nm);
             }
+            // float rounding of m, in bins: eight units of 2^-24 of the terms of a and
+            // d (512 x 512, two bins a pixel: 0.001), and a floor well above the usual
+            const float terms = fabsf(px) + fabsf(py) + 64.0f;
+            J.eps = 0.01f + 0x1p-21f * (G / d_min) * (terms + (a_max / d_min) * (R + terms));
             hit = lo_min < (float)J.hi + 1.0f && hi_max > (float)J.lo - 1.0f;
             // at most span + 1 integers lie between the edges; span from the
             // largest dm/dp on the tile
             const float span = 2.0f * G * num / (d_min * d_min);
-            J.K = (int)fminf(span + 4.0f * eps, 1.0e6f) + 1;
-            J.mlo = (int)floorf(lo_min - eps) - 1;
-            J.wn = (int)ceilf(fmaxf(lo_max + eps + (float)J.K, hi_max)) + 2 - J.mlo;
+            J.K = (int)fminf(span + 4.0f * J.eps, 1.0e6f) + 1;
+            J.mlo = (int)floorf(lo_min - J.eps) - 1;
+            J.wn = (int)ceilf(fmaxf(lo_max + J.eps + (float)J.K, hi_max)) + 2 - J.mlo;
             J.mc = cb - (float)J.mlo;
+            // K bins on from m(p - sgn) a ray is K d^2 / (G num - K d |dp|) pixels away
+            // at most (p as a function of m, inverted)
+            const float Kd = (float)J.K * d_max;
+            if (J.wn > AWIN || J.K > AKMAX || !(Kd * d_max < reach * (G * num_min - Kd * fabsf(J.dp)))) J.K = 0;
         }
         const unsigned bal = __ballot_sync(0xffffffffu, hit);
         __syncthreads();                // the previous list is consumed
@@ -348,8 +363,8 @@ __global__ void __launch_bounds__(256) fan_adj_kernel(const Lanes<TC, IB>* __res
                     if (wn <= 0) continue;
                     const L* wa = win + a * AWIN;
                     const typename FO::E* oa = off + a * AWIN;
-                    const float sf = (float)J.sgn, mc = J.mc - (float)(pc * AWIN);
-                    if (J.wn <= AWIN && J.K <= AKMAX) {
+                    const float sf = (float)J.sgn, mc = J.mc - (float)(pc * AWIN), eps = J.eps;
+                    if (J.K) {
                         int idx[4];
                         typename FO::U r[4], p[4];
 #pragma unroll
@@ -373,7 +388,7 @@ __global__ void __launch_bounds__(256) fan_adj_kernel(const Lanes<TC, IB>* __res
                             }
                         }
                     } else {
-                        // bins far denser than pixels, or a tile next to the source
+                        // bins far denser or sparser than pixels, or a tile next to the source
                         for (int u = 0; u < 4; ++u) {
                             const int di = ty + 8 * u, rr = J.rs ? di : tx, pp = J.rs ? tx : di;
                             if (i0 + di >= n1 || j0 + tx >= n2) continue;
@@ -381,8 +396,8 @@ __global__ void __launch_bounds__(256) fan_adj_kernel(const Lanes<TC, IB>* __res
                             const float a = J.a0 + J.ar * fr + J.ap * fp, d = J.d0 + J.dr * fr + J.dp * fp;
                             const float ml = mc + G * __fdividef(a - sf * J.ap, d - sf * J.dp);
                             const float mh = mc + G * __fdividef(a + sf * J.ap, d + sf * J.dp);
-                            const int c0 = (int)fmaxf(ceilf(ml - eps) - 1.0f, 0.0f);
-                            const int c1 = (int)fminf(floorf(mh + eps) + 1.0f, (float)(wn - 1));
+                            const int c0 = (int)fmaxf(ceilf(ml - eps), 0.0f);
+                            const int c1 = (int)fminf(floorf(mh + eps), (float)(wn - 1));
                             for (int c = c0; c <= c1; ++c) {
                                 const typename FO::E e = oa[c];
                                 const L v = wa[c];
@@ -622,13 +637,14 @@ int fanbeam_setup(nys_op* op) {
             }
         }
     }
-    // fraction bits of the adjoint's offsets: twice the largest spacing of
-    // neighbouring rays along a line, and some, has to fit beside them
+    // fraction bits of the adjoint's offsets.  A pixel's own bins end within eps
+    // (0.01 and some) bins of its neighbours on the line, so a twentieth of the
+    // largest spacing of rays along a line has to fit beside the fraction
     const double half_diag = 0.5 * std::sqrt((double)n1 * n1 + (double)n2 * n2);
     const double spacing = std::sqrt(2.0) * du * (R + half_diag + 2.0) / D;
-    int rb = 4;
-    while (rb < 24 && std::ldexp(1.0, rb) < 4.0 + 2.5 * spacing) ++rb;
-    op->fan.frac = (f64 ? 63 : 31) - rb;
+    int ib = f64 ? 9 : 5;
+    while (ib < 25 && std::ldexp(1.0, ib) < 8.0 + 0.05 * spacing) ++ib;
+    op->fan.frac = (f64 ? 64 : 32) - ib;
     // ---- upload
     size_t total = w_off + RA * es;
     std::vector<std::pair<const void*, std::pair<size_t, size_t>>> puts{{tab.get(), {0, total}}};
