@@ -105,13 +105,15 @@ __global__ void __launch_bounds__(256) fan_fwd_kernel(const Lanes<TC, IB>* __res
 #pragma unroll
         for (int c = 0; c < CB; ++c) {
             if (rs[c] != kind) continue;
-            const float a = ray_a(ray[c]) - 1.0f, b = ray_b(ray[c]);
+            // 0 <= 1 + a + b l < na + 1 with 1 + a anywhere from a0 - 1 to a0 + 1: the
+            // rounding of a moves a slow crossing by as much over |b| lines
+            const float a0 = floorf(ray_a(ray[c])), b = ray_b(ray[c]);
             int lo = 0, hi = nl;
-            if (fabsf(b) > 1e-6f) {
-                const float e1 = (-1.0f - a) / b, e2 = ((float)na - a) / b;
+            if (fabsf(b) * (float)nl > 1.0f) {
+                const float e1 = (-1.0f - a0) / b, e2 = ((float)(na + 2) - a0) / b;
                 lo = (int)fmaxf(0.0f, floorf(fminf(e1, e2)) - 2.0f);
                 hi = (int)fminf((float)nl, ceilf(fmaxf(e1, e2)) + 3.0f);
-            } else if (a < -3.0f || a > (float)(na + 2)) {
+            } else if (a0 < -5.0f || a0 > (float)(na + 5)) {
                 hi = 0;
             }
             if (lo < hi) {
