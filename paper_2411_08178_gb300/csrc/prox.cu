@@ -728,16 +728,19 @@ int ssn_run(nys_ctx* ctx, const nys_precond* pc, double tau, int64_t N, const T*
     const int ell = pv->ell_eff;
     cudaStream_t sm = ctx->stream;
     int st;
+    const int nb = (int)((N + SCH - 1) / SCH);
+    // sized for every column, whichever are active: a later set-up may activate
+    // more, and a solver's captured steps cannot allocate
+    const size_t L = pc->ell;
+    const size_t need = sizeof(SsnState) + 64 + 4 * L * 8 + (size_t)nb * L * 16 + (size_t)nb * L * L * 4;
+    char* w = (char*)scratch(ctx, SLOT_SSN, need, &st);
+    if (st) return st;
     if (ell == 0) {      // P = I
         if ((st = soft_run<T>(ctx, tau, N, s, out))) return st;
         if (gamma_io) NYS_CK(ctx, cudaMemsetAsync(gamma_io, 0, pc->ell * sizeof(double), sm));
         if (info) info->iterations = 0, info->converged = 1, info->residual = 0.0;
         return NYS_OK;
     }
-    const int nb = (int)((N + SCH - 1) / SCH);
-    const size_t need = sizeof(SsnState) + 64 + (size_t)4 * ell * 8 + (size_t)nb * ell * 16 + (size_t)nb * ell * ell * 4;
-    char* w = (char*)scratch(ctx, SLOT_SSN, need, &st);
-    if (st) return st;
     SsnState* state = (SsnState*)w;
     double* gamma = (double*)(w + ((sizeof(SsnState) + 63) & ~size_t(63)));
     double* gtrial = gamma + ell;
