@@ -27,6 +27,7 @@ struct nys_batch {
     cudaGraphExec_t g_fwd = nullptr, g_bwd = nullptr;
     bool fwd_done = false;
     uint64_t gen = 0;   // sum of the item contexts' scratch generations at capture
+    std::vector<int> cols;   // active columns of the items' preconditioners then
 };
 
 namespace nys {
@@ -81,9 +82,18 @@ uint64_t scratch_gens(const nys_batch* B) {
     return g;
 }
 
-// capture both graphs again if a scratch region they use was reallocated
+// and the launches that fit the active columns of the preconditioners, which
+// the caller may have factored or set up again
+std::vector<int> columns(const nys_batch* B) {
+    std::vector<int> c;
+    for (const nys_unroll* u : B->items) c.push_back(unroll_columns(u));
+    return c;
+}
+
+// capture both graphs again if a scratch region they use was reallocated or the
+// active columns of an item changed
 int refresh(nys_batch* B) {
-    if (B->gen == scratch_gens(B)) return NYS_OK;
+    if (B->gen == scratch_gens(B) && B->cols == columns(B)) return NYS_OK;
     for (nys_ctx* c : B->item_ctx) NYS_CK(B->ctx, cudaStreamSynchronize(c->stream));
     NYS_CK(B->ctx, cudaStreamSynchronize(B->ctx->stream));
     cudaGraphExec_t f = nullptr, b = nullptr;
@@ -98,6 +108,7 @@ int refresh(nys_batch* B) {
     B->g_fwd = f;
     B->g_bwd = b;
     B->gen = scratch_gens(B);
+    B->cols = columns(B);
     return NYS_OK;
 }
 
@@ -149,6 +160,7 @@ int nys_batch_create(nys_ctx* ctx, int n, nys_unroll* const* items, nys_ctx* con
     if (!st) st = capture(B, false, &B->g_fwd);
     if (!st) st = capture(B, true, &B->g_bwd);
     B->gen = scratch_gens(B);
+    B->cols = columns(B);
     if (st) {
         nys_batch_destroy(B);
         return st;

@@ -384,8 +384,10 @@ int precond_run(nys_ctx* ctx, const nys_precond* pc, int inverse, int dtype, con
 // launched, where the vectorised apply does not run
 int precond_axpy_run(nys_ctx* ctx, const nys_precond* pc, int dtype, const void* z, const void* base, double scale,
                      void* out);
-// the contexts an unrolled-solve handle launches on (unroll.cu)
+// the contexts an unrolled-solve handle launches on, and the active columns of
+// its preconditioner (unroll.cu)
 void unroll_contexts(const nys_unroll* U, nys_ctx** ctx, nys_ctx** op_ctx);
+int unroll_columns(const nys_unroll* U);
 // dual APG prox with the fused two-launch (TV) or three-launch (HS) step
 // (prox_fused.cu); returns
 // NYS_EINVAL without launching anything when the layout does not allow it

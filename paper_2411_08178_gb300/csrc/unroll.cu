@@ -583,6 +583,9 @@ void unroll_contexts(const nys_unroll* U, nys_ctx** ctx, nys_ctx** op_ctx) {
     *ctx = U->ctx;
     *op_ctx = U->op->ctx;
 }
+int unroll_columns(const nys_unroll* U) {
+    return U->pc && U->pc->priv ? ((const nys_precond_priv*)U->pc->priv)->ell_eff : 0;
+}
 }  // namespace nys
 
 using namespace nys;
@@ -644,6 +647,16 @@ int nys_unroll_create(nys_ctx* ctx, nys_op* op, const nys_precond* pc, const nys
     if (e != cudaSuccess) {
         nys_unroll_destroy(U);
         return cuda_fail(ctx, e, "unrolled-solve buffers");
+    }
+    if (pc) {
+        // the partial sums of P^{-1} for every column, whichever are active: passes
+        // captured after a later set-up cannot allocate (chunks of 512 .. 2048 pixels)
+        int st;
+        scratch(ctx, SLOT_PRECOND, ((N + 511) / 512 * pc->ell + 2 * (size_t)pc->ell) * es, &st);
+        if (st) {
+            nys_unroll_destroy(U);
+            return st;
+        }
     }
     *out = U;
     return NYS_OK;

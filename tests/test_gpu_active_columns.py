@@ -1,6 +1,6 @@
-"""A preconditioner whose active columns change under a solver that has captured
-its launches: later steps use the new columns, whichever way the count went,
-with the scratch that was reserved at creation."""
+"""A preconditioner whose active columns change under a solver or a batch that
+has captured its launches: later steps use the new columns, whichever way the
+count went, with the scratch that was reserved at creation."""
 import numpy as np
 import pytest
 
@@ -47,3 +47,37 @@ def test_solver(reg, n, ell, dt, grow):
     ref = make(ref_ctx, factor(torch, api, ref_ctx, n * n, ell, dtype, not grow))
     ref.step(3)
     assert torch.equal(sol.x(), ref.x())
+
+
+@pytest.mark.parametrize("grow", [True, False])
+@pytest.mark.parametrize("n,ell", [(64, 12), (64, 100), (33, 20)])
+def test_batch(n, ell, grow):
+    torch, api = require_gpu()
+    main = api.Context(0, torch.cuda.Stream(priority=-1))
+    stream = torch.cuda.Stream()
+    ctx = api.Context(0, stream)
+    with torch.cuda.stream(stream):
+        op = api.Operator(ctx, "blur", n, n, dtype=torch.float32, kernel=gaussian_kernel(7, 1.5))
+        pc = factor(torch, api, ctx, n * n, ell, torch.bfloat16, grow)
+        un = api.Unroll(ctx, op, 1e-2, 0.4, 3, n_inner=3, ckpt_every=2, pc=pc)
+        y = torch.from_numpy(phantom(n, 5, 1, "mixed")).float().cuda()
+        x, xbar = torch.zeros_like(y), torch.ones_like(y)
+    torch.cuda.synchronize()
+    B = api.Batch(main, [un], [y], [x], [xbar])
+    B.forward()
+    B.backward()
+    torch.cuda.synchronize()
+    first = x.clone()
+    with torch.cuda.stream(stream):
+        pc.setup(0.0, not grow)
+    torch.cuda.synchronize()
+    B.forward()
+    B.backward()
+    torch.cuda.synchronize()
+    got, g = x.clone(), B.grads[0].clone()
+    with torch.cuda.stream(stream):
+        ref = un.forward(y)
+        dl, dh = un.backward(xbar)
+    torch.cuda.synchronize()
+    assert torch.equal(got, ref) and not torch.equal(got, first)
+    assert float(g[0]) == float(dl) and torch.equal(g[1:], dh.reshape(-1))
