@@ -11,9 +11,9 @@
 // zero outside.  Pixel (i, j) sits at (j - c2, i - c1).
 //
 // The per-ray a, b come from a host table in float64; float32 operators keep
-// them as integers with 40 fraction bits and step positions in fixed point (32
-// fraction bits in the forward, 27 in the adjoint),
-// so that no weight carries the rounding of a float position.
+// them as integers with 40 fraction bits and step positions in fixed point (40
+// fraction bits in the forward, 27 in the adjoint), so that no weight carries
+// the rounding of a float position.
 //
 // Lanes (ray_lanes.cuh).  Over a full circle, -theta sees the image turned
 // upside down with its bins reversed exactly as theta sees the image, and with
@@ -141,10 +141,10 @@ __global__ void __launch_bounds__(256) fan_fwd_kernel(const Lanes<TC, IB>* __res
 #pragma unroll
             for (int c = 0; c < CB; ++c) {
                 const unsigned e = rs[c] == kind ? min((unsigned)pos[c].index(), last) : last;
-                const TC F = pos[c].one_plus_f();
+                TC w0, w1;
+                pos[c].weights(w0, w1);
                 pos[c].step(dt[c]);
                 const Lanes<TC, IB> a = line[e], b = line[e + 1];
-                const TC w1 = F - TC(1), w0 = TC(2) - F;
 #pragma unroll
                 for (int q = 0; q < IB; ++q) acc[c][q] = fma(w1, b.v[q], fma(w0, a.v[q], acc[c][q]));
             }

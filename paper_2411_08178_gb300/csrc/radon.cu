@@ -15,9 +15,9 @@
 // (u - position = (m - m*) / den): at most the two bins either side of m*,
 // since |den| <= 1.  The forward walks rays, the adjoint gathers per pixel;
 // both take their positions from float64 and step them in fixed point, so the
-// weights of the two agree to about 1e-7 (float32 operators: 32 fraction bits
-// in the forward, 26 in the adjoint, relative to a 32 x 32 tile) or to the
-// last float64 bits, and the two are transposes of each other to rounding.
+// weights of the two agree to a few roundings of their type (float32 operators:
+// 40 fraction bits in the forward, 26 in the adjoint, relative to a 32 x 32
+// tile), and the two are transposes of each other to that.
 //
 // Lanes (ray_lanes.cuh).  Over 180 degrees, angle n_angles - k sees the
 // left-right mirrored image exactly as angle k sees the image, and for a
@@ -135,9 +135,9 @@ __global__ void __launch_bounds__(256) radon_fwd_kernel(const Lanes<TL, IB>* __r
 #pragma unroll
         for (int c = 0; c < CB; ++c) {
             const unsigned e = min((unsigned)pos[c].index(), last);
-            const TC F = pos[c].one_plus_f();
+            TC w0, w1;
+            pos[c].weights(w0, w1);
             pos[c].step(dt);
-            const TC w1 = F - TC(1), w0 = TC(2) - F;
             if constexpr (BF) {
                 // pairs of images in the halves of packed FMAs
                 const uint4 ua = *reinterpret_cast<const uint4*>(line + e);

@@ -140,18 +140,23 @@ __global__ void __launch_bounds__(256) lane_sum_kernel(const TC* __restrict__ pl
 }
 
 // position of a ray on its line, stepped line by line: an integer part and a
-// binary fraction of 32 (float) or 64 (double) bits; one_plus_f() is the
-// fraction as 1 + f in [1, 2)
+// binary fraction f of 40 (float) or 64 (double) bits, so that the rounding of
+// the step stays below the weights' over thousands of lines; weights() are those
+// of the positions index() and index() + 1, 1 - f and f.  In float f is its top
+// 32 bits converted (rounded to 2^-25; 23 bits put into a float between 1 and 2
+// leave 2^-24 with rounding and twice that without)
 template <class TC>
 struct RayPos;
 template <>
 struct RayPos<float> {
     long long p;
-    __device__ __forceinline__ void set40(long long u) { p = (u + 128) >> 8; }   // from 40 fraction bits
+    __device__ __forceinline__ void set40(long long u) { p = u; }
     __device__ __forceinline__ void step(const RayPos& d) { p += d.p; }
-    __device__ __forceinline__ int index() const { return (int)(p >> 32); }
-    __device__ __forceinline__ float one_plus_f() const {
-        return __uint_as_float(((unsigned)p >> 9) + 0x3f800000u);
+    __device__ __forceinline__ int index() const { return (int)(p >> 40); }
+    __device__ __forceinline__ void weights(float& w0, float& w1) const {
+        const float F = __uint2float_rn((unsigned)(p >> 8));
+        w1 = F * 0x1p-32f;
+        w0 = fmaf(F, -0x1p-32f, 1.0f);
     }
 };
 template <>
@@ -169,8 +174,10 @@ struct RayPos<double> {
         f = s;
     }
     __device__ __forceinline__ int index() const { return i; }
-    __device__ __forceinline__ double one_plus_f() const {
-        return __longlong_as_double((long long)((f >> 12) | 0x3ff0000000000000ull));
+    __device__ __forceinline__ void weights(double& w0, double& w1) const {
+        const double F = __longlong_as_double((long long)((f >> 12) | 0x3ff0000000000000ull));   // 1 + f
+        w1 = F - 1.0;
+        w0 = 2.0 - F;
     }
 };
 
