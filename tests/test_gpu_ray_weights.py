@@ -1,7 +1,8 @@
 """The weights of the float32 ray transforms, read off one by one: a ray meets a
 pixel in one sample, so the transform of an image with a single pixel returns
 single weights.  They are held to a few roundings of 2^-24 for images of any
-size (positions are carried in more bits than the weights)."""
+size (positions are carried in more bits than the weights); the adjoint of a
+sinogram with one bin an angle likewise."""
 import math
 
 import numpy as np
@@ -64,4 +65,25 @@ def test_forward(geom, n, batch):
     err = np.concatenate(err)
     # the fraction and one less it (U / 2 each), 1 / |den| <= 1.415 and the product (U each)
     assert np.max(np.abs(err)) <= 1.415 * 3.0 * U
+    assert np.sqrt(np.mean(err ** 2)) <= U
+
+
+@pytest.mark.parametrize("n", [512, 2048, 4096])
+@pytest.mark.parametrize("batch", [1, 4])
+def test_parallel_adjoint(n, batch):
+    torch, api = require_gpu()
+    op, weights = parallel(torch, api, n)
+    A, B = op.meas_shape
+    err = []
+    for i, j in pixels(n, 9):
+        ref = weights(i, j)
+        for k in range(A):
+            for m in np.nonzero(ref[k])[0]:
+                s = torch.zeros((batch, A, B), device="cuda")
+                s[:, k, m] = 1.0
+                err.append(float(api.op_adjoint(op, s)[batch - 1, i, j]) - ref[k, m])
+    err = np.array(err)
+    # 1 / |den| and its difference to 1 / den^2 <= 2, 1 / den^2 itself, the fraction
+    # (U / 2, times 1 / den^2) and the sum: U each
+    assert np.max(np.abs(err)) <= 4.0 * U
     assert np.sqrt(np.mean(err ** 2)) <= U
