@@ -202,7 +202,8 @@ template <> struct FanOff<float> {
     using S = int;
     using U = unsigned;
     struct alignas(8) E { U u, b; };
-    // position of ray r at line l0 relative to p0, and its slope
+    // position of ray r at line l0 relative to p0, and its slope (l0 the tile's
+    // middle line: the slope's rounding counts at most half a tile's times)
     static __device__ __forceinline__ E make(const longlong2& r, int l0, int p0, int frac) {
         const int sh = 40 - frac;
         const long long h = 1ll << (sh - 1);
@@ -353,7 +354,7 @@ __global__ void __launch_bounds__(256) fan_adj_kernel(const Lanes<TC, IB>* __res
                         const TC wt = tab.w[ray] * inv_one;
 #pragma unroll
                         for (int q = 0; q < IB; ++q) v.v[q] *= wt;
-                        e = FO::make(tab.ray[ray], J.rs ? i0 : j0, J.rs ? j0 : i0, frac);
+                        e = FO::make(tab.ray[ray], (J.rs ? i0 : j0) + ATS / 2, J.rs ? j0 : i0, frac);
                     }
                     win[t] = v;
                     off[t] = e;
@@ -375,7 +376,7 @@ __global__ void __launch_bounds__(256) fan_adj_kernel(const Lanes<TC, IB>* __res
                             const float fr = (float)rr, fp = (float)pp - sf;
                             const float m = mc + G * __fdividef(J.a0 + J.ar * fr + J.ap * fp, J.d0 + J.dr * fr + J.dp * fp);
                             idx[u] = max(0, min((int)ceilf(m - eps), wn - J.K));   // in range for pixels of the image
-                            r[u] = (typename FO::U)rr;
+                            r[u] = (typename FO::U)(typename FO::S)(rr - ATS / 2);
                             p[u] = (typename FO::U)pp << frac;
                         }
                         for (int c = 0; c < J.K; ++c) {
@@ -403,7 +404,7 @@ __global__ void __launch_bounds__(256) fan_adj_kernel(const Lanes<TC, IB>* __res
                             for (int c = c0; c <= c1; ++c) {
                                 const typename FO::E e = oa[c];
                                 const L v = wa[c];
-                                const TC dd = (TC)(typename FO::S)(e.u + (typename FO::U)rr * e.b -
+                                const TC dd = (TC)(typename FO::S)(e.u + (typename FO::U)(typename FO::S)(rr - ATS / 2) * e.b -
                                                                   ((typename FO::U)pp << frac));
                                 const TC w = fmax(one - fabs(dd), TC(0));
 #pragma unroll

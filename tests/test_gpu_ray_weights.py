@@ -87,3 +87,25 @@ def test_parallel_adjoint(n, batch):
     # (U / 2, times 1 / den^2) and the sum: U each
     assert np.max(np.abs(err)) <= 4.0 * U
     assert np.sqrt(np.mean(err ** 2)) <= U
+
+
+@pytest.mark.parametrize("n,B,du", [(512, 1024, 1.0), (2048, 4096, 1.0), (512, 200, 12.0), (512, 60, 40.0)])
+def test_fan_adjoint(n, B, du):
+    """Bins of half a pixel to 40 pixels: the offsets keep their fraction bits."""
+    torch, api = require_gpu()
+    A, R, D, span = 9, 1.3 * n, 2.2 * n, 5.0
+    op = api.Operator(api.Context(0), "fanbeam", n, n, dtype=torch.float32, n_angles=A, n_bins=B, angle_span=span,
+                      src_dist=R, det_dist=D, det_spacing=du)
+    row, a, b, w = O.fanbeam_tables(n, n, A, B, R, D, du, span)
+    err = []
+    for i, j in pixels(n, 20):
+        ref = w * np.maximum(0.0, 1.0 - np.abs(a + b * np.where(row, i, j) - np.where(row, j, i)))
+        for k in range(A):
+            for m in np.nonzero(ref[k])[0]:
+                s = torch.zeros((1, A, B), device="cuda")
+                s[:, k, m] = 1.0
+                err.append((float(api.op_adjoint(op, s)[0, i, j]) - ref[k, m]) / w[k, m])
+    # the offset (2^-28, and as much 16 times from the slope), its conversion and one
+    # less it (U / 2 each), the ray's weight and the product (U each)
+    assert np.max(np.abs(err)) <= 4.1 * U
+    assert np.sqrt(np.mean(np.square(err))) <= U
