@@ -385,9 +385,13 @@ __global__ void __launch_bounds__(256) fan_adj_kernel(const Lanes<TC, IB>* __res
                                 const typename FO::E e = oa[idx[u] + c];
                                 const L v = wa[idx[u] + c];
                                 const TC d = (TC)(typename FO::S)(e.u + r[u] * e.b - p[u]);
-                                const TC w = fmax(one - fabs(d), TC(0));
+                                // (left out, not multiplied by zero: an infinity or a NaN reaches the
+                                // pixels of its ray only)
+                                const TC w = one - fabs(d);
+                                if (w > TC(0)) {
 #pragma unroll
-                                for (int q = 0; q < IB; ++q) acc[u][q] = fma(w, v.v[q], acc[u][q]);
+                                    for (int q = 0; q < IB; ++q) acc[u][q] = fma(w, v.v[q], acc[u][q]);
+                                }
                             }
                         }
                     } else {
@@ -406,9 +410,11 @@ __global__ void __launch_bounds__(256) fan_adj_kernel(const Lanes<TC, IB>* __res
                                 const L v = wa[c];
                                 const TC dd = (TC)(typename FO::S)(e.u + (typename FO::U)(typename FO::S)(rr - ATS / 2) * e.b -
                                                                   ((typename FO::U)pp << frac));
-                                const TC w = fmax(one - fabs(dd), TC(0));
+                                const TC w = one - fabs(dd);
+                                if (w > TC(0)) {
 #pragma unroll
-                                for (int q = 0; q < IB; ++q) acc[u][q] = fma(w, v.v[q], acc[u][q]);
+                                    for (int q = 0; q < IB; ++q) acc[u][q] = fma(w, v.v[q], acc[u][q]);
+                                }
                             }
                         }
                     }

@@ -259,7 +259,7 @@ template <class TC>
 struct alignas(16) TileAng {           // one base angle as a tile sees it
     typename TilePos<TC>::type pos0;           // position of the tile's pixel (16, 16)
     typename TilePos<TC>::step dj, di;         // steps along j and i
-    TC wb, w0, w1;                     // lower bin's weight max(0, w0 - wb F), upper's max(0, w1 + wb F), F = frac()
+    TC wb, w0, w1;                     // lower bin's weight w0 - wb F, upper's w1 + wb F where positive, F = frac()
     int mlo;                           // first staged bin
 };
 
@@ -375,9 +375,17 @@ __global__ void __launch_bounds__(256) radon_adj_kernel(const void* __restrict__
                 const L* e = w + TP::index(pu);
                 const TC F = TP::frac(pu);
                 const L s0 = e[0], s1 = e[1];
-                const TC a0 = fmax(fma(-t.wb, F, t.w0), TC(0)), a1 = fmax(fma(t.wb, F, t.w1), TC(0));
+                // a bin without weight is left out, not multiplied by zero: an infinity or
+                // a NaN reaches the pixels of its ray only
+                const TC a0 = fma(-t.wb, F, t.w0), a1 = fma(t.wb, F, t.w1);
+                if (a0 > TC(0)) {
 #pragma unroll
-                for (int q = 0; q < IB; ++q) acc[u][q] = fma(a1, s1.v[q], fma(a0, s0.v[q], acc[u][q]));
+                    for (int q = 0; q < IB; ++q) acc[u][q] = fma(a0, s0.v[q], acc[u][q]);
+                }
+                if (a1 > TC(0)) {
+#pragma unroll
+                    for (int q = 0; q < IB; ++q) acc[u][q] = fma(a1, s1.v[q], acc[u][q]);
+                }
             }
         }
     }
