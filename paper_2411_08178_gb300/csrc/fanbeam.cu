@@ -677,7 +677,7 @@ int fanbeam_setup(nys_op* op) {
         NYS_CK(op->ctx, cudaMemcpy((char*)op->rtab + q.second.first, q.first, q.second.second, cudaMemcpyHostToDevice));
     // interleaved sinogram lanes, image lines and the adjoint's planes, for
     // every part that a chunk of images can be cut into
-    op->chunk = 32;
+    op->chunk = ray_chunk(op);
     size_t lanes = 0, lines = 0, planes = 0;
     for (int left = 1; left <= op->chunk; ++left) {
         const Part p = next_part(op, left);

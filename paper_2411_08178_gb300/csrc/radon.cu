@@ -583,7 +583,7 @@ int radon_typed(nys_op* op, int which, const void* x, void* y, int batch) {
 
 int radon_setup(nys_op* op) {
     if (int st = build_tables(op)) return st;
-    op->chunk = 32;
+    op->chunk = ray_chunk(op);
     const size_t es = op->dtype == NYS_F64 ? 8 : 4;
     // interleaved sinogram lanes, image lines and the adjoint's planes, for
     // every part that a chunk of images can be cut into

@@ -184,15 +184,32 @@ struct RayPos<double> {
 // Lanes and mirror lanes for a part of a batch: fours of images while there
 // are four; a rest of one to three takes four mirror lanes an image where the
 // angles allow it (a quarter of the angles each), else two (two images to a
-// launch group), else plain lanes.
+// launch group), else plain lanes.  Images for which scratch is short
+// (ray_chunk) go one group at a time, the largest by themselves.
 struct Part {
     int nb, IB, V;
 };
+constexpr int RAY_CHUNK = 32;
 inline Part next_part(const nys_op* op, int left) {
+    if (op->chunk == 1) return {1, 1, 1};
     if (left >= 4) return {left / 4 * 4, 4, 1};
-    if (op->lane_sets & 4) return {left, 4, 4};
-    if (op->lane_sets & 2) return left == 1 ? Part{1, 2, 2} : Part{left, 4, 2};
+    const bool one = op->chunk < RAY_CHUNK;
+    if (op->lane_sets & 4) return {one ? 1 : left, 4, 4};
+    if (op->lane_sets & 2) return left == 1 ? Part{1, 2, 2} : Part{one ? 2 : left, 4, 2};
     return {left, left == 3 ? 4 : left, 1};
+}
+
+// images to a chunk: 32 while their lines (two copies each) stay within 2 GB
+// (2048 x 2048 in float64), then as many as do, at least a group (eight in
+// float32: the bf16 forward); one, in plain lanes, where a group with its planes
+// would take more than 64 GB.  32 throughout took 8.6 GB for an operator of 4096
+// x 4096 pixels in float64, whatever it was used on; this 2.7 GB.  (A^T A of 32
+// float32 images of 4096 x 4096, 90 angles: within 4 GB 37.1, 2 GB 38.3, 1 GB
+// 41.6 ms.)
+inline int ray_chunk(const nys_op* op) {
+    const int64_t image = op->N * (op->dtype == NYS_F64 ? 8 : 4), unit = op->dtype == NYS_F64 ? 4 : 8;
+    if ((2 * unit + 4) * image > (int64_t(64) << 30)) return 1;
+    return (int)std::max(unit, std::min<int64_t>(RAY_CHUNK, (int64_t(2) << 30) / (2 * image) / unit * unit));
 }
 
 template <class TI, class TC, int IB>
