@@ -66,12 +66,14 @@ __device__ __forceinline__ float ray_b(const double2& r) { return (float)r.y; }
 // has a slope of its own, and a warp whose rays are of both kinds walks its
 // lines once for each.  One 512 x 512 image, 720 angles x 1024 bins: 98 us, the
 // L1 data pipe 66% busy (one thread per ray, reading columns of the row-major
-// image for column-step rays, took 885 us).
+// image for column-step rays, took 885 us).  Registers for three CTAs to an SM
+// (one image 99 against 104 us with fewer), and a line at a time where a lane
+// has two bins (32 images: 2.57 ms, two lines 3.14).
 template <class TC, class TO, int IB, int CB, int SEG, bool LANES>
-__global__ void __launch_bounds__(256) fan_fwd_kernel(const Lanes<TC, IB>* __restrict__ rows,
-                                                      const Lanes<TC, IB>* __restrict__ cols, void* __restrict__ yv,
-                                                      int n1, int n2, int n_angles, int n_bins, int batch,
-                                                      FanTab<TC> tab, LaneSet set) {
+__global__ void __launch_bounds__(256, 3) fan_fwd_kernel(const Lanes<TC, IB>* __restrict__ rows,
+                                                         const Lanes<TC, IB>* __restrict__ cols, void* __restrict__ yv,
+                                                         int n1, int n2, int n_angles, int n_bins, int batch,
+                                                         FanTab<TC> tab, LaneSet set) {
     pdl_enter();
     constexpr int FANG = 8 / SEG;
     __shared__ Lanes<TC, IB> part[SEG > 1 ? SEG - 1 : 1][SEG > 1 ? FANG : 1][SEG > 1 ? CB : 1][32];
@@ -136,7 +138,7 @@ __global__ void __launch_bounds__(256) fan_fwd_kernel(const Lanes<TC, IB>* __res
         }
         const unsigned last = na + 1;   // a position outside [-1, na) reads the two zeros after the line
         const Lanes<TC, IB>* line = (kind ? rows : cols) + ((size_t)g * nl + l_beg) * pitch;
-#pragma unroll 2
+#pragma unroll (CB == 2 ? 1 : 2)
         for (int l = l_beg; l < l_end; ++l, line += pitch) {
 #pragma unroll
             for (int c = 0; c < CB; ++c) {
