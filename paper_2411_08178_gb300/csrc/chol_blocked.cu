@@ -5,7 +5,7 @@
 // GB300's float64 pipe issues about two FMAs per clock per SM, so the work is
 // spread over all SMs in panels of 32 columns, two launches a panel: every
 // CTA of chol_panel factors the 32 x 32 diagonal block for itself (one warp, a
-// row per lane, no square root or division on the dependent chain) and solves
+// row per lane, no square root on the dependent chain) and solves
 // for 32 rows of the panel; chol_update subtracts the panel's product from the
 // trailing matrix, one CTA per 16 x 16 tile.  A 16-CTA cluster kernel
 // (chol_cluster.cu) factored n = 400 in 1.00 ms, most of it latency (31 us a
@@ -16,15 +16,6 @@ namespace nys {
 namespace {
 
 constexpr int PB = 32;
-
-// 1 / d by two Newton-Raphson steps from the hardware's approximation (20 bits): one
-// rounding off at most, a third of the latency of a correctly rounded division
-__device__ __forceinline__ double recip(double d) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    r = fma(r, fma(-d, r, 1.0), r);
-    return fma(r, fma(-d, r, 1.0), r);
-}
 
 // A = sym(Omega^T Y) + v Omega^T Omega (lower triangle) from the Gram G2 of
 // [Omega | Y] (ld 2n), v = eps sqrt(trace Omega^T Omega); info = {0, v, 0}
@@ -74,7 +65,7 @@ __global__ void __launch_bounds__(128) chol_panel_kernel(const double* __restric
     auto publish = [&](int k, double d, double p) {
         cd[k & 1][lane] = d;
         cp[k & 1][lane] = p;
-        const double pk = __shfl_sync(0xffffffffu, d, k), ik = recip(pk);
+        const double pk = __shfl_sync(0xffffffffu, d, k), ik = 1.0 / pk;
         if (lane == 0) piv[k] = pk, inv[k] = ik;
     };
     if (w == 0) publish(0, ad[0], ap[0]);
