@@ -40,12 +40,16 @@ namespace {
 // per-angle geometry, float64; the ray positions of float32 operators also as
 // integers with 40 fraction bits (GB300 issues a float64 operation every 16
 // cycles per warp and SM: evaluated in float64, the positions of a few bins per
-// warp took as long as a quarter of a warp's lines)
+// warp took as long as a quarter of a warp's lines).  Bins and lines count from
+// the middle of the detector and of the image, so that positions near the image
+// stay exact whatever the detector's width; the integers may wrap on the way.
 struct RGeo {
-    double u0, inv, t;    // 1 + u(m, l) = u0 + m inv - l t
-    long long u0q, invq, tq;
+    double c, inv, t;     // 1 + u(m, l) = c + (m - cb) inv - (l - c_line) t
+    long long u0q, invq, tq;         // = u0q + m invq - l tq
     double cs, sn;
-    int rs, pad;          // row-step angle
+    int rs;               // row-step angle
+    int b2, l2;           // n_bins - 1, lines - 1
+    int m_lo, m_hi;       // rays outside miss the image (further out their integers wrap into it)
 };
 
 // the angles of a launch: geo[ang[kb V]] is the geometry of base angle kb
@@ -57,7 +61,7 @@ __device__ __forceinline__ void ray_at(RayPos<float>& p, const RGeo& g, int m, i
     p.set40(g.u0q + m * g.invq - l * g.tq);
 }
 __device__ __forceinline__ void ray_at(RayPos<double>& p, const RGeo& g, int m, int l) {
-    p.set(fma((double)m, g.inv, fma(-(double)l, g.t, g.u0)));
+    p.set(fma(m - 0.5 * g.b2, g.inv, fma(-(l - 0.5 * g.l2), g.t, g.c)));
 }
 __device__ __forceinline__ void ray_step(RayPos<float>& p, const RGeo& g) { p.set40(-g.tq); }
 __device__ __forceinline__ void ray_step(RayPos<double>& p, const RGeo& g) { p.set(-g.t); }
@@ -120,6 +124,7 @@ __global__ void __launch_bounds__(256) radon_fwd_kernel(const Lanes<TL, IB>* __r
     } else if (qmax < -3.0f || qmin > (float)(na + 2)) {
         l_end = 0;
     }
+    if (m0 > geo.m_hi || m0 + 32 * CB <= geo.m_lo) l_end = 0;
     if (SEG > 1) {
         const int per = (max(0, l_end - l_beg) + SEG - 1) / SEG;
         l_beg += seg * per;
@@ -305,7 +310,8 @@ __global__ void __launch_bounds__(256) radon_adj_kernel(const void* __restrict__
         const int k = k_beg + r * AK + threadIdx.x;
         if (threadIdx.x >= AK || k >= k_end) return;
         const RGeo geo = set.geo[set.ang[k * set.V]];
-        const double m00 = fma(geo.cs, j0 - 0.5 * (n2 - 1), fma(geo.sn, i0 - 0.5 * (n1 - 1), 0.5 * (n_bins - 1)));
+        // from the detector's middle bin (n_bins - 1) / 2 on
+        const double m00 = fma(geo.cs, j0 - 0.5 * (n2 - 1), fma(geo.sn, i0 - 0.5 * (n1 - 1), 0.5 * ((n_bins - 1) & 1)));
         const double lo = floor(m00 + fmin(0.0, (ATS - 1) * geo.cs) + fmin(0.0, (ATS - 1) * geo.sn) - 1e-3);
         const double a = fabs(geo.inv), b = a * a;
         TileAng<TC> t;
@@ -316,7 +322,7 @@ __global__ void __launch_bounds__(256) radon_adj_kernel(const void* __restrict__
         t.wb = (TC)b * TP::SCALE;
         t.w0 = (TC)(a + TP::BIAS * b);
         t.w1 = (TC)(a - (1 + TP::BIAS) * b);
-        t.mlo = (int)lo;
+        t.mlo = (int)lo + (n_bins - 1) / 2;
         tab[(r % 3) * AK + threadIdx.x] = t;
         if (RAW) {
 #pragma unroll
@@ -368,7 +374,9 @@ __global__ void __launch_bounds__(256) radon_adj_kernel(const void* __restrict__
         const L* w = win + (r & 1) * AK * AWIN;
         const TileAng<TC>* ta = tab + (r % 3) * AK;
         const int na = min(AK, k_end - k_beg - r * AK);
-#pragma unroll (PLANES ? 4 : 2)      // one image 159.5 with four, 161.4 us with two; batches the other way round
+        // measured, by the compiler's order of the loads: one image 159.5 with four, 161.4
+        // us with two; 400 images 33.4 ms with one, 34.9 with two or four
+#pragma unroll (PLANES ? 4 : 1)
         for (int a = 0; a < na; ++a, w += AWIN) {
             const TileAng<TC> t = ta[a];
             const P p = TP::at(t.pos0, tx - ATS / 2, t.dj, ty - ATS / 2, t.di);
@@ -418,17 +426,23 @@ __global__ void __launch_bounds__(256) radon_adj_kernel(const void* __restrict__
 
 int build_tables(nys_op* op) {
     const int A = op->n_angles, B = op->n_bins, n1 = op->n1, n2 = op->n2;
-    const double c1 = (n1 - 1) / 2.0, c2 = (n2 - 1) / 2.0, cb = (B - 1) / 2.0;
+    const double c1 = (n1 - 1) / 2.0, c2 = (n2 - 1) / 2.0;
     std::vector<RGeo> geo(A);
     for (int k = 0; k < A; ++k) {
         const double th = k * (op->span / A);
         const double cs = std::cos(th), sn = std::sin(th);
         const bool rs = std::fabs(cs) + 1e-9 >= std::fabs(sn);
-        const double c_line = rs ? c1 : c2, c_pos = rs ? c2 : c1;
+        const double c = 1.0 + (rs ? c2 : c1);
         const double den = rs ? cs : sn, oth = rs ? sn : cs;
-        const double u0 = c_pos + 1.0 - cb / den + c_line * (oth / den), inv = 1.0 / den, t = oth / den;
-        auto fix = [](double v) { return (long long)std::llrint(std::ldexp(v, 40)); };
-        geo[k] = RGeo{u0, inv, t, fix(u0), fix(inv), fix(t), cs, sn, rs ? 1 : 0, 0};
+        const double inv = 1.0 / den, t = oth / den;
+        const int b2 = B - 1, l2 = (rs ? n1 : n2) - 1;
+        // halves of the steps, so that the middles are whole numbers of them
+        auto fix = [](double v) { return (unsigned long long)std::llrint(std::ldexp(v, 40)); };
+        const unsigned long long ih = fix(0.5 * inv), th2 = fix(0.5 * t);
+        const long long far = (int64_t)n1 + n2 + 64;
+        geo[k] = RGeo{c, inv, t, (long long)(fix(c) - b2 * ih + l2 * th2), (long long)(2 * ih), (long long)(2 * th2),
+                      cs, sn, rs ? 1 : 0, b2, l2, (int)std::max<long long>(0, (b2 - far) / 2),
+                      (int)std::min<long long>(b2, (b2 + far) / 2)};
     }
     // the angle sets: every angle by itself, and over exactly 180 degrees the
     // mirror pairs and (square image, even number of angles) the fours

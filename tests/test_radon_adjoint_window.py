@@ -13,9 +13,10 @@ ATS, AWIN = 32, 48
 
 
 def positions(n1, n2, B, th, i0, j0, bits):
-    """(index, fraction) of the tile's pixels and the first staged bin."""
+    """(index, fraction) of the tile's pixels and the first staged bin (from the middle
+    bin (B - 1) // 2 on)."""
     cs, sn = math.cos(th), math.sin(th)
-    m00 = cs * (j0 - 0.5 * (n2 - 1)) + (sn * (i0 - 0.5 * (n1 - 1)) + 0.5 * (B - 1))
+    m00 = cs * (j0 - 0.5 * (n2 - 1)) + (sn * (i0 - 0.5 * (n1 - 1)) + 0.5 * ((B - 1) & 1))
     lo = math.floor(m00 + min(0.0, (ATS - 1) * cs) + min(0.0, (ATS - 1) * sn) - 1e-3)
     tx, ty = np.meshgrid(np.arange(ATS), np.arange(ATS))
     if bits == 32:
@@ -43,7 +44,7 @@ def test_positions(n1, n2, B, bits):
             assert idx.min() >= 0 and idx.max() + 1 < AWIN
             ld = np.longdouble
             cs, sn = np.cos(ld(th)), np.sin(ld(th))
-            m = cs * (j0 + tx - ld(n2 - 1) / 2) + sn * (i0 + ty - ld(n1 - 1) / 2) + ld(B - 1) / 2
+            m = cs * (j0 + tx - ld(n2 - 1) / 2) + sn * (i0 + ty - ld(n1 - 1) / 2) + ld((B - 1) & 1) / 2
             err = np.abs((lo + idx) + ld(1) * frac - m)
             # float64 rounding of the first pixel's position, then the fixed point
-            assert np.max(err) <= (2.0 ** -26 if bits == 32 else 2.0 ** -48) + 4 * np.finfo(float).eps * (n1 + n2 + B)
+            assert np.max(err) <= (2.0 ** -26 if bits == 32 else 2.0 ** -48) + 4 * np.finfo(float).eps * (n1 + n2)

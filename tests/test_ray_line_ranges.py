@@ -44,7 +44,8 @@ def test_fan_rays(nl, na, dt):
     assert live.any() and not (live & ((l < lo[:, None]) | (l >= hi[:, None]))).any()
 
 
-@pytest.mark.parametrize("n1,n2,B", [(512, 512, 736), (2048, 96, 2100), (96, 2048, 2100), (64, 64, 300)])
+@pytest.mark.parametrize("n1,n2,B", [(512, 512, 736), (2048, 96, 2100), (96, 2048, 2100), (64, 64, 300), (40, 33, 20_000), (32, 40, 12_600_001),
+                                     (32, 32, 60_000_000)])
 @pytest.mark.parametrize("CB", [1, 2])
 def test_parallel_warps(n1, n2, B, CB):
     """radon_fwd: a warp's 32 CB bins share a range, from the whole positions of
@@ -54,12 +55,24 @@ def test_parallel_warps(n1, n2, B, CB):
         cs, sn = math.cos(th), math.sin(th)
         rs = abs(cs) + 1e-9 >= abs(sn)
         (nl, na), (den, oth) = ((n1, n2), (cs, sn)) if rs else ((n2, n1), (sn, cs))
-        u0 = (na - 1) / 2 + 1.0 - (B - 1) / 2 / den + (nl - 1) / 2 * (oth / den)
-        u0q, invq, tq = (int(np.rint(v * 2.0 ** 40)) for v in (u0, 1.0 / den, oth / den))
+        cq, invh, th2 = (int(np.rint(v * 2.0 ** 40)) for v in ((na + 1) / 2, 0.5 / den, 0.5 * oth / den))
+        u0q, invq, tq = cq - (B - 1) * invh + (nl - 1) * th2, 2 * invh, 2 * th2
+        far = n1 + n2 + 64
+        m_lo, m_hi = max(0, (B - 1 - far) // 2), min(B - 1, (B - 1 + far) // 2)
+
+        def at(m, l):      # 64-bit integers that wrap
+            p = (u0q + np.asarray(m, object) * invq - np.asarray(l, object) * tq + 2 ** 63) % 2 ** 64 - 2 ** 63
+            return p.astype(np.int64) if isinstance(p, np.ndarray) else p
+
         tl = f(tq) * f(2.0 ** -40)
-        for m0 in range(0, B, 32 * CB):
+        step = 32 * CB
+        starts = range(0, B, step)
+        if B > 100_000:       # around the image, where positions wrap round onto it, and the ends
+            mids = [B // 2 + s * int(2 ** 24 * abs(den)) for s in (-1, 0, 1)] + [0, B - 1]
+            starts = sorted({(m // step + d) * step for m in mids for d in range(-4, 5) if 0 <= (m // step + d) * step < B})
+        for m0 in starts:
             m1 = min(m0 + 32 * CB - 1, B - 1)
-            qa, qb = (f(((u0q + m * invq) >> 40) - 1) for m in (m0, m1))
+            qa, qb = (f((at(m, 0) >> 40) - 1) for m in (m0, m1))
             qmin, qmax = min(qa, qb), max(qa, qb) + f(1)
             lo, hi = 0, nl
             if abs(tl) > f(1e-6):
@@ -68,7 +81,13 @@ def test_parallel_warps(n1, n2, B, CB):
                 hi = int(min(f(nl), np.ceil(max(e1, e2)) + f(3)))
             elif qmax < -3 or qmin > na + 2:
                 hi = 0
+            if m0 > m_hi or m0 + 32 * CB <= m_lo:
+                hi = 0
             m, l = np.arange(m0, m1 + 1)[:, None], np.arange(nl)[None, :]
-            u = (u0q + m * invq - l * tq) * 2.0 ** -40 - 1.0
-            live = (u > -1.0) & (u < na)
-            assert not (live & ((l < lo) | (l >= hi))).any()
+            u = ((u0q + m * np.int64(invq) - l * np.int64(tq)) if abs(u0q) < 2 ** 62 else at(m, l)) * 2.0 ** -40 - 1.0
+            exact = (na - 1) / 2 + (m - (B - 1) / 2) / den - (l - (nl - 1) / 2) * (oth / den)
+            seen = (exact > -1.0) & (exact < na)
+            assert np.all(np.abs(u - exact)[seen] <= 2.0 ** -40 * far)
+            walked = (l >= lo) & (l < hi)
+            assert not (walked & (u > -1.0 + 1e-6) & (u < na - 1e-6) & ~seen).any()
+            assert not (seen & ((l < lo) | (l >= hi))).any()
