@@ -9,7 +9,7 @@
 // for 32 rows of the panel; chol_update subtracts the panel's product from the
 // trailing matrix, one CTA per 16 x 16 tile.  A 16-CTA cluster kernel
 // (chol_cluster.cu) factored n = 400 in 1.00 ms, most of it latency (31 us a
-// 13-column panel); this takes 0.44 ms.  n = 200: 0.38 ms there, 0.22 ms here.
+// 13-column panel); this takes 0.47 ms.  n = 200: 0.38 ms there, 0.25 ms here.
 #include "internal.cuh"
 
 namespace nys {
@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(256) core_form_kernel(const double* __restrict
 // of one warp takes its scheduler 64 cycles, so the columns are dealt to four
 // warps (column j to warp j mod 4); the owner of the next column updates it
 // first and publishes it with the reciprocal of its pivot while the others
-// finish the step (49 us a panel with one warp, 28 us so).  The lower triangle
+// finish the step (51 us a panel with one warp, 30 us so).  The lower triangle
 // of A is read, L's panel written (block 0: the diagonal block, zeros above it).
 // info[slot] = 1 on a pivot that is not positive and finite.
 __global__ void __launch_bounds__(128) chol_panel_kernel(const double* __restrict__ A, double* __restrict__ L, int n,

@@ -25,7 +25,6 @@
 
 namespace nys {
 
-enum : int { TRI_A = 1, TRI_B = 2, GEMM_SYM = 4 };   // small.cu
 int launch_small_gemm(nys_ctx* ctx, const double* A, int ta, const double* B, int tb, int m, int n, int k,
                       const double* colscale, double* C, int flags);
 int sym_eig(nys_ctx* ctx, const double* G, int ell, bool use_f32, const double* info, void* work, double* Vout,
@@ -588,8 +587,8 @@ static int factor_small(nys_ctx* ctx, const double* G2, int ell, double eps, boo
     int st;
     // layout after the skipped doubles (float64 unless noted): C, H, Ci, T1,
     // Gm, Vs, scale, info (16) + sweeps (16), then the eigen work area: 2 n^2
-    // values of the Jacobi type and ell doubles
-    const size_t need = (skip + 6 * l2 + (size_t)ell + 32) * 8 + 2 * (size_t)n * n * 8 + 8 * (size_t)n + 256;
+    // doubles
+    const size_t need = (skip + 6 * l2 + (size_t)ell + 32) * 8 + 2 * (size_t)n * n * 8 + 256;
     double* w = (double*)scratch(ctx, SLOT_FACTOR, need, &st);
     if (st) return st;
     double* C = w + skip;
@@ -601,7 +600,7 @@ static int factor_small(nys_ctx* ctx, const double* G2, int ell, double eps, boo
     double* scale = Vs + l2;
     double* info = scale + ell;           // 16 doubles
     int* sweeps = (int*)(info + 16);
-    void* ework = (void*)(info + 32);     // eigen work (2 n^2 T + n doubles)
+    void* ework = (void*)(info + 32);     // eigen work (2 n^2 doubles)
     cudaStream_t s = ctx->stream;
     NYS_CK(ctx, cudaMemsetAsync(info, 0, 16 * sizeof(double), s));
     // shifted Cholesky (steps 4-5); the retries with larger shifts, which return
@@ -647,7 +646,7 @@ int nys_factor(nys_ctx* ctx, const void* Omega, const void* Y, int in_dt, int64_
     const int n = (ell + 1) & ~1;
     int st;
     // G2 at the start of the factor workspace, sized for factor_small too
-    const size_t need = ((size_t)L2 * L2 + 6 * l2 + (size_t)ell + 32) * 8 + 2 * (size_t)n * n * 8 + 8 * (size_t)n + 256;
+    const size_t need = ((size_t)L2 * L2 + 6 * l2 + (size_t)ell + 32) * 8 + 2 * (size_t)n * n * 8 + 256;
     double* G2 = (double*)scratch(ctx, SLOT_FACTOR, need, &st);
     if (st) return st;
     cudaStream_t s = ctx->stream;

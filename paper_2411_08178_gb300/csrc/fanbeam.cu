@@ -64,7 +64,7 @@ __device__ __forceinline__ float ray_b(const double2& r) { return (float)r.y; }
 // Forward: a warp takes 32 CB consecutive bins of one base entry and steps
 // along a SEG-th of the lines its rays cross, as radon_fwd_kernel; every ray
 // has a slope of its own, and a warp whose rays are of both kinds walks its
-// lines once for each.  One 512 x 512 image, 720 angles x 1024 bins: 98 us, the
+// lines once for each.  One 512 x 512 image, 720 angles x 1024 bins: 99 us, the
 // L1 data pipe 66% busy (one thread per ray, reading columns of the row-major
 // image for column-step rays, took 885 us).  Registers for three CTAs to an SM
 // (one image 99 against 104 us with fewer), and a line at a time where a lane
@@ -243,7 +243,7 @@ struct FanJob {
 // quarter warp holds 4 x 2 pixels, so that its bins stay close for both kinds
 // of ray.  Windows larger than AWIN bins are taken in pieces.
 // Bound by instruction issue (about 60%) and the uneven tiles: one 512 x 512
-// image, 720 angles x 1024 bins, 0.22 ms, where one thread per pixel testing
+// image, 720 angles x 1024 bins, 0.21 ms, where one thread per pixel testing
 // every candidate ray against float tables in L2 took 4.56 ms.
 template <class TC, class TO, int IB, bool PLANES>
 __global__ void __launch_bounds__(256) fan_adj_kernel(const Lanes<TC, IB>* __restrict__ s, TO* __restrict__ out,
@@ -474,7 +474,7 @@ LaneSet fan_set(const nys_op* op, int V) {
 // segment ranges of the adjoint: about 20 CTAs to an SM, at least 16 segments
 // each (tiles near the sources take several times the bins of those opposite,
 // so few long CTAs leave SMs idle: one 512 x 512 image of 720 angles x 1024
-// bins, A^T A with 2 ranges 401 us, 7 ranges 357 us, 11 ranges 343 us)
+// bins, A^T A with 2 ranges 392 us, 7 ranges 342 us, 11 ranges 329 us, 16 341 us)
 int adj_ranges(const nys_op* op, int groups, int n_seg) {
     const int64_t ctas = (int64_t)((op->n1 + ATS - 1) / ATS) * ((op->n2 + ATS - 1) / ATS) * groups;
     const int64_t want = (int64_t)op->ctx->sm_count * 20;

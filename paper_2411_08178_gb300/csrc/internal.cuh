@@ -122,7 +122,7 @@ struct nys_op {
     int n_angles = 0, n_bins = 0;
     double span = 0.0;
     void* rtab = nullptr;             // per-angle tables, see radon.cu
-    void* lines = nullptr;            // rays: `chunk` images as interleaved lines (along rows and along columns)
+    void* lines = nullptr;            // rays: a chunk's images as interleaved lines (along rows and along columns)
     void* planes = nullptr;           // ray adjoints: partial images (lanes and angle ranges) of a launch
     int lane_sets = 1;                // rays: mirror lanes the angles allow (1, 2 and 4 or'ed, see ray_lanes.cuh)
     double src_dist = 0.0, det_dist = 0.0, det_spacing = 1.0;   // fan beam
@@ -298,6 +298,10 @@ int fanbeam_run(nys_op* op, int which, const void* x, void* y, int batch, int in
 int haar_run(nys_op* op, const void* in, void* out, int batch, int inverse, int in_dtype, int out_dtype);
 // generic: which = 0 A, 1 A^T, 2 A^T A ; dtypes may differ from op dtype (bf16 io)
 int op_run(nys_op* op, int which, const void* x, void* y, int batch, int in_dtype, int out_dtype);
+
+// flags of the ell x ell products (small.cu): op(A), op(B) triangular, the result
+// symmetric
+enum : int { TRI_A = 1, TRI_B = 2, GEMM_SYM = 4 };
 
 // dense helpers (dense.cu)
 // C[p x q] (double) = A^T B, A: N x p, B: N x q (column j at offset j*N)

@@ -77,10 +77,10 @@ __device__ __forceinline__ void ray_step(RayPos<double>& p, const RGeo& g) { p.s
 // adjoint reads (LANES).  Bound by the L1 data pipe: 96% busy on that batch,
 // where a load's 32 positions, 1 to 1.41 pixels of 16 bytes apart, take about
 // 7 wavefronts instead of 4; before the lanes (scalar loads, four images per
-// warp) 48.4 ms, and 183 us for one image (now 94 us: 181 base angles leave
+// warp) 48.4 ms, and 183 us for one image (now 82 us: 181 base angles leave
 // half of the warp slots empty).
 // TL: type of the lines, TC or bf16 (a bf16 batch, eight images to a 16-byte
-// load: half the L1 traffic per image, 14.7 against 25.5 ms for the batch above).
+// load: half the L1 traffic per image, 14.0 against 25.5 ms for the batch above).
 template <class TL, class TC, class TO, int IB, int CB, int SEG, bool LANES>
 __global__ void __launch_bounds__(256) radon_fwd_kernel(const Lanes<TL, IB>* __restrict__ rows,
                                                         const Lanes<TL, IB>* __restrict__ cols, void* __restrict__ yv,
@@ -227,7 +227,7 @@ struct TilePos<float> {
     // 32 fraction bits, steps (at most 1) 30: 2^-31 off, up to 16 times in each
     // direction, below the conversion's 2^-25 (26 bits throughout, in 32-bit words,
     // left weights 1.4e-7 off, rms).  Four positions from one, not each from the
-    // last: the batch of 400 images below 33.9 against 35.0 ms for A^T A
+    // last: 400 images of 512 x 512, 720 x 736, 33.9 against 35.0 ms for A^T A
     using type = long long;
     using step = int;
     static constexpr float SCALE = 0x1p-32f;
@@ -284,7 +284,7 @@ struct alignas(16) TileAng {           // one base angle as a tile sees it
 // called from Python: 4 launches for 5, 153 to 150 us, host-bound).  Bound
 // by shared memory: two 16-byte loads per pixel and angle, 8 wavefronts per
 // warp and four lanes, 91% of the L1 data pipe busy on a batch of 400 images
-// of 512 x 512, 720 x 736: 18.1 ms (one image: 64 us).  The per-line scatter
+// of 512 x 512, 720 x 736: 18.6 ms (one image: 66 us).  The per-line scatter
 // into shared memory before it, 3.7 times the instructions and read-modify-
 // writes of a private row, took 117 ms (411 us).
 template <class TC, class TO, int IB, bool PLANES, bool RAW>
@@ -489,8 +489,8 @@ RSet angle_set(const nys_op* op, int V) {
 
 // angle ranges of the adjoint: as many as keep all CTAs resident at once (4 to
 // an SM) when the image has few tiles, at least 16 base angles each (one 512 x
-// 512 image, 256 tiles: 2 ranges 64 us, 3 ranges, a second wave of a quarter
-// of the SMs, 69 us)
+// 512 image, 256 tiles, A^T A: 1 range 216 us, 2 ranges 161, 3 ranges, a second
+// wave of a quarter of the SMs, 164 us)
 int adj_ranges(const nys_op* op, int groups, int n_base) {
     const int64_t ctas = (int64_t)((op->n1 + ATS - 1) / ATS) * ((op->n2 + ATS - 1) / ATS) * groups;
     const int64_t want = (int64_t)op->ctx->sm_count * 4;
@@ -530,9 +530,9 @@ int fwd_part(nys_op* op, const TI* x, void* y, int nb, int V) {
     };
     // two bins per lane share the loop and the line when that leaves 32 warps
     // to an SM; otherwise a warp takes one bin per lane and a quarter of the
-    // lines, four warps to a ray (one 512 x 512 image: 94 against 117 us
-    // without the quarters; two bins per lane for a batch: 25.5 against 28.4
-    // ms for three and 35 ms with one)
+    // lines, four warps to a ray (one 512 x 512 image, its lines prepared: 94
+    // against 141 us without the quarters; two bins per lane for a batch: 25.5
+    // against 28.4 ms for three and 35 ms with one)
     const int64_t warps = (int64_t)set.n_base * ((op->n_bins + 63) / 64) * groups;
     if (warps >= (int64_t)op->ctx->sm_count * 32)
         NYS_CK(op->ctx, go(radon_fwd_kernel<TC, TC, TO, IB, 2, 1, LANES>, 2, 1));

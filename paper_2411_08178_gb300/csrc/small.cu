@@ -79,7 +79,6 @@ __global__ void form_H_kernel(const double* __restrict__ G2, int ell, const doub
 // is lower-triangular C^{-1} (k <= i / k <= j) or, transposed, upper (k >= i);
 // GEMM_SYM computes the tiles on and below the diagonal and mirrors them.  The
 // four products at ell = 400: 534 us in full, 275 us so.
-enum : int { TRI_A = 1, TRI_B = 2, GEMM_SYM = 4 };
 __global__ void small_gemm_kernel(const double* __restrict__ A, int ta, const double* __restrict__ B, int tb, int m,
                                   int n, int k, const double* __restrict__ colscale, double* __restrict__ C,
                                   int flags) {
